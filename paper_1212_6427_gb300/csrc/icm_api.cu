@@ -892,24 +892,6 @@ icm_status ensure_hstage(icm_sim* s) {
 
 }  // namespace
 
-namespace {
-template <typename R>
-void enqueue_coupling(icm_sim* s, long long n, const double* qdev, const double* unit, double a, double b,
-                      double* outdev) {
-  const BlobParams bp = blob_params(s);
-  const FftCtx<R> fc = fft_ctx<R>(s);
-  R* work = (R*)s->work;
-  const size_t fbytes = 3 * (size_t)s->ncell * sizeof(R);
-  for (long long p = 0; p < n; ++p)
-    for (int c = 0; c < 3; ++c) {
-      cudaMemsetAsync(work, 0, fbytes, s->stream);
-      blob_spread<R>(bp, 1, qdev + 3 * (n + p), unit + 3 * c, work, s->stream);
-      spectral_solve<R>(fc, work, work, nullptr, OUT_STORE, a, b, nullptr, 0.0, s->stream);
-      blob_interp<R>(bp, 1, qdev + 3 * p, work, false, outdev + 9 * p + 3 * c, s->stream);   // column c
-    }
-}
-}  // namespace
-
 // A device copy of everything a step changes (fields, blob arrays, scalars, counters),
 // for the autotuner's trial steps.
 struct StateCopy {
@@ -1603,26 +1585,24 @@ icm_status icm_op_coupling(icm_sim* s, int64_t n, const double* qi, const double
     return fail(ICM_EINVAL, "need a >= 0, b >= 0, a + b > 0");
   if (n == 0) return ICM_OK;
   if (!finite_all(qi, 3 * n) || !finite_all(qj, 3 * n)) return fail(ICM_EINVAL, "non-finite position");
-  std::vector<double> q(6 * (size_t)n);
-  memcpy(q.data(), qi, sizeof(double) * 3 * n);
-  memcpy(q.data() + 3 * n, qj, sizeof(double) * 3 * n);
-  wrap_host(q.data(), 2 * n, s);
-  const double unit[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
-  Tmp tq(s, sizeof(double) * q.size()), tu(s, sizeof(unit)), to(s, sizeof(double) * 9 * n);
-  if (!tq.p || !tu.p || !to.p) return fail(ICM_ENOMEM, "allocation failed");
-  ICM_CK(cudaMemcpyAsync(tq.p, q.data(), sizeof(double) * q.size(), cudaMemcpyHostToDevice, s->stream));
-  ICM_CK(cudaMemcpyAsync(tu.p, unit, sizeof(unit), cudaMemcpyHostToDevice, s->stream));
-  if (s->prec == 32)
-    enqueue_coupling<float>(s, n, (const double*)tq.p, (const double*)tu.p, a, b, (double*)to.p);
-  else
-    enqueue_coupling<double>(s, n, (const double*)tq.p, (const double*)tu.p, a, b, (double*)to.p);
-  ICM_CK(cudaGetLastError());
-  std::vector<double> colmajor(9 * (size_t)n);
-  ICM_CK(cudaMemcpyAsync(colmajor.data(), to.p, sizeof(double) * 9 * n, cudaMemcpyDeviceToHost, s->stream));
-  ICM_CK(cudaStreamSynchronize(s->stream));
-  for (long long p = 0; p < n; ++p)
-    for (int r = 0; r < 3; ++r)
-      for (int c = 0; c < 3; ++c) out[9 * p + 3 * r + c] = colmajor[9 * p + 3 * c + r];
+  // chunks of pairs bound the scratch (tables of at most 41 KB per position)
+  const long long chunk = std::min<long long>(n, 512);
+  std::vector<double> q(6 * (size_t)chunk);
+  Tmp tq(s, sizeof(double) * 6 * chunk), to(s, sizeof(double) * 9 * chunk);
+  Tmp ts(s, sizeof(double) * couple_scratch_doubles(s->nx, s->ny, s->nz, (int)chunk));
+  if (!tq.p || !to.p || !ts.p) return fail(ICM_ENOMEM, "allocation failed");
+  for (long long p0 = 0; p0 < n; p0 += chunk) {
+    const long long m = std::min(chunk, (long long)n - p0);
+    memcpy(q.data(), qi + 3 * p0, sizeof(double) * 3 * m);
+    memcpy(q.data() + 3 * m, qj + 3 * p0, sizeof(double) * 3 * m);
+    wrap_host(q.data(), 2 * m, s);
+    ICM_CK(cudaMemcpyAsync(tq.p, q.data(), sizeof(double) * 6 * m, cudaMemcpyHostToDevice, s->stream));
+    couple_pairs(s->nx, s->ny, s->nz, s->h, s->kernel, (int)m, (const double*)tq.p, a, b, (double*)ts.p, (double*)to.p,
+                 s->stream);
+    ICM_CK(cudaGetLastError());
+    ICM_CK(cudaMemcpyAsync(out + 9 * p0, to.p, sizeof(double) * 9 * m, cudaMemcpyDeviceToHost, s->stream));
+    ICM_CK(cudaStreamSynchronize(s->stream));
+  }
   return ICM_OK;
 }
 
