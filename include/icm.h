@@ -143,10 +143,12 @@ typedef struct icm_plan {
                           bins (sides 32, 48, 64, 96, 128, 192, 256, 384, 512); 0: separate kernels */
   int32_t tma_z;       /* 1: persistent z pass fed by TMA (z sides <= 256 with register kernels);
                           0: one block per z tile                                                  */
-  int32_t rhs_kz;      /* right-hand-side kernel: 4..64 z planes marched by each block, or 0 for
-                          persistent blocks (as many as the SMs hold) marching even shares of
-                          all tile-planes (default 0 when each of two blocks per SM gets at least
-                          8 tile-planes of 32 x 16 cells, else 8 for Nz <= 48 and 16 otherwise)    */
+  int32_t rhs_kz;      /* right-hand-side kernel of FP32 grids above 2^20 cells: 4..64 z planes marched
+                          by each block, or 0 for persistent blocks (as many as the SMs hold)
+                          marching even shares of all tile-planes (default 0 when each of two
+                          blocks per SM gets at least 8 tile-planes of 32 x 16 cells, else 8 for
+                          Nz <= 48 and 16 otherwise).  Smaller grids and FP64 draw the stress
+                          normals in a pass of their own and do not march                          */
   int32_t fork;        /* 1: the blob-side prologue runs on a second stream beside the RHS          */
   int32_t fused_xy;    /* 1: forward x and y FFT passes fused on thread-block clusters (FP32,
                           Nx = Ny in 32, 64, 128, 256); 0 (default): two passes                    */

@@ -100,6 +100,7 @@ struct icm_sim {
   void* adv = nullptr;   // A^{n-1}, overwritten by A^n
   void* work = nullptr;  // right-hand side / spread sources / dv~ / dv
   void* spec = nullptr;  // spectrum scratch
+  void* normals = nullptr;   // stress normals of the step (grids whose right-hand side stores them), 6 ncell
   // FFT plans and symbol tables
   AxisPlan px, py, pz;
   void *dx = nullptr, *ddx = nullptr, *dy = nullptr, *ddy = nullptr, *dz = nullptr, *ddz = nullptr;
@@ -252,6 +253,11 @@ GridParams grid_params(const icm_sim* s) {
   g.rk = philox_round_keys(g.key0, g.key1);
   g.advection = s->advection ? 1 : 0;
   g.kz = s->plan.rhs_kz;
+  g.dnx = FastDiv((uint32_t)s->nx);
+  g.dny = FastDiv((uint32_t)s->ny);
+  const RhsConst<double> c = rhs_const(g);
+  g.cd = c;
+  g.cf = RhsConst<float>{(float)c.ce, (float)c.cc, (float)c.aq, (float)c.sd, (float)c.so};
   return g;
 }
 
@@ -554,7 +560,7 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
     ICM_STAGE("bins", nb * (24.0 + 2 * geob + 8.0 * kAccPerBlob), build_row_bins<R>(bp, s->nb, s->qh, bins, sb));
   if (fork) cudaEventRecord(s->ev_join, sb);
   // step 2: unperturbed fluid solve (Eq. provisional_step-1)
-  ICM_STAGE("rhs", 4 * F, explicit_rhs<R>(gp, v, adv, work, s->step_dev, s->hist_dev, st));
+  ICM_STAGE("rhs", 4 * F, explicit_rhs<R>(gp, v, adv, work, (R*)s->normals, s->step_dev, s->hist_dev, st));
   if (fork) cudaStreamWaitEvent(st, s->ev_join, 0);
   if (drift) ICM_STAGE("drift", 2 * gath + nb * 32, blob_spread_drift<R>(bp, bs, work, st));
   if (fused) {
@@ -984,7 +990,11 @@ icm_status icm_create(const int32_t grid[3], double h, double rho, double eta, d
     return fail(ICM_ECUDA, "creation of the auxiliary stream failed");
   }
   fft_prepare();
-  grid_prepare();
+  if (!grid_prepare(s->stream)) {
+    cudaGetLastError();
+    icm_destroy(s);
+    return fail(ICM_ECUDA, "upload of the noise tables failed");
+  }
   s->kx = s->nx / 2 + 1;
   s->kxp = (s->kx + 15) / 16 * 16;
   const size_t rs = s->rsize();
@@ -993,12 +1003,14 @@ icm_status icm_create(const int32_t grid[3], double h, double rho, double eta, d
   s->adv = dalloc(s, fbytes);
   s->work = dalloc(s, fbytes);
   s->spec = dalloc(s, 3 * (size_t)s->nz * s->ny * s->kxp * 2 * rs);
+  const bool stored = kT > 0.0 && rhs_stored_normals(s->prec, s->ncell);
+  if (stored) s->normals = dalloc(s, 2 * fbytes);
   s->scal = (double*)dalloc(s, sizeof(double) * SC_COUNT);
   s->step_dev = (long long*)dalloc(s, 256);
   s->hist_dev = (int*)dalloc(s, 256);
   s->err_dev = (int*)dalloc(s, 256);
   s->partial = (double*)dalloc(s, sizeof(double) * 3 * icm_sim::kPartials);
-  if (!s->v || !s->adv || !s->work || !s->spec || !s->scal || !s->step_dev || !s->hist_dev || !s->err_dev ||
+  if (!s->v || !s->adv || !s->work || !s->spec || (stored && !s->normals) || !s->scal || !s->step_dev || !s->hist_dev || !s->err_dev ||
       !s->partial) {
     icm_destroy(s);
     return fail(ICM_ENOMEM, "device allocation of %.1f MB of grid state failed", (4.0 * fbytes) / 1e6);
@@ -1043,6 +1055,7 @@ icm_status icm_create(const int32_t grid[3], double h, double rho, double eta, d
     icm_destroy(s);
     return fail(ICM_ECUDA, "initialisation failed: %s", cudaGetErrorString(e));
   }
+  grid_ready();
   *out = s;
   return ICM_OK;
 }
@@ -1625,10 +1638,10 @@ icm_status icm_op_explicit_rhs(icm_sim* s, const double* fluid_v, const double* 
   ICM_CK(cudaMemcpyAsync((char*)tc.p + 64, &hist, sizeof(int), cudaMemcpyHostToDevice, s->stream));
   const GridParams gp = grid_params(s);
   if (s->prec == 32)
-    explicit_rhs<float>(gp, (const float*)tv.p, (float*)ta.p, (float*)s->work, (const long long*)tc.p,
+    explicit_rhs<float>(gp, (const float*)tv.p, (float*)ta.p, (float*)s->work, (float*)s->normals, (const long long*)tc.p,
                         (const int*)((char*)tc.p + 64), s->stream);
   else
-    explicit_rhs<double>(gp, (const double*)tv.p, (double*)ta.p, (double*)s->work, (const long long*)tc.p,
+    explicit_rhs<double>(gp, (const double*)tv.p, (double*)ta.p, (double*)s->work, (double*)s->normals, (const long long*)tc.p,
                          (const int*)((char*)tc.p + 64), s->stream);
   ICM_CK(cudaGetLastError());
   if ((st = download_field(s, s->work, out_rhs)) != ICM_OK) return st;
@@ -1914,11 +1927,12 @@ icm_status batch_capture_stages(icm_batch* b) {
     r.v = (const R*)s->v;
     r.adv = (R*)s->adv;
     r.rhs = (R*)s->work;
+    r.normals = (R*)s->normals;
     r.step_dev = s->step_dev;
     r.hist_dev = s->hist_dev;
     long long& tot = s->kT > 0.0 ? tot_noise : tot_quiet;
     r.w0 = tot;
-    tot += rhs_tile_planes(s->nx, s->ny, s->nz);
+    tot += rhs_batch_units(s->prec, s->nx, s->ny, s->nz);
     (s->kT > 0.0 ? rhs_noise : rhs_quiet).push_back(r);
   }
   bool any_force = false;
@@ -2218,7 +2232,8 @@ int64_t icm_estimate_device_bytes(const int32_t grid[3], int32_t precision, int6
   const int64_t kxp = (grid[0] / 2 + 1 + 15) / 16 * 16;
   int64_t cap = 64;
   while (cap < nblobs) cap *= 2;
-  const int64_t fields = 3 * (3 * ncell * rs);
+  // velocities, advective fluxes, work, and the stress normals where they are stored
+  const int64_t fields = 3 * (3 * ncell * rs) + (rhs_stored_normals(precision, ncell) ? 6 * ncell * rs : 0);
   const int64_t spec = 3 * (int64_t)grid[2] * grid[1] * kxp * 2 * rs;
   const int64_t tables = 3 * (int64_t)kMaxSide * (3 * 2 * rs + 4) + 16 * 256;
   const int64_t blobs = nblobs > 0 ? 41 * cap * 8 + (int64_t)bin_blob_bytes(cap) : 0;

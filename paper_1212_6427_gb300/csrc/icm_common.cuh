@@ -28,6 +28,18 @@ template <typename C> __device__ __forceinline__ C cmul_mi(C a) { return mk(a.y,
 template <typename C> __device__ __forceinline__ C cmul_pi(C a) { return mk(-a.y, a.x); }
 template <typename C, typename R> __device__ __forceinline__ C cscale(C a, R s) { return mk(a.x * s, a.y * s); }
 
+// Division of n < 2^31 by a fixed divisor (Granlund and Montgomery, 1994: the upper half of
+// a 33-bit multiply, then a shift), for kernels that split flat indices by run-time sides.
+struct FastDiv {
+  uint32_t d = 1, mul = 1, sh = 0;
+  FastDiv() = default;
+  explicit FastDiv(uint32_t d_) : d(d_) {
+    while ((1ull << sh) < d) ++sh;
+    mul = (uint32_t)((((1ull << sh) - d) << 32) / d + 1);
+  }
+  __device__ __forceinline__ uint32_t div(uint32_t n) const { return (__umulhi(n, mul) + n) >> sh; }
+};
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10.  Round: words 0 and 2 are multiplied (full 64-bit products) by
 // two constants; the high halves are xored with words 1, 3 and the key; the key
@@ -77,19 +89,8 @@ __device__ __forceinline__ u32x4 philox4x32_10(u32x4 c, const PhiloxRoundKeys& r
 }
 
 // Box-Muller: two 32-bit words -> two unit normals (cos branch, sin branch).
-// u = (x + 1/2) 2^-32 in (0, 1).
+// u = (x + 1/2) 2^-32 in (0, 1).  The FP64 form is in icm_grid.cu (its tables live there).
 template <typename R> struct BoxMuller;
-template <> struct BoxMuller<double> {
-  __device__ __forceinline__ static void apply(uint32_t a, uint32_t b, double& z0, double& z1) {
-    const double u1 = ((double)a + 0.5) * 2.3283064365386963e-10;
-    const double u2 = ((double)b + 0.5) * 2.3283064365386963e-10;
-    const double rad = sqrt(-2.0 * log(u1));
-    double s, c;
-    sincospi(2.0 * u2, &s, &c);
-    z0 = rad * c;
-    z1 = rad * s;
-  }
-};
 template <> struct BoxMuller<float> {
   __device__ __forceinline__ static void apply(uint32_t a, uint32_t b, float& z0, float& z1) {
     // u = (x + 1/2) 2^-32 with one rounding: exact for x < 2^23 (u < 2^-9, the tail
@@ -111,22 +112,6 @@ template <> struct BoxMuller<float> {
 // The key as two words (the round keys formed in every call).
 struct PhiloxKey { uint32_t k0, k1; };
 __device__ __forceinline__ u32x4 philox4x32_10(u32x4 c, PhiloxKey k) { return philox4x32_10(c, k.k0, k.k1); }
-
-// The 6 stress normals of one cell and step: (xx, yy, zz, xy, xz, yz).  Counters
-// (cell, step, call, 0), key (seed_lo, seed_hi): call 0 of the cell gives xx, yy, zz,
-// xy; call 1 serves two z planes: at the cell of plane 2m its words 0-1 give xz, yz of
-// that cell, words 2-3 those of the cell above it (plane 2m + 1).  `odd`: the cell's
-// plane is odd (its call 1 is the one at cell - plane).  KEYS: PhiloxKey or
-// PhiloxRoundKeys.
-template <typename R, typename KEYS>
-__device__ __forceinline__ void cell_normals(uint32_t cell, uint32_t plane, bool odd, uint32_t step, const KEYS& key,
-                                             R z[6]) {
-  const u32x4 a = philox4x32_10(u32x4{cell, step, 0u, 0u}, key);
-  const u32x4 b = philox4x32_10(u32x4{odd ? cell - plane : cell, step, 1u, 0u}, key);
-  BoxMuller<R>::apply(a.x, a.y, z[0], z[1]);
-  BoxMuller<R>::apply(a.z, a.w, z[2], z[3]);
-  BoxMuller<R>::apply(odd ? b.z : b.x, odd ? b.w : b.y, z[4], z[5]);
-}
 
 // ---------------------------------------------------------------------------
 // Peskin kernel functions of r in grid units.

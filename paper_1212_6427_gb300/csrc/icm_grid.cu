@@ -7,6 +7,8 @@
 //     (Eq. Adams_Bashforth).  A^n overwrites A^{n-1} in place.
 //   * FP64 compensated sums of face fields (momentum bookkeeping, Sec. II).
 #include <algorithm>
+#include <atomic>
+#include <cmath>
 
 #include "icm_internal.h"
 
@@ -21,6 +23,81 @@ constexpr int NHALO = 2 * HX + 2 * TY;   // ring of halo cells around the TX x T
 __device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 // Periodic index for any i (a tile can be several times wider than a short side).
 __device__ __forceinline__ int wrapm(int i, int n) { return ((i % n) + n) % n; }
+
+// ---------------------------------------------------------------------------
+// FP64 Box-Muller.  FP64 operations are the scarce resource here (64 times slower than
+// FP32), and log, sqrt and sincospi take about 97 of them per pair of normals.  With
+// tables (Tang's table-driven method, ACM TOMS 16, 1990) and short Taylor polynomials the
+// pair takes 28, at the same accuracy (-2 ln u within 3.2e-16 relative, sin and cos within
+// 1.9e-16): 1024 intervals put the reduced arguments below 2^-10 and pi/1024, where
+// degrees 6 (log), 5 (sin) and 4 (cos) are enough; gathers of 16 bytes from 33 KB of tables stay
+// in L1.  u = m 2^-33 with m = 2 x + 1 keeps every reduction exact.
+// ---------------------------------------------------------------------------
+constexpr int kTab = 1024;
+__device__ double2 g_log_tab[kTab];     // interval i of the mantissa: -2/c_i, 2 ln(1/c_i)
+__device__ double2 g_circle_tab[kTab];  // cos, sin of 2 pi (i + 1/2)/1024
+__device__ double g_ln2_tab[34];        // 2 k ln 2
+
+// -2 ln((x + 1/2) 2^-32).  The mantissa is taken in [3/4, 3/2), so that u near 1 has exponent
+// 0 and interval centre 1: the result keeps its relative accuracy there.
+__device__ __forceinline__ double minus_two_log(uint32_t x) {
+  const uint64_t m = 2ull * x + 1ull;
+  const int lz = __clzll((long long)m);
+  const uint64_t norm = m << lz;                 // leading one at bit 63
+  const uint32_t hi = (uint32_t)(norm >> 32);
+  const uint32_t half = (hi >> 30) & 1u;         // mantissa >= 3/2: halved
+  const double2 t = __ldg(&g_log_tab[(hi >> 21) & (kTab - 1)]);
+  const double k2 = __ldg(&g_ln2_tab[lz - 30 - (int)half]);
+  const double f = __longlong_as_double((long long)(((norm >> 11) & 0xFFFFFFFFFFFFFull) |
+                                                    ((uint64_t)(1023u - half) << 52)));
+  const double s = fma(f, t.x, 2.0);             // -2 r, r = f/c - 1
+  double p = fma(s, 1.0 / 192.0, 1.0 / 80.0);    // -2 ln(1 - s/2) = s + s^2/4 + s^3/12 + ...
+  p = fma(s, p, 1.0 / 32.0);
+  p = fma(s, p, 1.0 / 12.0);
+  p = fma(s, p, 0.25);
+  return (k2 + t.y) + fma(s * s, p, s);
+}
+
+// sqrt(x), x in [2e-10, 46]: the approximate reciprocal root instruction and one Householder
+// step of third order, sqrt = g + g e (1/2 + 3/8 e) with g = x y, e = 1 - g y.
+__device__ __forceinline__ double root_of(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double g = x * y, e = fma(-g, y, 1.0);
+  return fma(g * e, fma(e, 0.375, 0.5), g);
+}
+
+template <typename R> struct NormalPair : BoxMuller<R> {};
+template <> struct NormalPair<double> {
+  __device__ __forceinline__ static void apply(uint32_t a, uint32_t b, double& z0, double& z1) {
+    const double rad = root_of(minus_two_log(a));
+    // 2 pi (b + 1/2) 2^-32 = centre of sector b >> 22 plus t, |t| < pi/1024
+    const double2 cs = __ldg(&g_circle_tab[b >> 22]);
+    const double d = __hiloint2double(0x43300000, (int)(2u * (b & 0x3FFFFFu) + 1u)) - 4503599631564800.0;   // 2^52 + 2^22
+    const double t = d * 7.314590396335798e-10;
+    const double t2 = t * t;
+    const double st = fma(t * t2, fma(t2, 1.0 / 120.0, -1.0 / 6.0), t);
+    const double cm = t2 * fma(t2, 1.0 / 24.0, -0.5);   // cos t - 1
+    z0 = rad * fma(cs.x, cm, fma(-cs.y, st, cs.x));
+    z1 = rad * fma(cs.y, cm, fma(cs.x, st, cs.y));
+  }
+};
+
+// The 6 stress normals of one cell and step: (xx, yy, zz, xy, xz, yz).  Counters
+// (cell, step, call, 0), key (seed_lo, seed_hi): call 0 of the cell gives xx, yy, zz,
+// xy; call 1 serves two z planes: at the cell of plane 2m its words 0-1 give xz, yz of
+// that cell, words 2-3 those of the cell above it (plane 2m + 1).  `odd`: the cell's
+// plane is odd (its call 1 is the one at cell - plane).  KEYS: PhiloxKey or
+// PhiloxRoundKeys.
+template <typename R, typename KEYS>
+__device__ __forceinline__ void cell_normals(uint32_t cell, uint32_t plane, bool odd, uint32_t step, const KEYS& key,
+                                             R z[6]) {
+  const u32x4 a = philox4x32_10(u32x4{cell, step, 0u, 0u}, key);
+  const u32x4 b = philox4x32_10(u32x4{odd ? cell - plane : cell, step, 1u, 0u}, key);
+  NormalPair<R>::apply(a.x, a.y, z[0], z[1]);
+  NormalPair<R>::apply(a.z, a.w, z[2], z[3]);
+  NormalPair<R>::apply(odd ? b.z : b.x, odd ? b.w : b.y, z[4], z[5]);
+}
 
 // Shared memory of the marching block.
 //  * v: a ring of four velocity planes (three components, one-cell halo in x and y).
@@ -170,14 +247,7 @@ __device__ __forceinline__ void rhs_run(RhsSmem<R>& sm, const R* __restrict__ v,
   // offsets in 32 bits: 3 ncell <= 3 x 512^3 < 2^32
   const uint32_t nc = (uint32_t)g.ncell;
   const uint32_t plane = (uint32_t)g.nx * (uint32_t)g.ny;
-  // r = cc v + ce (sum of the six neighbours) + div Sigma - AB2, with cc = rho/dt - 6 ce,
-  // ce = (eta/2)/h^2; the 1/2 of every face or edge average of the advection is folded
-  // into its factor aq = rho/(4h)
-  const R ce = (R)(0.5 * g.eta / (g.h * g.h));
-  const R cc = (R)(g.rho / g.dt - 3.0 * g.eta / (g.h * g.h));
-  const R aq = g.advection ? (R)(0.25 * g.rho / g.h) : R(0);
-  const double s_amp = sqrt(g.kT * g.eta / (g.h * g.h * g.h * g.dt));
-  const R sd = (R)(2.0 * s_amp * (1.0 / g.h)), so = (R)(1.4142135623730951 * s_amp * (1.0 / g.h));
+  const R ce = rhs_c<R>(g).ce, cc = rhs_c<R>(g).cc, aq = rhs_c<R>(g).aq, sd = rhs_c<R>(g).sd, so = rhs_c<R>(g).so;
   const int lx = tx + 1, ly = ty + 1;
   {
     const int i0 = (int)(tile % ntx) * TX, j0 = (int)(tile / ntx) * TY;
@@ -402,6 +472,162 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 2 : 1) k_rhs_batch(const 
   }
 }
 
+// ---------------------------------------------------------------------------
+// The right-hand side in two passes, the normals stored in between: one thread per pair of
+// cells (planes 2m and 2m + 1 share a Philox call) draws them, one thread per cell takes the
+// stencils through L1.  No thread waits for another, no normal is drawn twice and a
+// grid of any size spreads over the whole device, where the marching block below needs its 512
+// threads' worth of cells per plane and a prologue of two planes.  Used
+//  * in FP64, always: the work is bound by the FP64 pipe, and the march draws 9% of its
+//    normals twice, for halos;
+//  * in FP32, up to kFlatCells: what the march saves (48 bytes per cell of stored normals)
+//    only pays where every SM marches many planes.
+// Measured with noise, both launches (us), march against stored normals: FP32 19.0 / 11.0 on
+// 32^3, 29.8 / 15.1 on 64^3, 29.9 / 25.3 on 96^3, 45.3 / 56.3 on 128^3, 275 / 386 on 256^3;
+// FP64 449 / 24 on 32^3 (eight marching blocks) and 1422 / 702 on 128^3, where half of the
+// gain is the cheaper normals above.
+// ---------------------------------------------------------------------------
+constexpr int kFlatThreads = 128;
+constexpr long long kFlatCells = 1ll << 20;
+
+// Normals of the pair `t` of cells: column t mod plane, planes 2 (t / plane) and the next.
+template <typename R>
+__device__ __forceinline__ void noise_pair(const GridParams& g, uint32_t t, uint32_t step, R* __restrict__ z) {
+  const uint32_t plane = (uint32_t)g.nx * (uint32_t)g.ny, nc = (uint32_t)g.ncell;
+  const uint32_t m = g.dny.div(g.dnx.div(t));
+  const uint32_t c0 = t + m * plane, c1 = c0 + plane;   // t = column + m plane
+  if (c0 >= nc) return;
+  const PhiloxKey key{g.key0, g.key1};
+  const u32x4 b = philox4x32_10(u32x4{c0, step, 1u, 0u}, key);
+  const u32x4 a = philox4x32_10(u32x4{c0, step, 0u, 0u}, key);
+  R p, q;
+  const auto put = [&](uint32_t cell, int first, int second) {
+    z[(size_t)first * nc + cell] = p;
+    z[(size_t)second * nc + cell] = q;
+  };
+  NormalPair<R>::apply(a.x, a.y, p, q);
+  put(c0, 0, 1);
+  NormalPair<R>::apply(a.z, a.w, p, q);
+  put(c0, 2, 3);
+  NormalPair<R>::apply(b.x, b.y, p, q);
+  put(c0, 4, 5);
+  if (c1 >= nc) return;
+  const u32x4 d = philox4x32_10(u32x4{c1, step, 0u, 0u}, key);
+  NormalPair<R>::apply(d.x, d.y, p, q);
+  put(c1, 0, 1);
+  NormalPair<R>::apply(d.z, d.w, p, q);
+  put(c1, 2, 3);
+  NormalPair<R>::apply(b.z, b.w, p, q);
+  put(c1, 4, 5);
+}
+
+// The right-hand side of one cell, the same sums as rhs_run's (its comments apply).
+template <typename R, bool NOISE>
+__device__ __forceinline__ void rhs_cell(const GridParams& g, uint32_t o, bool hist, const R* __restrict__ v,
+                                         R* __restrict__ adv, R* __restrict__ rhs, const R* __restrict__ z) {
+  const uint32_t nc = (uint32_t)g.ncell, nx = g.nx, plane = nx * (uint32_t)g.ny;
+  const uint32_t row = g.dnx.div(o), i = o - row * nx;
+  const uint32_t k = g.dny.div(row), j = row - k * (uint32_t)g.ny;
+  const uint32_t xp = i + 1 == nx ? o - (nx - 1) : o + 1, xm = i == 0 ? o + (nx - 1) : o - 1;
+  const uint32_t sy = plane - nx, sz = nc - plane;
+  const bool jl = j + 1 == (uint32_t)g.ny, jf = j == 0, kl = k + 1 == (uint32_t)g.nz, kf = k == 0;
+  const auto up = [&](uint32_t c) { return jl ? c - sy : c + nx; };
+  const auto down = [&](uint32_t c) { return jf ? c + sy : c - nx; };
+  const auto above = [&](uint32_t c) { return kl ? c - sz : c + plane; };
+  const auto below = [&](uint32_t c) { return kf ? c + sz : c - plane; };
+  const uint32_t yp = up(o), ym = down(o), zp = above(o), zm = below(o);
+  const R ce = rhs_c<R>(g).ce, cc = rhs_c<R>(g).cc, aq = rhs_c<R>(g).aq;
+  R ao[3] = {R(0), R(0), R(0)};
+  if (hist) {
+    ao[0] = adv[o];
+    ao[1] = adv[o + nc];
+    ao[2] = adv[o + 2 * nc];
+  }
+  const R *vx = v, *vy = v + nc, *vz = v + 2 * (size_t)nc;
+  const R x_c = vx[o], x_xp = vx[xp], x_xm = vx[xm], x_yp = vx[yp], x_ym = vx[ym], x_zp = vx[zp], x_zm = vx[zm];
+  const R y_c = vy[o], y_xp = vy[xp], y_xm = vy[xm], y_yp = vy[yp], y_ym = vy[ym], y_zp = vy[zp], y_zm = vy[zm];
+  const R z_c = vz[o], z_xp = vz[xp], z_xm = vz[xm], z_yp = vz[yp], z_ym = vz[ym], z_zp = vz[zp], z_zm = vz[zm];
+  R a[3] = {R(0), R(0), R(0)};
+  if (g.advection) {
+    const R x_xpym = vx[down(xp)], x_xpzm = vx[below(xp)], y_ypxm = vy[up(xm)], y_ypzm = vy[below(yp)];
+    const R z_zpxm = vz[above(xm)], z_zpym = vz[above(ym)];
+    const R exy_c = (x_c + x_ym) * (y_c + y_xm), exz_c = (x_c + x_zm) * (z_c + z_xm), eyz_c = (y_c + y_zm) * (z_c + z_ym);
+    const R ubx_c = x_xp + x_c, ubx_m = x_c + x_xm, uby_c = y_yp + y_c, uby_m = y_c + y_ym;
+    const R ubz_c = z_zp + z_c, ubz_m = z_c + z_zm;
+    // differences of products: (ubx_c^2 - ubx_m^2) + (exy(+y) - exy) + (exz(+z) - exz), ...
+    a[0] = aq * (fma(ubx_c, ubx_c, -ubx_m * ubx_m) + fma(x_yp + x_c, y_yp + y_ypxm, -exy_c) +
+                 fma(x_zp + x_c, z_zp + z_zpxm, -exz_c));
+    a[1] = aq * (fma(uby_c, uby_c, -uby_m * uby_m) + fma(x_xp + x_xpym, y_xp + y_c, -exy_c) +
+                 fma(y_zp + y_c, z_zp + z_zpym, -eyz_c));
+    a[2] = aq * (fma(ubz_c, ubz_c, -ubz_m * ubz_m) + fma(x_xp + x_xpzm, z_xp + z_c, -exz_c) +
+                 fma(y_yp + y_ypzm, z_yp + z_c, -eyz_c));
+  }
+  R f[3] = {R(0), R(0), R(0)};
+  if (NOISE) {
+    const R sd = rhs_c<R>(g).sd, so = rhs_c<R>(g).so;
+    const R *zxx = z, *zyy = z + nc, *zzz = z + 2 * (size_t)nc, *zxy = z + 3 * (size_t)nc, *zxz = z + 4 * (size_t)nc,
+            *zyz = z + 5 * (size_t)nc;
+    const R xy = zxy[o], xz = zxz[o], yz = zyz[o];
+    f[0] = fma(sd, zxx[o] - zxx[xm], so * ((zxy[yp] - xy) + (zxz[zp] - xz)));
+    f[1] = fma(sd, zyy[o] - zyy[ym], so * ((zxy[xp] - xy) + (zyz[zp] - yz)));
+    f[2] = fma(sd, zzz[o] - zzz[zm], so * ((zxz[xp] - xz) + (zyz[yp] - yz)));
+  }
+  if (!hist) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ao[c] = a[c];
+  }
+  const R nb[3] = {x_xp + x_xm + x_yp + x_ym + x_zp + x_zm, y_xp + y_xm + y_yp + y_ym + y_zp + y_zm,
+                   z_xp + z_xm + z_yp + z_ym + z_zp + z_zm};
+  const R own[3] = {x_c, y_c, z_c};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    adv[o + c * nc] = a[c];
+    rhs[o + c * nc] = fma(cc, own[c], fma(ce, nb[c], fma(R(0.5), ao[c], fma(R(-1.5), a[c], f[c]))));
+  }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kFlatThreads / 2) k_noise(GridParams g, R* __restrict__ z,
+                                                           const long long* __restrict__ step_dev) {
+  noise_pair<R>(g, blockIdx.x * (kFlatThreads / 2) + threadIdx.x, (uint32_t)(*step_dev), z);
+}
+
+template <typename R, bool NOISE>
+__global__ void __launch_bounds__(kFlatThreads) k_rhs_flat(GridParams g, const R* __restrict__ v, R* __restrict__ adv,
+                                                         R* __restrict__ rhs, const R* __restrict__ z,
+                                                         const int* __restrict__ hist_dev) {
+  const uint32_t o = blockIdx.x * kFlatThreads + threadIdx.x;
+  if (o < (uint32_t)g.ncell) rhs_cell<R, NOISE>(g, o, *hist_dev != 0, v, adv, rhs, z);
+}
+
+// The same over every member of a batch: block u of a member (units of 128 cells or 64 pairs).
+template <typename R>
+__device__ __forceinline__ int member_of_unit(const RhsMember<R>* __restrict__ mem, int nm, long long w) {
+  int a = 0, b = nm - 1;
+  while (a < b) {
+    const int c = (a + b + 1) / 2;
+    if (mem[c].w0 <= w) a = c; else b = c - 1;
+  }
+  return a;
+}
+template <typename R>
+__global__ void __launch_bounds__(kFlatThreads / 2) k_noise_batch(const RhsMember<R>* __restrict__ mem, int nm) {
+  const RhsMember<R>& m = mem[member_of_unit(mem, nm, blockIdx.x)];
+  noise_pair<R>(m.g, (uint32_t)(blockIdx.x - m.w0) * (kFlatThreads / 2) + threadIdx.x, (uint32_t)(*m.step_dev),
+                m.normals);
+}
+template <typename R, bool NOISE>
+__global__ void __launch_bounds__(kFlatThreads) k_rhs_flat_batch(const RhsMember<R>* __restrict__ mem, int nm) {
+  const RhsMember<R>& m = mem[member_of_unit(mem, nm, blockIdx.x)];
+  const uint32_t o = (uint32_t)(blockIdx.x - m.w0) * kFlatThreads + threadIdx.x;
+  if (o < (uint32_t)m.g.ncell) rhs_cell<R, NOISE>(m.g, o, *m.hist_dev != 0, m.v, m.adv, m.rhs, m.normals);
+}
+
+long long flat_units(long long plane, int nz) {
+  const long long pairs = plane * ((nz + 1) / 2), cells = plane * nz;
+  return std::max((cells + kFlatThreads - 1) / kFlatThreads, (2 * pairs + kFlatThreads - 1) / kFlatThreads);
+}
+
 template <typename R>
 __global__ void k_normals(GridParams g, uint32_t step, R* __restrict__ out) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -513,60 +739,83 @@ size_t rhs_smem() { return sizeof(RhsSmem<R>); }
 
 }  // namespace
 
+bool rhs_stored_normals(int precision, long long ncell) { return precision == 64 || ncell <= kFlatCells; }
+
 template <typename R>
-void explicit_rhs(const GridParams& g, const R* v, R* adv, R* rhs, const long long* step_dev, const int* hist_dev,
-                  cudaStream_t st) {
-  const dim3 block(TX, TY);
-  dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, 1);
-  if (g.kz > 0) {
-    grid.z = (g.nz + g.kz - 1) / g.kz;
-  } else {
-    // persistent: as many blocks as the SMs hold at once, never more than tile-planes
-    static int resident[2] = {0, 0};
-    int& res = resident[sizeof(R) == 4 ? 0 : 1];
-    if (res == 0) {
-      int dev = 0, nsm = 0, per = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-      if (g.kT > 0.0)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rhs<R, true>, NT, rhs_smem<R>());
-      else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rhs<R, false>, NT, rhs_smem<R>());
-      res = std::max(1, nsm) * std::max(1, per);
+void explicit_rhs(const GridParams& g, const R* v, R* adv, R* rhs, R* normals, const long long* step_dev,
+                  const int* hist_dev, cudaStream_t st) {
+  if (rhs_stored_normals(8 * sizeof(R), g.ncell)) {
+    const unsigned cells = (unsigned)((g.ncell + kFlatThreads - 1) / kFlatThreads);
+    if (g.kT > 0.0) {
+      const long long pairs = (long long)g.nx * g.ny * ((g.nz + 1) / 2);
+      k_noise<R><<<(unsigned)((2 * pairs + kFlatThreads - 1) / kFlatThreads), kFlatThreads / 2, 0, st>>>(g, normals, step_dev);
+      k_rhs_flat<R, true><<<cells, kFlatThreads, 0, st>>>(g, v, adv, rhs, normals, hist_dev);
+    } else {
+      k_rhs_flat<R, false><<<cells, kFlatThreads, 0, st>>>(g, v, adv, rhs, normals, hist_dev);
     }
-    // whole groups of grid.x blocks (one per tile of a tile row), never more groups
-    // than tile-row planes
-    const long long rows = (long long)grid.y * g.nz;
-    const long long ngrp = std::max<long long>(1, std::min<long long>(res / grid.x, rows));
-    grid = dim3((unsigned)(ngrp * grid.x), 1, 1);
+    return;
   }
-  if (g.kT > 0.0)
-    k_rhs<R, true><<<grid, block, rhs_smem<R>(), st>>>(v, adv, rhs, g, step_dev, hist_dev);
-  else
-    k_rhs<R, false><<<grid, block, rhs_smem<R>(), st>>>(v, adv, rhs, g, step_dev, hist_dev);
+  if constexpr (sizeof(R) == 4) {
+    const dim3 block(TX, TY);
+    dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, 1);
+    if (g.kz > 0) {
+      grid.z = (g.nz + g.kz - 1) / g.kz;
+    } else {
+      // persistent: as many blocks as the SMs hold at once, never more than tile-planes
+      static int res = 0;
+      if (res == 0) {
+        int dev = 0, nsm = 0, per = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (g.kT > 0.0)
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rhs<R, true>, NT, rhs_smem<R>());
+        else
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rhs<R, false>, NT, rhs_smem<R>());
+        res = std::max(1, nsm) * std::max(1, per);
+      }
+      // whole groups of grid.x blocks (one per tile of a tile row), never more groups
+      // than tile-row planes
+      const long long rows = (long long)grid.y * g.nz;
+      const long long ngrp = std::max<long long>(1, std::min<long long>(res / grid.x, rows));
+      grid = dim3((unsigned)(ngrp * grid.x), 1, 1);
+    }
+    if (g.kT > 0.0)
+      k_rhs<R, true><<<grid, block, rhs_smem<R>(), st>>>(v, adv, rhs, g, step_dev, hist_dev);
+    else
+      k_rhs<R, false><<<grid, block, rhs_smem<R>(), st>>>(v, adv, rhs, g, step_dev, hist_dev);
+  }
 }
 
-long long rhs_tile_planes(int nx, int ny, int nz) {
+long long rhs_batch_units(int precision, int nx, int ny, int nz) {
+  if (precision == 64) return flat_units((long long)nx * ny, nz);
   return (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY) * nz;
 }
 
 template <typename R>
 void batch_rhs(const RhsMember<R>* members, int nm, long long total, bool noise, cudaStream_t st) {
   if (nm <= 0 || total <= 0) return;
-  static int resident[2] = {0, 0};
-  int& res = resident[sizeof(R) == 4 ? 0 : 1];
-  if (res == 0) {
-    int dev = 0, nsm = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rhs_batch<R, true>, NT, rhs_smem<R>());
-    res = std::max(1, nsm) * std::max(1, per);
+  if constexpr (sizeof(R) == 8) {
+    if (noise) {
+      k_noise_batch<R><<<(unsigned)total, kFlatThreads / 2, 0, st>>>(members, nm);
+      k_rhs_flat_batch<R, true><<<(unsigned)total, kFlatThreads, 0, st>>>(members, nm);
+    } else {
+      k_rhs_flat_batch<R, false><<<(unsigned)total, kFlatThreads, 0, st>>>(members, nm);
+    }
+  } else {
+    static int res = 0;
+    if (res == 0) {
+      int dev = 0, nsm = 0, per = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_rhs_batch<R, true>, NT, rhs_smem<R>());
+      res = std::max(1, nsm) * std::max(1, per);
+    }
+    const dim3 grid((unsigned)std::min<long long>(res, total)), block(TX, TY);
+    if (noise)
+      k_rhs_batch<R, true><<<grid, block, rhs_smem<R>(), st>>>(members, nm, total);
+    else
+      k_rhs_batch<R, false><<<grid, block, rhs_smem<R>(), st>>>(members, nm, total);
   }
-  const dim3 grid((unsigned)std::min<long long>(res, total)), block(TX, TY);
-  if (noise)
-    k_rhs_batch<R, true><<<grid, block, rhs_smem<R>(), st>>>(members, nm, total);
-  else
-    k_rhs_batch<R, false><<<grid, block, rhs_smem<R>(), st>>>(members, nm, total);
 }
 
 template <typename R>
@@ -623,16 +872,49 @@ double fma_rate(int precision, int iters, int blocks_per_sm, cudaStream_t st, do
   return 2.0 * kFmaChains * (double)iters * blocks * threads / (ms * 1e-3);
 }
 
-void grid_prepare() {
+namespace {
+std::atomic<bool> g_tables_ready[64];   // by device
+int current_device() {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? dev : -1;
+}
+// The Box-Muller tables, correctly rounded from long double.
+struct NormalTables {
+  double2 log_tab[kTab], circle[kTab];
+  double ln2[34];
+  NormalTables() {
+    const long double pi = 3.141592653589793238462643383279502884L;
+    for (int i = 0; i < kTab; ++i) {
+      long double c = 1.0L + (i + 0.5L) / kTab;
+      if (i >= kTab / 2) c *= 0.5L;
+      const double inv = i == 0 || i == kTab - 1 ? 1.0 : (double)(1.0L / c);   // the intervals next to 1
+      log_tab[i] = make_double2(-2.0 * inv, (double)(2.0L * logl((long double)inv)));
+      circle[i] = make_double2((double)cosl(2.0L * pi * (i + 0.5L) / kTab), (double)sinl(2.0L * pi * (i + 0.5L) / kTab));
+    }
+    for (int k = 0; k < 34; ++k) ln2[k] = (double)(2.0L * k * logl(2.0L));
+  }
+};
+}  // namespace
+
+bool grid_prepare(cudaStream_t st) {
   cudaFuncSetAttribute(k_rhs<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<float>());
-  cudaFuncSetAttribute(k_rhs<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<double>());
   cudaFuncSetAttribute(k_rhs<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<float>());
-  cudaFuncSetAttribute(k_rhs<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<double>());
   cudaFuncSetAttribute(k_rhs_batch<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<float>());
-  cudaFuncSetAttribute(k_rhs_batch<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<double>());
   cudaFuncSetAttribute(k_rhs_batch<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<float>());
-  cudaFuncSetAttribute(k_rhs_batch<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)rhs_smem<double>());
+  const int dev = current_device();
+  if (dev >= 0 && g_tables_ready[dev].load()) return true;
+  static const NormalTables tables;   // outlives the copies below
+  return cudaMemcpyToSymbolAsync(g_log_tab, tables.log_tab, sizeof(tables.log_tab), 0, cudaMemcpyHostToDevice, st) ==
+             cudaSuccess &&
+         cudaMemcpyToSymbolAsync(g_circle_tab, tables.circle, sizeof(tables.circle), 0, cudaMemcpyHostToDevice, st) ==
+             cudaSuccess &&
+         cudaMemcpyToSymbolAsync(g_ln2_tab, tables.ln2, sizeof(tables.ln2), 0, cudaMemcpyHostToDevice, st) ==
+             cudaSuccess;
+}
+
+void grid_ready() {
+  const int dev = current_device();
+  if (dev >= 0) g_tables_ready[dev].store(true);
 }
 
 void scalars_before_step(double* scal, double dt, double, double, cudaStream_t st) {
@@ -644,7 +926,7 @@ void scalars_after_step(double* scal, double, double, double, bool inertial, lon
 }
 
 #define ICM_INST(R)                                                                                          \
-  template void explicit_rhs<R>(const GridParams&, const R*, R*, R*, const long long*, const int*, cudaStream_t); \
+  template void explicit_rhs<R>(const GridParams&, const R*, R*, R*, R*, const long long*, const int*, cudaStream_t); \
   template void batch_rhs<R>(const RhsMember<R>*, int, long long, bool, cudaStream_t);                        \
   template void stress_normals<R>(const GridParams&, long long, R*, cudaStream_t);                           \
   template void field_sums<R>(const R*, long long, double*, double*, int, cudaStream_t);                      \

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "icm_common.cuh"
@@ -138,11 +139,21 @@ double fma_rate(int precision, int iters, int blocks_per_sm, cudaStream_t st, do
 
 // Raise the dynamic shared-memory limits of the kernels (call once, outside capture).
 void fft_prepare();
-void grid_prepare();
+// (grid_prepare also queues the upload of the FP64 Box-Muller tables on st, once per device;
+// false if that fails.  grid_ready records that it has landed.)
+bool grid_prepare(cudaStream_t st);
+void grid_ready();
 
 // ---------------------------------------------------------------------------
 // Grid kernels (icm_grid.cu)
 // ---------------------------------------------------------------------------
+// The constants of the right-hand side, formed once on the host: formed from the parameters in
+// every thread they cost some 150 FP64 operations (a root and divisions at 1/64 of the FP32
+// rate), about 20 us per block of the marching kernel.
+template <typename R>
+struct RhsConst {
+  R ce, cc, aq, sd, so;   // see rhs_const
+};
 struct GridParams {
   int nx, ny, nz;
   long long ncell;
@@ -151,14 +162,32 @@ struct GridParams {
   PhiloxRoundKeys rk;   // the round keys of (key0, key1)
   int advection;
   int kz;           // z planes marched per block of the RHS kernel (>= 1)
+  FastDiv dnx, dny; // division by nx and ny
+  RhsConst<float> cf;
+  RhsConst<double> cd;
 };
+// r = cc v + ce (sum of the six neighbours) + div Sigma - AB2, with cc = rho/dt - 6 ce,
+// ce = (eta/2)/h^2; aq = rho/(4h) holds the 1/4 of the advection's averages; sd and so are
+// the amplitudes of the diagonal and off-diagonal stress differences.
+inline RhsConst<double> rhs_const(const GridParams& g) {
+  const double amp = sqrt(g.kT * g.eta / (g.h * g.h * g.h * g.dt));
+  return RhsConst<double>{0.5 * g.eta / (g.h * g.h), g.rho / g.dt - 3.0 * g.eta / (g.h * g.h),
+                          g.advection ? 0.25 * g.rho / g.h : 0.0, 2.0 * amp * (1.0 / g.h),
+                          1.4142135623730951 * amp * (1.0 / g.h)};
+}
+template <typename R> __host__ __device__ inline const RhsConst<R>& rhs_c(const GridParams& g);
+template <> __host__ __device__ inline const RhsConst<float>& rhs_c<float>(const GridParams& g) { return g.cf; }
+template <> __host__ __device__ inline const RhsConst<double>& rhs_c<double>(const GridParams& g) { return g.cd; }
 
 // r = (rho/dt) v + (eta/2) L v + div Sigma^n - (3/2 A^n - 1/2 A^{n-1}); adv <- A^n.
 // step_dev: device int64 time level (Philox counter word 1).  has_hist_dev: device
 // int, 0 = no history (A^{n-1} := A^n); set to 1 by the kernel launch sequence.
+// normals: scratch for the stress normals, 6 ncell values, where rhs_stored_normals says so.
 template <typename R>
-void explicit_rhs(const GridParams& g, const R* v, R* adv, R* rhs, const long long* step_dev,
+void explicit_rhs(const GridParams& g, const R* v, R* adv, R* rhs, R* normals, const long long* step_dev,
                   const int* has_hist_dev, cudaStream_t st);
+// Whether the right-hand side of a grid draws its normals in a pass of its own.
+bool rhs_stored_normals(int precision, long long ncell);
 
 template <typename R>
 void stress_normals(const GridParams& g, long long step, R* out, cudaStream_t st);
@@ -372,15 +401,17 @@ struct RhsMember {
   const R* v;
   R* adv;
   R* rhs;
+  R* normals;             // the member's scratch for its stress normals (FP64)
   const long long* step_dev;
   const int* hist_dev;
-  long long w0;           // first global tile-plane of the member
+  long long w0;           // first global work unit of the member: tile-planes (FP32), blocks of
+                          // the stored-normals passes (FP64)
 };
-// members[0 .. nm) in order of w0; total = the last member's w0 + its tile-planes.
+// members[0 .. nm) in order of w0; total = the last member's w0 + its units.
 template <typename R>
 void batch_rhs(const RhsMember<R>* members, int nm, long long total, bool noise, cudaStream_t st);
-// Tile-planes (32 x 16 cells per tile) of a grid in the RHS kernel.
-long long rhs_tile_planes(int nx, int ny, int nz);
+// Work units of a grid in the batched right-hand side.
+long long rhs_batch_units(int precision, int nx, int ny, int nz);
 
 // Scalar bookkeeping kernels.
 void scalars_before_step(double* scal, double dt, double rho, double dvf, cudaStream_t st);
