@@ -21,7 +21,9 @@ INCLUDE = os.path.join(os.path.dirname(PKG), "include")
 # (source, object name, extra flags): the FFT file is compiled as six shards in
 # parallel (x forward / y-z / x inverse passes, FP32 / FP64), the largest unit otherwise.
 SOURCES = [("icm_api.cu", "icm_api", ()), ("icm_grid.cu", "icm_grid", ()), ("icm_blob.cu", "icm_blob", ()),
-           ("icm_static.cu", "icm_static", ()), ("icm_couple.cu", "icm_couple", ())] + [
+           ("icm_static.cu", "icm_static", ()), ("icm_couple.cu", "icm_couple", ()),
+           ("icm_plane.cu", "icm_plane_32", ("-DICM_PLANE_PREC=32",)),
+           ("icm_plane.cu", "icm_plane_64", ("-DICM_PLANE_PREC=64",))] + [
     ("icm_fft.cu", "icm_fft_%d" % k, ("-DICM_FFT_SHARD=%d" % k,)) for k in range(6)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "--expt-relaxed-constexpr"]

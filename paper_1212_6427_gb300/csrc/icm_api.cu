@@ -54,15 +54,25 @@ bool side_ok(int n) {
   return n == 1;
 }
 
+// The factors of a side without two-stage register kernels, each in {2, 3, 4, 6, 8, 9, 12}: as few
+// as possible (every further one is a pass over shared memory), then as even as
+// possible, the smallest last (the z pass holds three components of that many values).
 std::vector<int> factor_radices(int n) {
-  std::vector<int> r;
-  int m = n;
-  while (m % 16 == 0) { r.push_back(16); m /= 16; }
-  if (m % 8 == 0) { r.push_back(8); m /= 8; }
-  if (m % 4 == 0) { r.push_back(4); m /= 4; }
-  if (m % 2 == 0) { r.push_back(2); m /= 2; }
-  while (m % 3 == 0) { r.push_back(3); m /= 3; }
-  return r;
+  static const int rad[] = {2, 3, 4, 6, 8, 9, 12};
+  std::vector<int> best;
+  for (int a : rad) {
+    if (n % a) continue;
+    for (int b : rad) {
+      if (b > a || (n / a) % b) continue;
+      const int c = n / a / b;
+      if (c == 1) {
+        if (best.empty() || best.size() > 2 || best[0] > a) best = {a, b};
+      } else if (c <= b && c != 5 && c != 7 && c != 10 && c != 11 && (best.empty() || (best.size() == 3 && best[0] > a))) {
+        best = {a, b, c};
+      }
+    }
+  }
+  return best;
 }
 
 double kernel_sum_sq(int kernel) { return kernel == 3 ? 0.5 : 0.375; }
@@ -125,6 +135,7 @@ struct icm_sim {
   bool any_me = false, any_force = false;
   // row-block bins of the blob work fused into the x passes (register FFT sides)
   bool fused = false;
+  bool plane = false;         // the grid's planes have passes of their own (plane_has_passes)
   int nrowblk = 0;
   int* bin_idx = nullptr;     // count [nrowblk], start [nrowblk + 1], cursor [nrowblk]
   void* bin_blob = nullptr;   // list [kBinsPerBlob cap] ints, geometry [cap], accumulators [12 cap]
@@ -172,9 +183,10 @@ namespace {
 // Per blob slot: the bin list (kBinsPerBlob ints), the stencil record and 4 (n,3)
 // FP64 accumulators.
 constexpr size_t kGeoBytes = kStencilBytes;
-constexpr int kAccPerBlob = 12;
+constexpr int kAccPerBlob = 12;       // accumulators of the x passes
+constexpr int kPartsPerBlob = 3 * kPlaneParts;   // or the partial sums of the plane passes, in the same place
 size_t bin_list_bytes(long long cap) { return ((size_t)kBinsPerBlob * 4 * cap + 255) / 256 * 256; }
-size_t bin_blob_bytes(long long cap) { return bin_list_bytes(cap) + (kGeoBytes + 8 * kAccPerBlob) * cap; }
+size_t bin_blob_bytes(long long cap) { return bin_list_bytes(cap) + (kGeoBytes + 8 * kPartsPerBlob) * cap; }
 
 void* dalloc(icm_sim* s, size_t bytes) {
   void* p = nullptr;
@@ -513,8 +525,17 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
   const double gath = nb * 3.0 * w3 * sizeof(R);
   // forward x and y passes fused on clusters (a plan choice on grids that allow it)
   const bool xy = s->plan.fused_xy && fft_has_xy_passes(s->prec, s->nx, s->ny);
+  // whole planes in shared memory: the x and y passes of a solve in one launch per direction
+  const bool plane = s->plane && !xy;
   auto solve = [&](const char* tag, const R* src, R* dst, R* dst2, int mode, double a, double b, const double* k0) {
     std::string t(tag);
+    if (plane) {
+      ICM_STAGE((t + ".xy_fwd").c_str(), F + S, plane_forward<R>(fc, src, nullptr, nullptr, 1, st));
+      ICM_STAGE((t + ".z_sym").c_str(), 2 * S, fft_z_symbol<R>(fc, a, b, k0, k0 ? k0scale : 0.0, st));
+      ICM_STAGE((t + ".yx_inv").c_str(), S + (mode == OUT_STORE ? F : 3 * F),
+                plane_inverse<R>(fc, dst, dst2, mode, nullptr, nullptr, 1, st));
+      return;
+    }
     if (xy) {
       ICM_STAGE((t + ".xy_fwd").c_str(), F + S, fft_xy_forward<R>(fc, src, nullptr, st));
     } else {
@@ -532,9 +553,11 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
       s->nb == 0 ? nullptr : ((s->trap_k != 0.0 || wca) ? s->fe : (s->any_force ? s->f : nullptr));
   // thermal drift (Appendix B.2) at q^{n+1/2}, added to the right-hand side of the first solve
   const bool drift = (s->flags & ICM_FLAG_THERMAL_DRIFT) && s->kT > 0.0 && s->nb > 0;
-  const bool fused = s->fused && s->plan.fused_blobs && s->nb > 0 && segment < 0;
-  const RowBins bins = row_bins(s);
   const double geob = (double)(12 * sizeof(int) + 36 * sizeof(R));   // stencil record per blob
+  // blob work inside the plane passes or the x passes
+  const bool in_plane = plane && s->plan.fused_blobs && s->nb > 0 && segment < 0;
+  const bool fused = !in_plane && s->fused && s->plan.fused_blobs && s->nb > 0 && segment < 0;
+  const RowBins bins = row_bins(s);
 
   // The blob-side prologue (scalars, predictor, pair forces, bins) reads only v and the
   // blob state: in the step graph it runs on a second stream beside the RHS and joins
@@ -553,7 +576,10 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
   }
   ICM_STAGE("scalars", 0, scalars_before_step(s->scal, s->dt, s->rho, dvf, sb));
   // step 1: midpoint predictor (Eq. particle_pred)
-  ICM_STAGE("predict", 2 * gath + nb * 72, blob_predict<R>(bp, bs, v, sb));
+  PlaneRecords rec{};
+  if (in_plane) rec = PlaneRecords{s->geo, s->bin_list, (int)s->cap};
+  ICM_STAGE("predict", 2 * gath + nb * (72 + (in_plane ? geob + 8.0 : 0.0)),
+            blob_predict<R>(bp, bs, v, sb, rec));
   // pair forces at q^{n+1/2} (four kernels: cell count, scan, fill, forces)
   if (wca) ICM_STAGE("wca", nb * 96, blob_wca_forces(bp, bs, wca_params(s), s->trap_k != 0.0, sb));
   if (fused)
@@ -563,6 +589,48 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
   ICM_STAGE("rhs", 4 * F, explicit_rhs<R>(gp, v, adv, work, (R*)s->normals, s->step_dev, s->hist_dev, st));
   if (fork) cudaStreamWaitEvent(st, s->ev_join, 0);
   if (drift) ICM_STAGE("drift", 2 * gath + nb * 32, blob_spread_drift<R>(bp, bs, work, st));
+  if (in_plane) {
+    // The blob work of steps 2-9 runs inside the plane passes: the spreads (with the elementwise
+    // updates of steps 4 and 6 that feed them) in the forward pass of the solve they feed,
+    // the interpolations in the inverse pass of the solve whose output they read.
+    PlaneBlobs pb;
+    pb.p = bp;
+    pb.s = bs;
+    pb.geo = s->geo;
+    pb.zfirst = s->bin_list;
+    pb.zstride = (int)s->cap;
+    const long long n3 = 3 * s->nb;
+    pb.jvt = s->acc;
+    pb.jdvt = s->acc + 4 * n3;
+    const double blobio = nb * (geob + 24.0);
+    auto passes = [&](const char* tag, const R* src, int source, const double* vec, double a, double b, const double* k0,
+                      R* dst, int mode, double* part, double* part_lap) {
+      std::string t(tag);
+      PlaneBlobs w = pb;
+      w.source = source;
+      w.vec = vec;
+      w.part = part;
+      w.part_lap = part_lap;
+      const bool spreads = source != PLANE_VEC || vec != nullptr;
+      ICM_STAGE((t + ".xy_fwd").c_str(), (src ? F : 0.0) + S + (spreads ? blobio : 0.0),
+                plane_forward<R>(fc, src, spreads ? &w : nullptr, nullptr, 1, st));
+      ICM_STAGE((t + ".z_sym").c_str(), 2 * S, fft_z_symbol<R>(fc, a, b, k0, k0 ? k0scale : 0.0, st));
+      const double out = mode == OUT_STORE ? F : (mode == OUT_ADD ? 2 * F : 0.0);
+      ICM_STAGE((t + ".yx_inv").c_str(), S + out + blobio, plane_inverse<R>(fc, dst, nullptr, mode, &w, nullptr, 1, st));
+    };
+    passes("rt1", work, PLANE_VEC, fvec, s->rho / s->dt, 0.5 * s->eta, s->scal + SC_K0, v, OUT_STORE, s->acc, nullptr);
+    if (s->any_me) {
+      // steps 4 and 5: dv~ = m~_f / (rho (m~_f + m_e)) P S dp; only J dv~ is kept
+      passes("rt2", nullptr, PLANE_CDP, nullptr, 1.0, 0.0, nullptr, v, OUT_NONE, s->acc + 4 * n3, nullptr);
+      // steps 6 and 7: (rho - dt/2 eta L) dv + dt grad dpi = S (dp - m_e J dv~); v = v~ + dv
+      passes("rt3", nullptr, PLANE_SRC, nullptr, s->rho, 0.5 * s->dt * s->eta, s->scal + SC_SUMSRC, v, OUT_ADD,
+             s->acc + 8 * n3, s->acc + 12 * n3);
+    }
+    // steps 8 and 9, the lagged slip term and the end-of-step scalars
+    ICM_STAGE("finish", nb * (s->any_me ? 264 : 144),
+              blob_finish_plane(bp, bs, s->acc, s->any_me, s->step_dev, s->hist_dev, st));
+    return;
+  }
   if (fused) {
     // The blob work of steps 2-9 runs inside the x passes of the three solves: the
     // spreads in the forward pass of the solve they feed, the interpolations in the
@@ -732,7 +800,7 @@ icm_status grow_blobs(icm_sim* s, long long need) {
     ICM_CK(cudaMemcpyAsync(me, s->me, sizeof(double) * s->nb, cudaMemcpyDeviceToDevice, s->stream));
   }
   void* nbin = nullptr;
-  if (s->fused) {
+  if (s->fused || s->plane) {
     nbin = dalloc(s, bin_blob_bytes(cap));
     if (!nbin) {
       ICM_CK(cudaStreamSynchronize(s->stream));
@@ -743,7 +811,7 @@ icm_status grow_blobs(icm_sim* s, long long need) {
   ICM_CK(cudaStreamSynchronize(s->stream));
   if (s->blob) dfree(s, s->blob);
   s->blob = nbuf;
-  if (s->fused) {
+  if (s->fused || s->plane) {
     if (s->bin_blob) dfree(s, s->bin_blob);
     s->bin_blob = nbin;
     s->bin_list = (int*)nbin;
@@ -1034,6 +1102,7 @@ icm_status icm_create(const int32_t grid[3], double h, double rho, double eta, d
   }
   s->has_zmap = make_zmap(s->zmap, s->spec, s->prec, s->kx, s->kxp, s->ny, s->nz);
   s->fused = fft_has_blob_passes(s->nx);
+  s->plane = plane_has_passes(s->prec, s->nx, s->ny, s->nz);
   if (s->fused) {
     s->nrowblk = (int)((s->ny * (long long)s->nz + 31) / 32);
     s->bin_idx = (int*)dalloc(s, sizeof(int) * (3 * (size_t)s->nrowblk + 1));
@@ -1276,7 +1345,7 @@ icm_status icm_autotune(icm_sim* s, int32_t nsteps, icm_plan* chosen, double* ms
   st = trial(best, best_ms);
   // one choice at a time, the others held at the best so far
   std::vector<std::pair<int icm_plan::*, std::vector<int>>> knobs;
-  if (s->fused) knobs.push_back({&icm_plan::fused_blobs, {1, 0}});
+  if (s->fused || s->plane) knobs.push_back({&icm_plan::fused_blobs, {1, 0}});
   if (s->has_zmap) knobs.push_back({&icm_plan::tma_z, {1, 0}});
   knobs.push_back({&icm_plan::rhs_kz, {0, 8, 16, 32}});
   knobs.push_back({&icm_plan::fork, {1, 0}});
@@ -2001,7 +2070,10 @@ icm_status batch_capture_stages(icm_batch* b) {
   };
   cudaGraph_t graph = nullptr;
   ICM_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-  batch_scalars_before(d_all, n_all, st);
+  if constexpr (sizeof(R) == 8)
+    batch_noise<R>(d_rn, (int)rhs_noise.size(), tot_noise, d_all, n_all, st);
+  else
+    batch_scalars_before(d_all, n_all, st);
   batch_predict<R>(d_all, d_mall, nb_all, st);
   if (blobs) batch_bins<R>(d_all, d_mall, nb_all, n_all, st);
   batch_rhs<R>(d_rn, (int)rhs_noise.size(), tot_noise, true, st);

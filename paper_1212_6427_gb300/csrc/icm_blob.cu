@@ -207,9 +207,11 @@ __device__ __forceinline__ double pick3(const double v[3], int a) { return a == 
 // image of the centre), goes to fe and dt times its trap part to the prescribed grid
 // sum K0 of the first solve (one atomic per block and component).
 // Blob b of the predictor, by one warp; returns (in lanes 0-2) the trap force component.
+// With rec set, the stencil at q^{n+1/2} also goes to the blob's record for the plane passes.
 template <typename R, int K>
 __device__ __forceinline__ double predict_blob(const BlobParams& p, const BlobState& s, const R* __restrict__ v,
-                                               long long b, int lane, WarpStencil<R, K>& S) {
+                                               long long b, int lane, WarpStencil<R, K>& S,
+                                               const PlaneRecords& rec = PlaneRecords{}) {
   double q[3], w0[3], qh[3], w1[3];
   load3(s.q, b, q);
   build_stencil<R, K>(S, q, p, false, lane);
@@ -220,6 +222,17 @@ __device__ __forceinline__ double predict_blob(const BlobParams& p, const BlobSt
   for (int a = 0; a < 3; ++a) qh[a] = __shfl_sync(0xffffffffu, mine, a);
   __syncwarp();
   build_stencil<R, K>(S, qh, p, false, lane);
+  if (rec.geo != nullptr) {
+    BlobStencil<R>& out = reinterpret_cast<BlobStencil<R>*>(rec.geo)[b];
+    if (lane < 9) {
+      const int comp = lane / 3, ax = lane % 3;
+      out.first[comp][ax] = S.first[comp][ax];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) out.w[comp][ax][a] = a < K ? S.w[comp][ax][a < K ? a : 0] : R(0);
+    } else if (lane < 11) {
+      rec.zfirst[(lane - 9) * rec.zstride + b] = S.first[lane == 9 ? 2 : 0][2];
+    }
+  }
   gather<R, K>(S, v, p, lane, w1);
   if (lane == 0) {
     store3(s.w0, b, w0);
@@ -237,13 +250,14 @@ __device__ __forceinline__ double predict_blob(const BlobParams& p, const BlobSt
 }
 
 template <typename R, int K>
-__global__ void __launch_bounds__(32 * kWarps) k_predict(BlobParams p, BlobState s, const R* __restrict__ v) {
+__global__ void __launch_bounds__(32 * kWarps) k_predict(BlobParams p, BlobState s, const R* __restrict__ v,
+                                                         PlaneRecords rec) {
   __shared__ WarpStencil<R, K> sten[kWarps];
   __shared__ double red[kWarps][3];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long b = (long long)blockIdx.x * kWarps + wid;
   double ftrap = 0.0;
-  if (b < s.nb) ftrap = predict_blob<R, K>(p, s, v, b, lane, sten[wid]);
+  if (b < s.nb) ftrap = predict_blob<R, K>(p, s, v, b, lane, sten[wid], rec);
   if (p.trap_k == 0.0) return;   // uniform over the launch
   if (lane < 3) red[wid][lane] = ftrap;
   __syncthreads();
@@ -546,11 +560,7 @@ __global__ void k_bzero(const BlobMember* __restrict__ mem, const long long* __r
 __global__ void k_bscal_before(const BlobMember* __restrict__ mem) {
   const BlobMember& m = mem[blockIdx.x];
   const int a = threadIdx.x;
-  if (a < 3) {
-    double* scal = m.s.scal;
-    scal[SC_K0 + a] = scal[SC_PBAR + a] + m.p.dt * scal[SC_SUMF + a];
-    scal[SC_SUMSRC + a] = 0.0;
-  }
+  if (a < 3) scalars_before(m.s.scal, m.p.dt, a);
 }
 
 __global__ void k_bscal_after(const BlobMember* __restrict__ mem) {
@@ -732,6 +742,40 @@ __global__ void k_finish_from(BlobParams p, BlobState s, const double* __restric
   }
 }
 
+// The same for the plane passes, which form the sources of steps 5 and 6 on the fly: the slip
+// correction and u^{n+1} = J (v~ + dv~) + du of step 8 are formed here, from the state of step n.
+__global__ void k_finish_plane(BlobParams p, BlobState s, const double* __restrict__ parts, int inertial,
+                               long long* __restrict__ step_dev, int* __restrict__ hist_dev) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x, n3 = 3 * s.nb;
+  if (i < n3) {
+    const int a = (int)(i % 3);
+    const int K = p.kernel;
+    const double jvt = plane_sum(parts, n3, i, K);
+    double u = jvt, jv = jvt, g = 0.0;
+    if (inertial) {
+      double du = p.slip == 1 ? 0.0 : 0.5 * (p.eta / p.rho) * p.dt * s.g[i];
+      if (p.slip == 2) du += s.w1[i] - s.w0[i];
+      u = jvt + plane_sum(parts + 4 * n3, n3, i, K) + du;
+      jv = jvt + plane_sum(parts + 8 * n3, n3, i, K);
+      g = plane_sum(parts + 12 * n3, n3, i, K + 2) * (p.inv_h * p.inv_h);
+    }
+    const double qn = wrap_pos(fma(0.5 * p.dt, jv + s.w1[i], s.q[i]), p.box[a], p.inv_box[a]);
+    s.q[i] = qn;
+    s.u[i] = u;
+    s.g[i] = g;
+    if (!isfinite(qn) || !isfinite(u)) atomicOr(s.err, DEV_ERR_NONFINITE);
+    if (fabs(u) * p.dt > p.h) atomicOr(s.err, DEV_ERR_CFL);
+  }
+  if (blockIdx.x == 0) {
+    const int a = threadIdx.x;
+    if (a < 3) s.scal[SC_PBAR + a] = s.scal[SC_K0 + a] + (inertial ? s.scal[SC_SUMSRC + a] : 0.0);
+    if (a == 0) {
+      *step_dev += 1;
+      *hist_dev = 1;
+    }
+  }
+}
+
 // The same over every member of a batch: one thread per blob (bins) or per blob
 // component (the elementwise steps); the member's accumulators are its bins.acc.
 template <typename R>
@@ -893,6 +937,11 @@ void blob_finish_from(const BlobParams& p, BlobState s, const double* base, cons
     k_finish_from<<<eblocks(3 * s.nb), 256, 0, st>>>(p, s, base, add, g, inertial ? 1 : 0, step_dev, hist_dev);
 }
 
+void blob_finish_plane(const BlobParams& p, BlobState s, const double* parts, bool inertial, long long* step_dev,
+                       int* hist_dev, cudaStream_t st) {
+  if (s.nb > 0) k_finish_plane<<<eblocks(3 * s.nb), 256, 0, st>>>(p, s, parts, inertial ? 1 : 0, step_dev, hist_dev);
+}
+
 #define ICM_KSWITCH(call3, call4) \
   if (p.kernel == 3) {            \
     call3;                        \
@@ -959,10 +1008,10 @@ ICM_BINST(double)
 #undef ICM_BINST
 
 template <typename R>
-void blob_predict(const BlobParams& p, BlobState s, const R* v, cudaStream_t st) {
+void blob_predict(const BlobParams& p, BlobState s, const R* v, cudaStream_t st, PlaneRecords rec) {
   if (s.nb <= 0) return;
-  ICM_KSWITCH((k_predict<R, 3><<<nblocks(s.nb), 32 * kWarps, 0, st>>>(p, s, v)),
-              (k_predict<R, 4><<<nblocks(s.nb), 32 * kWarps, 0, st>>>(p, s, v)))
+  ICM_KSWITCH((k_predict<R, 3><<<nblocks(s.nb), 32 * kWarps, 0, st>>>(p, s, v, rec)),
+              (k_predict<R, 4><<<nblocks(s.nb), 32 * kWarps, 0, st>>>(p, s, v, rec)))
 }
 template <typename R>
 void blob_spread(const BlobParams& p, long long nb, const double* q, const double* vec, R* field, cudaStream_t st) {
@@ -1093,7 +1142,7 @@ void blob_spread_drift(const BlobParams& p, BlobState s, R* field, cudaStream_t 
 }
 
 #define ICM_INST(R)                                                                                            \
-  template void blob_predict<R>(const BlobParams&, BlobState, const R*, cudaStream_t);                        \
+  template void blob_predict<R>(const BlobParams&, BlobState, const R*, cudaStream_t, PlaneRecords);          \
   template void blob_spread<R>(const BlobParams&, long long, const double*, const double*, R*, cudaStream_t); \
   template void blob_momentum_change<R>(const BlobParams&, BlobState, const R*, cudaStream_t);                \
   template void blob_inertial<R>(const BlobParams&, BlobState, const R*, cudaStream_t);                       \

@@ -27,114 +27,13 @@
 #include "icm_internal.h"
 #include "icm_fft_reg.cuh"
 #include "icm_rows.cuh"
+#include "icm_symbol.cuh"
 
 // Each shard uses only part of the helpers below.
 #pragma nv_diag_suppress 177
 
 namespace icm {
 namespace {
-
-// ---------------------------------------------------------------------------
-// Small DFTs in registers (forward, W = exp(-2 pi i / R)).
-// ---------------------------------------------------------------------------
-template <typename C> __device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3) {
-  const C s02 = cadd(a0, a2), d02 = csub(a0, a2), s13 = cadd(a1, a3), d13 = csub(a1, a3);
-  a0 = cadd(s02, s13);
-  a2 = csub(s02, s13);
-  a1 = cadd(d02, cmul_mi(d13));
-  a3 = cadd(d02, cmul_pi(d13));
-}
-
-// multiply by exp(-2 pi i m / 16); m is a compile-time constant after unrolling
-template <typename R> __device__ __forceinline__ cplx_t<R> w16mul(cplx_t<R> a, int m) {
-  const R c1 = R(0.92387953251128675613), s1 = R(0.38268343236508977173), r2 = R(0.70710678118654752440);
-  R c, s;  // exp(-i t) = c - i s
-  switch (m & 15) {
-    case 0: return a;
-    case 1: c = c1; s = s1; break;
-    case 2: c = r2; s = r2; break;
-    case 3: c = s1; s = c1; break;
-    case 4: return cmul_mi(a);
-    case 5: c = -s1; s = c1; break;
-    case 6: c = -r2; s = r2; break;
-    case 7: c = -c1; s = s1; break;
-    case 8: return mk(-a.x, -a.y);
-    case 9: c = -c1; s = -s1; break;
-    case 10: c = -r2; s = -r2; break;
-    case 11: c = -s1; s = -c1; break;
-    case 12: return cmul_pi(a);
-    case 13: c = s1; s = -c1; break;
-    case 14: c = r2; s = -r2; break;
-    default: c = c1; s = -s1; break;
-  }
-  return mk(a.x * c + a.y * s, a.y * c - a.x * s);
-}
-
-template <typename R, int RAD> struct Dft;
-template <typename R> struct Dft<R, 2> {
-  __device__ __forceinline__ static void run(cplx_t<R>* a) {
-    const cplx_t<R> t = a[0];
-    a[0] = cadd(t, a[1]);
-    a[1] = csub(t, a[1]);
-  }
-};
-template <typename R> struct Dft<R, 3> {
-  __device__ __forceinline__ static void run(cplx_t<R>* a) {
-    const R s = R(0.86602540378443864676);
-    const cplx_t<R> t1 = cadd(a[1], a[2]);
-    const cplx_t<R> t2 = mk(a[0].x - R(0.5) * t1.x, a[0].y - R(0.5) * t1.y);
-    const cplx_t<R> d = csub(a[1], a[2]);
-    const cplx_t<R> t3 = mk(s * d.x, s * d.y);
-    a[0] = cadd(a[0], t1);
-    a[1] = cadd(t2, cmul_mi(t3));
-    a[2] = cadd(t2, cmul_pi(t3));
-  }
-};
-template <typename R> struct Dft<R, 4> {
-  __device__ __forceinline__ static void run(cplx_t<R>* a) { dft4(a[0], a[1], a[2], a[3]); }
-};
-template <typename R> struct Dft<R, 8> {
-  // 8 = 2 x 4: b_k2[n1] = W8^(n1 k2) sum_n2 x[n1 + 4 n2] W2^(n2 k2); X[2 k1 + k2] = DFT4(b_k2)[k1]
-  __device__ __forceinline__ static void run(cplx_t<R>* a) {
-    cplx_t<R> b0[4], b1[4];
-#pragma unroll
-    for (int n1 = 0; n1 < 4; ++n1) {
-      b0[n1] = cadd(a[n1], a[n1 + 4]);
-      b1[n1] = w16mul<R>(csub(a[n1], a[n1 + 4]), 2 * n1);
-    }
-    dft4(b0[0], b0[1], b0[2], b0[3]);
-    dft4(b1[0], b1[1], b1[2], b1[3]);
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) {
-      a[2 * k1] = b0[k1];
-      a[2 * k1 + 1] = b1[k1];
-    }
-  }
-};
-template <typename R> struct Dft<R, 16> {
-  // 16 = 4 x 4: t[n1][k2] = W16^(n1 k2) DFT4_n2(x[n1 + 4 n2])[k2]; X[4 k1 + k2] = DFT4_n1(t[.][k2])[k1]
-  __device__ __forceinline__ static void run(cplx_t<R>* a) {
-    cplx_t<R> t[16];
-#pragma unroll
-    for (int n1 = 0; n1 < 4; ++n1) {
-      cplx_t<R> y0 = a[n1], y1 = a[n1 + 4], y2 = a[n1 + 8], y3 = a[n1 + 12];
-      dft4(y0, y1, y2, y3);
-      t[n1 * 4 + 0] = y0;
-      t[n1 * 4 + 1] = w16mul<R>(y1, n1);
-      t[n1 * 4 + 2] = w16mul<R>(y2, 2 * n1);
-      t[n1 * 4 + 3] = w16mul<R>(y3, 3 * n1);
-    }
-#pragma unroll
-    for (int k2 = 0; k2 < 4; ++k2) {
-      cplx_t<R> z0 = t[k2], z1 = t[4 + k2], z2 = t[8 + k2], z3 = t[12 + k2];
-      dft4(z0, z1, z2, z3);
-      a[k2] = z0;
-      a[4 + k2] = z1;
-      a[8 + k2] = z2;
-      a[12 + k2] = z3;
-    }
-  }
-};
 
 // One in-place stage over ncomp groups of NL interleaved lines: element (pos, line)
 // of group c is s[c*cs + pos*LS + line].  Sub-transform length M, radix RAD.
@@ -166,11 +65,11 @@ __device__ __forceinline__ void fft_stage(cplx_t<R>* s, int N, int M, int LS, in
         a[r] = cconj(a[r]);
         if (r > 0) a[r] = cmul(a[r], tw[n1 * r * tws]);
       }
-      Dft<R, RAD>::run(a);
+      SDft<R, RAD>::run(a);
 #pragma unroll
       for (int r = 0; r < RAD; ++r) a[r] = cconj(a[r]);
     } else {
-      Dft<R, RAD>::run(a);
+      SDft<R, RAD>::run(a);
 #pragma unroll
       for (int r = 1; r < RAD; ++r) a[r] = cmul(a[r], tw[n1 * r * tws]);
     }
@@ -195,6 +94,9 @@ __device__ void run_fft(cplx_t<R>* s, const AxisPlan& P, int LS, int ncomp, int 
       case 2: fft_stage<R, 2, INV, NL>(s, P.n, m, LS, ncomp, cs, tw, tid, nthr); break;
       case 3: fft_stage<R, 3, INV, NL>(s, P.n, m, LS, ncomp, cs, tw, tid, nthr); break;
       case 4: fft_stage<R, 4, INV, NL>(s, P.n, m, LS, ncomp, cs, tw, tid, nthr); break;
+      case 6: fft_stage<R, 6, INV, NL>(s, P.n, m, LS, ncomp, cs, tw, tid, nthr); break;
+      case 9: fft_stage<R, 9, INV, NL>(s, P.n, m, LS, ncomp, cs, tw, tid, nthr); break;
+      case 12: fft_stage<R, 12, INV, NL>(s, P.n, m, LS, ncomp, cs, tw, tid, nthr); break;
       case 8: fft_stage<R, 8, INV, NL>(s, P.n, m, LS, ncomp, cs, tw, tid, nthr); break;
       default: fft_stage<R, 16, INV, NL>(s, P.n, m, LS, ncomp, cs, tw, tid, nthr); break;
     }
@@ -328,111 +230,6 @@ __global__ void __launch_bounds__(kThreads) k_ypass(cplx_t<R>* __restrict__ spec
   for (int idx = tid; idx < N * NL; idx += kThreads) {
     const int t = idx % NL, y = idx / NL;
     if (kx0 + t < kx) base[(size_t)y * kxp + t] = lines[idx];
-  }
-}
-
-template <typename R>
-struct SymParams {
-  R a, b, inv_ntot;
-  R mean_scale;   // the symbol's scale on the mean mode: 1/(a ncell), 0 when a = 0
-  const cplx_t<R>* dx; const R* ddx;
-  const cplx_t<R>* dy; const R* ddy;
-  const cplx_t<R>* dz; const R* ddz;
-  const double* k0sum;
-  double k0mul;   // k0scale / ncell
-};
-
-// P^ w / (a + b|d|^2) / ncell on one wave vector: (P^ w)_a = w_a - conj(d_a)(d . w)/|d|^2,
-// identity on the mean mode, whose value is replaced by the FP64 bookkeeping if given
-// (and which is zero when a = 0).
-// 1/x: the hardware reciprocal in FP32 (within one ulp: a few roundings more than two
-// divisions per wave vector, far inside the FP32 path's tolerance), exact division in FP64.
-template <typename R> __device__ __forceinline__ R recip(R x);
-template <> __device__ __forceinline__ float recip<float>(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));   // within one ulp; x is never denormal here
-  return r;
-}
-template <> __device__ __forceinline__ double recip<double>(double x) { return 1.0 / x; }
-
-template <typename R>
-__device__ __forceinline__ void apply_symbol(cplx_t<R>& c0, cplx_t<R>& c1, cplx_t<R>& c2, cplx_t<R> d0,
-                                             cplx_t<R> d1, cplx_t<R> d2, R dd, const SymParams<R>& sp,
-                                             bool mean_mode) {
-  // FP32: one reciprocal r = 1/(|d|^2 (a + b|d|^2)) serves both divisions; |d|^2 = 0
-  // only on the mean mode, whose scale is precomputed.
-  const R den = sp.a + sp.b * dd;
-  const R prod = dd * den;
-  const R r = sizeof(R) == 4 ? recip<R>(prod > R(0) ? prod : R(1)) : R(0);
-  if (dd > R(0)) {
-    const cplx_t<R> div = cadd(cadd(cmul(d0, c0), cmul(d1, c1)), cmul(d2, c2));
-    const R inv_dd = sizeof(R) == 4 ? den * r : recip<R>(dd);
-    const cplx_t<R> q = mk(div.x * inv_dd, div.y * inv_dd);
-    c0 = csub(c0, cmul(cconj(d0), q));
-    c1 = csub(c1, cmul(cconj(d1), q));
-    c2 = csub(c2, cmul(cconj(d2), q));
-  }
-  // a = 0 (the steady Stokes solve): the mean mode has no solution and is dropped
-  R scale;
-  if (sizeof(R) == 4)
-    scale = prod > R(0) ? sp.inv_ntot * (dd * r) : (dd > R(0) ? R(0) : sp.mean_scale);
-  else
-    scale = den > R(0) ? sp.inv_ntot * recip<R>(den) : R(0);
-  c0 = cscale(c0, scale);
-  c1 = cscale(c1, scale);
-  c2 = cscale(c2, scale);
-  if (mean_mode && sp.k0sum != nullptr) {
-    c0 = mk((R)(sp.k0sum[0] * sp.k0mul), R(0));
-    c1 = mk((R)(sp.k0sum[1] * sp.k0mul), R(0));
-    c2 = mk((R)(sp.k0sum[2] * sp.k0mul), R(0));
-  }
-}
-
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_zsym(cplx_t<R>* __restrict__ spec, AxisPlan P, int ny, int kx,
-                                                   int kxp, SymParams<R> sp) {
-  using C = cplx_t<R>;
-  constexpr int NL = seg_lines<R>();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int N = P.n;  // nz
-  C* lines = reinterpret_cast<C*>(smem_raw);
-  const int cs = N * NL;
-  C* tw = lines + 3 * cs;
-  const int tid = threadIdx.x;
-  load_tables<R>(tw, nullptr, P, tid);
-  const int kx0 = blockIdx.x * NL;
-  const int py = blockIdx.y;
-  const size_t zstride = (size_t)ny * kxp;
-  const size_t cstride = (size_t)N * zstride;
-  C* base = spec + (size_t)py * kxp + kx0;
-  const C zero = mk(R(0), R(0));
-  for (int idx = tid; idx < 3 * cs; idx += kThreads) {
-    const int c = idx / cs, rem = idx - c * cs;
-    const int t = rem % NL, z = rem / NL;
-    lines[idx] = (kx0 + t < kx) ? base[c * cstride + z * zstride + t] : zero;
-  }
-  __syncthreads();
-  run_fft<R, false, NL>(lines, P, NL, 3, cs, tw, tid, kThreads);
-  const C dyv = sp.dy[py];
-  const R ddy = sp.ddy[py];
-  for (int idx = tid; idx < cs; idx += kThreads) {
-    const int t = idx % NL, pz = idx / NL;
-    const int k = kx0 + t;
-    if (k >= kx) continue;
-    const C d0 = sp.dx[k], d2 = sp.dz[pz];
-    const R dd = sp.ddx[k] + ddy + sp.ddz[pz];
-    C c0 = lines[idx], c1 = lines[cs + idx], c2 = lines[2 * cs + idx];
-    apply_symbol<R>(c0, c1, c2, d0, dyv, d2, dd, sp, k == 0 && py == 0 && pz == 0);
-    lines[idx] = c0;
-    lines[cs + idx] = c1;
-    lines[2 * cs + idx] = c2;
-  }
-  __syncthreads();
-  run_fft<R, true, NL>(lines, P, NL, 3, cs, tw, tid, kThreads);
-  for (int idx = tid; idx < 3 * cs; idx += kThreads) {
-    const int c = idx / cs, rem = idx - c * cs;
-    const int t = rem % NL, z = rem / NL;
-    if (kx0 + t < kx) base[c * cstride + z * zstride + t] = lines[idx];
   }
 }
 
@@ -1308,7 +1105,6 @@ template <typename R, int N, int R2> int xgrid(int nrows) {
 
 template <typename R> size_t smem_x(int n) { return (size_t)n * kXLS * sizeof(cplx_t<R>) + n * sizeof(cplx_t<R>) + n * sizeof(int); }
 template <typename R> size_t smem_y(int n) { return (size_t)n * seg_lines<R>() * sizeof(cplx_t<R>) + n * sizeof(cplx_t<R>); }
-template <typename R> size_t smem_z(int n) { return 3 * (size_t)n * seg_lines<R>() * sizeof(cplx_t<R>) + n * sizeof(cplx_t<R>); }
 
 // Sides of the fused x-y forward pass whose clusters the device can hold.
 int g_xy_sides = 0;   // bit per entry of ICM_XY_SIDES
@@ -1396,7 +1192,6 @@ void set_yz_attributes() {
 #undef ICM_ATTR
   cudaFuncSetAttribute(k_ypass<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
   cudaFuncSetAttribute(k_ypass<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-  cudaFuncSetAttribute(k_zsym<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
 
 }  // namespace
@@ -1409,18 +1204,6 @@ void set_yz_attributes() {
 #define ICM_FFT_SHARD -1
 #endif
 #define ICM_SHARD(k) (ICM_FFT_SHARD < 0 || ICM_FFT_SHARD == (k))
-
-// SMs of the current device (persistent grids), read once.
-inline int device_sms() {
-  static int nsm = 0;
-  if (nsm == 0) {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    nsm = n > 0 ? n : 1;
-  }
-  return nsm;
-}
 
 template <typename R> void fft_prepare_xf() { set_xf_attributes<R>(); }
 template <typename R> void fft_prepare_xi() { set_xi_attributes<R>(); }
@@ -1467,8 +1250,6 @@ void fft_y(const FftCtx<R>& f, bool inverse, cudaStream_t st) {
 
 template <typename R>
 void fft_z_symbol(const FftCtx<R>& f, double a, double b, const double* k0sum, double k0scale, cudaStream_t st) {
-  constexpr int NL = seg_lines<R>();
-  const int kxt = (f.kx + NL - 1) / NL;
   SymParams<R> sp;
   sp.a = (R)a;
   sp.b = (R)b;
@@ -1514,7 +1295,7 @@ void fft_z_symbol(const FftCtx<R>& f, double a, double b, const double* k0sum, d
 #undef ICM_CASE
     default: break;
   }
-  k_zsym<R><<<dim3(kxt, f.ny), kThreads, smem_z<R>(f.nz), st>>>(f.spec, f.pz, f.ny, f.kx, f.kxp, sp);
+  fft_z_any<R>(f, sp, st);
 }
 
 template <typename R>
@@ -1644,6 +1425,12 @@ void fft_x_inverse_blobs(const FftCtx<R>& f, R* dst, int mode, const RowBlobs& r
 template <typename R>
 void spectral_solve(const FftCtx<R>& f, const R* src, R* dst, R* dst2, int mode, double a, double b,
                     const double* k0sum, double k0scale, cudaStream_t st) {
+  if (plane_has_passes(8 * sizeof(R), f.nx, f.ny, f.nz)) {
+    plane_forward<R>(f, src, nullptr, nullptr, 1, st);
+    fft_z_symbol<R>(f, a, b, k0sum, k0scale, st);
+    plane_inverse<R>(f, dst, dst2, mode, nullptr, nullptr, 1, st);
+    return;
+  }
   fft_x_forward<R>(f, src, st);
   fft_y<R>(f, false, st);
   fft_z_symbol<R>(f, a, b, k0sum, k0scale, st);
@@ -1770,6 +1557,12 @@ void fft_x_inverse_group(const FftCtx<R>& f, const RepFft* reps, int G, int mode
 template <typename R>
 void spectral_solve_group(const FftCtx<R>& f, const RepFft* reps, int G, int mode, cudaStream_t st,
                           const void* gzmap, bool blobs) {
+  if (!blobs && plane_has_passes(8 * sizeof(R), f.nx, f.ny, f.nz)) {
+    plane_forward<R>(f, nullptr, nullptr, reps, G, st);
+    fft_yz_group<R>(f, reps, G, 1, st, gzmap);
+    plane_inverse<R>(f, nullptr, nullptr, mode, nullptr, reps, G, st);
+    return;
+  }
   fft_x_forward_group<R>(f, reps, G, st, blobs);
   fft_yz_group<R>(f, reps, G, 0, st, nullptr);
   fft_yz_group<R>(f, reps, G, 1, st, gzmap);
@@ -1888,6 +1681,8 @@ void fft_prepare() {
   fft_prepare_xf<double>();
   fft_prepare_yz<double>();
   fft_prepare_xi<double>();
+  plane_prepare<float>();
+  plane_prepare<double>();
 }
 
 template void spectral_solve<float>(const FftCtx<float>&, const float*, float*, float*, int, double, double,

@@ -611,7 +611,14 @@ __device__ __forceinline__ int member_of_unit(const RhsMember<R>* __restrict__ m
   return a;
 }
 template <typename R>
-__global__ void __launch_bounds__(kFlatThreads / 2) k_noise_batch(const RhsMember<R>* __restrict__ mem, int nm) {
+__global__ void __launch_bounds__(kFlatThreads / 2) k_noise_batch(const RhsMember<R>* __restrict__ mem, int nm,
+                                                                 long long total, const BlobMember* __restrict__ all,
+                                                                 int n_all) {
+  if (blockIdx.x >= total) {   // the blocks past the normals: the members' scalars
+    const int e = (int)(blockIdx.x - total) * (kFlatThreads / 2) + threadIdx.x;
+    if (e < 3 * n_all) scalars_before(all[e / 3].s.scal, all[e / 3].p.dt, e % 3);
+    return;
+  }
   const RhsMember<R>& m = mem[member_of_unit(mem, nm, blockIdx.x)];
   noise_pair<R>(m.g, (uint32_t)(blockIdx.x - m.w0) * (kFlatThreads / 2) + threadIdx.x, (uint32_t)(*m.step_dev),
                 m.normals);
@@ -699,10 +706,7 @@ __global__ void k_convert(const A* __restrict__ src, B* __restrict__ dst, long l
 
 __global__ void k_scal_before(double* scal, double dt) {
   const int a = threadIdx.x;
-  if (a < 3) {
-    scal[SC_K0 + a] = scal[SC_PBAR + a] + dt * scal[SC_SUMF + a];
-    scal[SC_SUMSRC + a] = 0.0;
-  }
+  if (a < 3) scalars_before(scal, dt, a);
 }
 
 __global__ void k_scal_after(double* scal, int inertial, long long* step_dev, int* hist_dev) {
@@ -796,7 +800,6 @@ void batch_rhs(const RhsMember<R>* members, int nm, long long total, bool noise,
   if (nm <= 0 || total <= 0) return;
   if constexpr (sizeof(R) == 8) {
     if (noise) {
-      k_noise_batch<R><<<(unsigned)total, kFlatThreads / 2, 0, st>>>(members, nm);
       k_rhs_flat_batch<R, true><<<(unsigned)total, kFlatThreads, 0, st>>>(members, nm);
     } else {
       k_rhs_flat_batch<R, false><<<(unsigned)total, kFlatThreads, 0, st>>>(members, nm);
@@ -817,6 +820,18 @@ void batch_rhs(const RhsMember<R>* members, int nm, long long total, bool noise,
       k_rhs_batch<R, false><<<grid, block, rhs_smem<R>(), st>>>(members, nm, total);
   }
 }
+
+template <typename R>
+void batch_noise(const RhsMember<R>* members, int nm, long long total, const BlobMember* all, int n_all,
+                 cudaStream_t st) {
+  if (nm <= 0 || total <= 0) {
+    batch_scalars_before(all, n_all, st);
+    return;
+  }
+  const int extra = (3 * n_all + kFlatThreads / 2 - 1) / (kFlatThreads / 2);
+  k_noise_batch<R><<<(unsigned)(total + extra), kFlatThreads / 2, 0, st>>>(members, nm, total, all, n_all);
+}
+template void batch_noise<double>(const RhsMember<double>*, int, long long, const BlobMember*, int, cudaStream_t);
 
 template <typename R>
 void stress_normals(const GridParams& g, long long step, R* out, cudaStream_t st) {

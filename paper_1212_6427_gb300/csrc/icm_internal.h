@@ -14,6 +14,18 @@ namespace icm {
 // Record the message returned by icm_last_error for this thread; returns st.
 int record_error(int st, const char* msg);
 
+// SMs of the current device (persistent grids), read once.
+inline int device_sms() {
+  static int nsm = 0;
+  if (nsm == 0) {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    nsm = n > 0 ? n : 1;
+  }
+  return nsm;
+}
+
 constexpr int kMaxSide = 512;
 constexpr int kMaxStages = 12;
 
@@ -253,7 +265,15 @@ enum ScalarSlot : int {
   SC_COUNT = 20
 };
 
-template <typename R> void blob_predict(const BlobParams& p, BlobState s, const R* v, cudaStream_t st);
+// Where a predictor leaves the stencil records at q^{n+1/2} for the plane passes (null pointers:
+// nowhere).
+struct PlaneRecords {
+  void* geo;
+  int* zfirst;
+  int zstride;
+};
+template <typename R>
+void blob_predict(const BlobParams& p, BlobState s, const R* v, cudaStream_t st, PlaneRecords rec = PlaneRecords{});
 template <typename R> void blob_spread(const BlobParams& p, long long nb, const double* q, const double* vec,
                                        R* field, cudaStream_t st);
 template <typename R> void blob_momentum_change(const BlobParams& p, BlobState s, const R* vt, cudaStream_t st);
@@ -321,6 +341,54 @@ void fft_xy_forward(const FftCtx<R>& f, const R* src, const RowBlobs* rb, cudaSt
 template <typename R>
 void fft_x_inverse_blobs(const FftCtx<R>& f, R* dst, int mode, const RowBlobs& rb, cudaStream_t st);
 bool fft_has_blob_passes(int nx);
+
+// ---------------------------------------------------------------------------
+// Whole z planes in shared memory: the x and y transforms in one pass (icm_plane.cu)
+// ---------------------------------------------------------------------------
+// What a plane's blobs spread: given vectors, or the sources of steps 5 and 6 formed on the fly.
+enum PlaneSource : int { PLANE_VEC = 0, PLANE_CDP = 1, PLANE_SRC = 2 };
+struct PlaneBlobs {
+  BlobParams p;
+  BlobState s;
+  const void* geo;      // stencil records
+  const int* zfirst;    // first z node of every blob: component z, then (at zstride) x and y
+  int zstride;
+  int source;           // PlaneSource of a forward pass
+  const double* vec;    // PLANE_VEC: the vectors
+  const double* jvt;    // partial sums of J v~ (PLANE_CDP, PLANE_SRC)
+  const double* jdvt;   // and of J dv~ (PLANE_SRC, which also adds up the source's grid sum)
+  // An inverse pass gathers J x, and J L x (without 1/h^2), plane by plane: the part of blob b
+  // and component a that plane c of its support holds goes to part[c (3 nb) + 3 b + a], one
+  // writer each, and whoever needs the value adds the planes in order (plane_sum).
+  double* part;         // kernel planes
+  double* part_lap;     // kernel + 2 planes
+};
+constexpr int kPlaneParts = 4 + 4 + 4 + 6;   // J v~, J dv~, J dv, J L dv: doubles per blob component
+// The value of element i = 3 b + a from `planes` partial sums.
+__device__ __forceinline__ double plane_sum(const double* __restrict__ part, long long n3, long long i, int planes) {
+  double x = part[i];
+  for (int c = 1; c < planes; ++c) x += part[c * n3 + i];
+  return x;
+}
+// Whether a grid's planes fit in shared memory (and are worth it).
+bool plane_has_passes(int precision, int nx, int ny, int nz);
+template <typename R> void plane_prepare();
+// The spectrum fft_x_forward + fft_y leave, with the blobs' spread (pb, or null); src may be null
+// with blobs.  reps: the G replicas of a group solve (no blobs), or null.
+template <typename R>
+void plane_forward(const FftCtx<R>& f, const R* src, const PlaneBlobs* pb, const RepFft* reps, int G, cudaStream_t st);
+// mode: OUT_STORE, OUT_ADD_AND_STORE2 without blobs; OUT_STORE, OUT_NONE, OUT_ADD (which also
+// gathers the Laplacian) with blobs.
+template <typename R>
+void plane_inverse(const FftCtx<R>& f, R* dst, R* dst2, int mode, const PlaneBlobs* pb, const RepFft* reps, int G,
+                   cudaStream_t st);
+template <typename R> struct SymParams;
+// z transform, symbol and inverse of a side without two-stage register kernels.
+template <typename R> void fft_z_any(const FftCtx<R>& f, const SymParams<R>& sp, cudaStream_t st);
+// Step 9 and the blob side of step 8 from the gathered J v~, J dv~, J dv, J L dv (partial sums of 4, 4,
+// 4 and 6 planes' room), with the end-of-step bookkeeping.
+void blob_finish_plane(const BlobParams& p, BlobState s, const double* parts, bool inertial, long long* step_dev,
+                       int* hist_dev, cudaStream_t st);
 
 // Coupling matrices J(qi) (a - b L)^-1 P S(qj) (row-major 3 x 3 each) of npair pairs of
 // positions as sums over wave vectors (icm_couple.cu).  q_dev: the npair positions qi, then
@@ -392,6 +460,10 @@ template <typename R> void batch_finish(const BlobMember* m, const int* member_o
 // sums of the members' work sizes in 16-byte words, total16 their sum.
 void batch_zero_work(const BlobMember* m, const long long* prefix16, int nm, long long total16, cudaStream_t st);
 void batch_scalars_before(const BlobMember* m, int nm, cudaStream_t st);
+__device__ __forceinline__ void scalars_before(double* scal, double dt, int a) {
+  scal[SC_K0 + a] = scal[SC_PBAR + a] + dt * scal[SC_SUMF + a];
+  scal[SC_SUMSRC + a] = 0.0;
+}
 void batch_scalars_after(const BlobMember* m, int nm, cudaStream_t st);
 
 // The right-hand side of every member (persistent blocks over all members' tile-planes).
@@ -410,6 +482,10 @@ struct RhsMember {
 // members[0 .. nm) in order of w0; total = the last member's w0 + its units.
 template <typename R>
 void batch_rhs(const RhsMember<R>* members, int nm, long long total, bool noise, cudaStream_t st);
+// The stress normals of the members with noise where they are stored (FP64), and the scalars before the
+// step of all members (blobs), in one launch.
+template <typename R>
+void batch_noise(const RhsMember<R>* members, int nm, long long total, const BlobMember* all, int n_all, cudaStream_t st);
 // Work units of a grid in the batched right-hand side.
 long long rhs_batch_units(int precision, int nx, int ny, int nz);
 

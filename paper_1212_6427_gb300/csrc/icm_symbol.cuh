@@ -1,0 +1,72 @@
+// The Helmholtz/projection symbol of the z passes (arXiv:1212.6427, Sec. III.D), applied to
+// the three components of one wave vector in registers.
+#pragma once
+
+#include "icm_internal.h"
+
+namespace icm {
+
+template <typename R>
+struct SymParams {
+  R a, b, inv_ntot;
+  R mean_scale;   // the symbol's scale on the mean mode: 1/(a ncell), 0 when a = 0
+  const cplx_t<R>* dx; const R* ddx;
+  const cplx_t<R>* dy; const R* ddy;
+  const cplx_t<R>* dz; const R* ddz;
+  const double* k0sum;
+  double k0mul;   // k0scale / ncell
+};
+
+namespace {
+// P^ w / (a + b|d|^2) / ncell on one wave vector: (P^ w)_a = w_a - conj(d_a)(d . w)/|d|^2,
+// identity on the mean mode, whose value is replaced by the FP64 bookkeeping if given
+// (and which is zero when a = 0).
+// One reciprocal r = 1/(|d|^2 (a + b|d|^2)) serves both divisions; |d|^2 = 0 only on the mean mode,
+// whose scale is precomputed.
+// 1/x, x normal and positive: the hardware reciprocal in FP32 (within one ulp); in FP64 the
+// approximate reciprocal instruction and one step of third order, y (1 + e + e^2) with
+// e = 1 - x y, three FP64 operations where a division takes about ten (FP64 operations bound
+// the FP64 z pass).
+template <typename R> __device__ __forceinline__ R recip(R x);
+template <> __device__ __forceinline__ float recip<float>(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));   // within one ulp; x is never denormal here
+  return r;
+}
+template <> __device__ __forceinline__ double recip<double>(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+template <typename R>
+__device__ __forceinline__ void apply_symbol(cplx_t<R>& c0, cplx_t<R>& c1, cplx_t<R>& c2, cplx_t<R> d0,
+                                             cplx_t<R> d1, cplx_t<R> d2, R dd, const SymParams<R>& sp,
+                                             bool mean_mode) {
+  const R den = sp.a + sp.b * dd;
+  const R prod = dd * den;
+  const R r = recip<R>(prod > R(0) ? prod : R(1));
+  if (dd > R(0)) {
+    const cplx_t<R> div = cadd(cadd(cmul(d0, c0), cmul(d1, c1)), cmul(d2, c2));
+    const R inv_dd = den * r;
+    const cplx_t<R> q = mk(div.x * inv_dd, div.y * inv_dd);
+    c0 = csub(c0, cmul(cconj(d0), q));
+    c1 = csub(c1, cmul(cconj(d1), q));
+    c2 = csub(c2, cmul(cconj(d2), q));
+  }
+  // a = 0 (the steady Stokes solve): the mean mode has no solution and is dropped
+  const R scale = prod > R(0) ? sp.inv_ntot * (dd * r) : (dd > R(0) ? R(0) : sp.mean_scale);
+  c0 = cscale(c0, scale);
+  c1 = cscale(c1, scale);
+  c2 = cscale(c2, scale);
+  if (mean_mode && sp.k0sum != nullptr) {
+    c0 = mk((R)(sp.k0sum[0] * sp.k0mul), R(0));
+    c1 = mk((R)(sp.k0sum[1] * sp.k0mul), R(0));
+    c2 = mk((R)(sp.k0sum[2] * sp.k0mul), R(0));
+  }
+}
+
+
+}  // namespace
+}  // namespace icm

@@ -21,7 +21,8 @@ def icm():
 
 
 CASES = [((6, 6, 9), 64), ((6, 6, 9), 32), ((27, 8, 27), 64), ((27, 8, 27), 32), ((8, 162, 6), 64), ((8, 162, 6), 32),
-         ((128, 128, 64), 32), ((128, 128, 72), 32)]
+         ((128, 128, 64), 32), ((128, 128, 72), 32),
+         ((108, 144, 81), 32)]
 
 
 @pytest.mark.parametrize("grid,precision", CASES)
