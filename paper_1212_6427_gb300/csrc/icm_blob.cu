@@ -850,49 +850,113 @@ __global__ void k_wca_fill(BlobState s, WcaParams w) {
   if (pos < s.nb) w.list[pos] = (int)b;
 }
 
+// Count, scan and fill in one block, the counts in shared memory: for lists short enough that three
+// launches cost more than one SM's work (1000 blobs, 2744 cells: 12 us with gaps against 6).
+constexpr int kWcaBlockCells = 8192, kWcaBlockBlobs = 8192;
+__global__ void __launch_bounds__(1024) k_wca_bin(BlobState s, WcaParams w) {
+  __shared__ int cnt[kWcaBlockCells];
+  __shared__ int warp_tot[32];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nb = (int)s.nb;
+  for (int i = t; i < w.ncells; i += 1024) cnt[i] = 0;
+  __syncthreads();
+  int cell[kWcaBlockBlobs / 1024];
+#pragma unroll
+  for (int k = 0; k < kWcaBlockBlobs / 1024; ++k) {
+    const int b = t + 1024 * k;
+    if (b >= nb) continue;
+    int c[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) c[a] = wca_cell_axis(s.qh[3 * b + a], w.cell_inv[a], w.nc[a]);
+    cell[k] = c[0] + w.nc[0] * (c[1] + w.nc[1] * c[2]);
+    atomicAdd(&cnt[cell[k]], 1);
+  }
+  __syncthreads();
+  const int per = (w.ncells + 1023) / 1024, lo = min(t * per, w.ncells), hi = min(lo + per, w.ncells);
+  int sum = 0;
+  for (int i = lo; i < hi; ++i) sum += cnt[i];
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) warp_tot[wid] = incl;
+  __syncthreads();
+  if (wid == 0) {
+    int x = warp_tot[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += v;
+    }
+    warp_tot[lane] = x;
+  }
+  __syncthreads();
+  int run = incl - sum + (wid > 0 ? warp_tot[wid - 1] : 0);
+  for (int i = lo; i < hi; ++i) {
+    const int c = cnt[i];
+    cnt[i] = run;       // the cell's cursor
+    w.start[i] = run;
+    run += c;
+  }
+  if (t == 1023) w.start[w.ncells] = nb;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kWcaBlockBlobs / 1024; ++k) {
+    const int b = t + 1024 * k;
+    if (b < nb) w.list[atomicAdd(&cnt[cell[k]], 1)] = b;
+  }
+}
+
 // F_i = sum_j 24 eps (2 s^12/r^14 - s^6/r^8) d_ij over the pairs within the cut-off,
-// d_ij = q_i - q_j to the nearest image (FP64).
-__global__ void __launch_bounds__(256) k_wca_force(BlobParams p, BlobState s, WcaParams w, int with_trap) {
-  __shared__ double red[3][256];
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+// d_ij = q_i - q_j to the nearest image (FP64).  One warp per blob, one lane per neighbour cell: the
+// dependent loads (cell, list, position) of the 27 cells and their FP64 arithmetic overlap, where one
+// thread per blob took them in turn on a few SMs (1000 blobs on 32^3: 41 us).
+__global__ void __launch_bounds__(32 * kWarps) k_wca_force(BlobParams p, BlobState s, WcaParams w, int with_trap) {
+  __shared__ double red[kWarps][3];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long long i = (long long)blockIdx.x * kWarps + wid;
   double f[3] = {0.0, 0.0, 0.0};
   if (i < s.nb) {
     const double qi[3] = {s.qh[3 * i], s.qh[3 * i + 1], s.qh[3 * i + 2]};
-    int c[3];
-    for (int a = 0; a < 3; ++a) c[a] = wca_cell_axis(qi[a], w.cell_inv[a], w.nc[a]);
+    int c[3], n[3];
+    for (int a = 0; a < 3; ++a) {
+      c[a] = wca_cell_axis(qi[a], w.cell_inv[a], w.nc[a]);
+      n[a] = w.hi[a] - w.lo[a] + 1;
+    }
     const double s2 = w.sigma * w.sigma;
-    for (int dz = w.lo[2]; dz <= w.hi[2]; ++dz)
-      for (int dy = w.lo[1]; dy <= w.hi[1]; ++dy)
-        for (int dx = w.lo[0]; dx <= w.hi[0]; ++dx) {
-          const int cx = (c[0] + dx + w.nc[0]) % w.nc[0], cy = (c[1] + dy + w.nc[1]) % w.nc[1];
-          const int cz = (c[2] + dz + w.nc[2]) % w.nc[2];
-          const int cell = cx + w.nc[0] * (cy + w.nc[1] * cz);
-          const int e = w.start[cell + 1];
-          for (int k = w.start[cell]; k < e; ++k) {
-            const int j = w.list[k];
-            if (j == i) continue;
-            double d[3], r2 = 0.0;
-            for (int a = 0; a < 3; ++a) {
-              const double x = qi[a] - s.qh[3 * j + a];
-              d[a] = fma(-p.box[a], rint(x * p.inv_box[a]), x);
-              r2 = fma(d[a], d[a], r2);
-            }
-            if (r2 >= w.rc2) continue;
-            const double s6 = (s2 / r2) * (s2 / r2) * (s2 / r2);
-            const double mag = 24.0 * w.eps * (2.0 * s6 * s6 - s6) / r2;
-            for (int a = 0; a < 3; ++a) f[a] = fma(mag, d[a], f[a]);
-          }
+    if (lane < n[0] * n[1] * n[2]) {
+      const int cx = (c[0] + w.lo[0] + lane % n[0] + w.nc[0]) % w.nc[0];
+      const int cy = (c[1] + w.lo[1] + lane / n[0] % n[1] + w.nc[1]) % w.nc[1];
+      const int cz = (c[2] + w.lo[2] + lane / (n[0] * n[1]) + w.nc[2]) % w.nc[2];
+      const int cell = cx + w.nc[0] * (cy + w.nc[1] * cz);
+      const int e = w.start[cell + 1];
+      for (int k = w.start[cell]; k < e; ++k) {
+        const int j = w.list[k];
+        if (j == i) continue;
+        double d[3], r2 = 0.0;
+        for (int a = 0; a < 3; ++a) {
+          const double x = qi[a] - s.qh[3 * j + a];
+          d[a] = fma(-p.box[a], rint(x * p.inv_box[a]), x);
+          r2 = fma(d[a], d[a], r2);
         }
-    for (int a = 0; a < 3; ++a) s.fe[3 * i + a] = (with_trap ? s.fe[3 * i + a] : s.f[3 * i + a]) + f[a];
+        if (r2 >= w.rc2) continue;
+        const double i2 = 1.0 / r2, t = s2 * i2, s6 = t * t * t;
+        const double mag = 24.0 * w.eps * fma(2.0 * s6, s6, -s6) * i2;
+        for (int a = 0; a < 3; ++a) f[a] = fma(mag, d[a], f[a]);
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) f[a] = warp_sum(f[a]);
+    if (lane < 3) s.fe[3 * i + lane] = (with_trap ? s.fe[3 * i + lane] : s.f[3 * i + lane]) + pick3(f, lane);
   }
-  for (int a = 0; a < 3; ++a) red[a][threadIdx.x] = f[a];
+  if (lane < 3) red[wid][lane] = pick3(f, lane);
   __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if (threadIdx.x < h)
-      for (int a = 0; a < 3; ++a) red[a][threadIdx.x] += red[a][threadIdx.x + h];
-    __syncthreads();
+  if (threadIdx.x < 3) {
+    double t = 0.0;
+    for (int k = 0; k < kWarps; ++k) t += red[k][threadIdx.x];
+    atomicAdd(&s.scal[SC_K0 + threadIdx.x], p.dt * t);
   }
-  if (threadIdx.x < 3) atomicAdd(&s.scal[SC_K0 + threadIdx.x], p.dt * red[threadIdx.x][0]);
 }
 
 }  // namespace
@@ -909,20 +973,24 @@ template void build_row_bins<double>(const BlobParams&, long long, const double*
 
 void blob_wca_forces(const BlobParams& p, BlobState s, const WcaParams& w, bool with_trap, cudaStream_t st) {
   if (s.nb <= 0) return;
-  k_wca_count<<<eblocks(s.nb), 256, 0, st>>>(s, w);
-  RowBins cells;
-  cells.count = w.count;
-  cells.start = w.start;
-  cells.cursor = w.cursor;
-  cells.list = w.list;
-  cells.geo = nullptr;
-  cells.acc = nullptr;
-  cells.nacc = 0;
-  cells.nblocks = w.ncells;
-  cells.capacity = s.nb;
-  k_bin_scan<<<1, 1024, 0, st>>>(cells);
-  k_wca_fill<<<eblocks(s.nb), 256, 0, st>>>(s, w);
-  k_wca_force<<<eblocks(s.nb), 256, 0, st>>>(p, s, w, with_trap ? 1 : 0);
+  if (s.nb <= kWcaBlockBlobs && w.ncells <= kWcaBlockCells) {
+    k_wca_bin<<<1, 1024, 0, st>>>(s, w);
+  } else {
+    k_wca_count<<<eblocks(s.nb), 256, 0, st>>>(s, w);
+    RowBins cells;
+    cells.count = w.count;
+    cells.start = w.start;
+    cells.cursor = w.cursor;
+    cells.list = w.list;
+    cells.geo = nullptr;
+    cells.acc = nullptr;
+    cells.nacc = 0;
+    cells.nblocks = w.ncells;
+    cells.capacity = s.nb;
+    k_bin_scan<<<1, 1024, 0, st>>>(cells);
+    k_wca_fill<<<eblocks(s.nb), 256, 0, st>>>(s, w);
+  }
+  k_wca_force<<<nblocks(s.nb), 32 * kWarps, 0, st>>>(p, s, w, with_trap ? 1 : 0);
 }
 
 void blob_dp_from(const BlobParams& p, BlobState s, const double* jvt, cudaStream_t st) {
