@@ -262,7 +262,7 @@ template <typename R, int N, int R2> constexpr int x_plain_lines() {
 // two-output mode, which would spill) all loads are in flight at once and one record
 // per thread is staged.
 template <typename R, int N, int MODE> constexpr bool xi2_lean() {
-  return sizeof(R) == 4 && N <= 256 && MODE != OUT_ADD_AND_STORE2;
+  return sizeof(R) == 4 && MODE != OUT_ADD_AND_STORE2;
 }
 template <typename R, int N, int MODE> constexpr int xi2_stage() { return xi2_lean<R, N, MODE>() ? 128 : kThreads; }
 
@@ -584,12 +584,20 @@ constexpr int y_planes() {
   return sizeof(R) != 4 || N > 64 ? 1 : (R2 * seg_lines<R>() * 4 <= kThreads ? 4 : 2);
 }
 
+// Threads of a y-pass block.  FP64 takes one thread per first-stage item: with 256 only 64 of them had one
+// at 128, and what two resident blocks kept active did not fill the FP64 pipe (Y64NOTE).
+template <typename R, int N, int R2>
+constexpr int y_threads() {
+  return sizeof(R) == 4 ? kThreads : (R2 * seg_lines<R>() < 64 ? 64 : (R2 * seg_lines<R>() > kThreads ? kThreads : R2 * seg_lines<R>()));
+}
+
 template <typename R, int N, int R1, int R2, bool INV>
-__global__ void __launch_bounds__(kThreads) k_ypass2(cplx_t<R>* __restrict__ spec, const cplx_t<R>* __restrict__ gtw,
+__global__ void __launch_bounds__(y_threads<R, N, R2>()) k_ypass2(cplx_t<R>* __restrict__ spec, const cplx_t<R>* __restrict__ gtw,
                                                      int nz, int kx, int kxp, const RepFft* __restrict__ reps) {
   using C = cplx_t<R>;
   constexpr int NL = seg_lines<R>();
   constexpr int ZB = y_planes<R, N, R2>();
+  constexpr int NT = y_threads<R, N, R2>();
   if (reps != nullptr) spec = reinterpret_cast<C*>(reps[blockIdx.z / 3].spec);   // group solve: 3 components per replica
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);   // [ZB][N][NL]
@@ -616,9 +624,9 @@ __global__ void __launch_bounds__(kThreads) k_ypass2(cplx_t<R>* __restrict__ spe
     };
     C a[R1];
     if (tid < ZB * R2 * NL) load_item(tid, a);
-    load_stage_twiddles<R, R1, R2>(tw, gtw, tid, kThreads);
+    load_stage_twiddles<R, R1, R2>(tw, gtw, tid, NT);
     __syncthreads();
-    for (int it = tid; it < ZB * R2 * NL; it += kThreads) {
+    for (int it = tid; it < ZB * R2 * NL; it += NT) {
       const int line = it % NL, rest = it / NL, n1 = rest % R2, zb = rest / R2;
       if (it != tid) load_item(it, a);
       stage_a_fwd<R, R1, R2>(a, tw + n1);
@@ -626,7 +634,7 @@ __global__ void __launch_bounds__(kThreads) k_ypass2(cplx_t<R>* __restrict__ spe
       for (int k2 = 0; k2 < R1; ++k2) buf[(zb * N + n1 + R2 * k2) * NL + line] = a[k2];
     }
     __syncthreads();
-    for (int it = tid; it < ZB * R1 * NL; it += kThreads) {
+    for (int it = tid; it < ZB * R1 * NL; it += NT) {
       const int line = it % NL, rest = it / NL, blk = rest % R1, zb = rest / R1;
       if (kx0 + line >= kx || z0 + zb >= nz) continue;
       C* base = base0 + (size_t)zb * N * kxp;
@@ -640,7 +648,7 @@ __global__ void __launch_bounds__(kThreads) k_ypass2(cplx_t<R>* __restrict__ spe
   } else {
     // the second stage comes first and needs no twiddles: its loads go out first, the
     // table is staged after it, before the barrier the first stage waits at anyway
-    for (int it = tid; it < ZB * R1 * NL; it += kThreads) {
+    for (int it = tid; it < ZB * R1 * NL; it += NT) {
       const int line = it % NL, rest = it / NL, blk = rest % R1, zb = rest / R1;
       const bool ok = kx0 + line < kx && z0 + zb < nz;
       const C* base = base0 + (size_t)zb * N * kxp;
@@ -651,9 +659,9 @@ __global__ void __launch_bounds__(kThreads) k_ypass2(cplx_t<R>* __restrict__ spe
 #pragma unroll
       for (int n = 0; n < R2; ++n) buf[(zb * N + R2 * blk + n) * NL + line] = b[n];
     }
-    load_stage_twiddles<R, R1, R2>(tw, gtw, tid, kThreads);
+    load_stage_twiddles<R, R1, R2>(tw, gtw, tid, NT);
     __syncthreads();
-    for (int it = tid; it < ZB * R2 * NL; it += kThreads) {
+    for (int it = tid; it < ZB * R2 * NL; it += NT) {
       const int line = it % NL, rest = it / NL, n1 = rest % R2, zb = rest / R2;
       if (kx0 + line >= kx || z0 + zb >= nz) continue;
       C* base = base0 + (size_t)zb * N * kxp;
@@ -895,7 +903,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_xyf(const float* __restrict__ s
 // (without 1/h^2) to rb.acc_lap.  x stays in shared memory for the gathers.
 // GRP: a group solve whose replicas gather into their own accumulators (reps[i].rb).
 template <typename R, int N, int R1, int R2, int MODE, int GATHER, bool GRP = false>
-__global__ void __launch_bounds__(kThreads, xi2_lean<R, N, MODE>() ? 4 : 1) k_xinv2(const cplx_t<R>* __restrict__ spec, R* __restrict__ dst,
+__global__ void __launch_bounds__(kThreads, xi2_lean<R, N, MODE>() ? (N <= 256 ? 4 : 2) : 1) k_xinv2(const cplx_t<R>* __restrict__ spec, R* __restrict__ dst,
                                                     R* __restrict__ dst2, const cplx_t<R>* __restrict__ gtw,
                                                     int nrows, long long ncell, int kxp, RowBlobs rb0,
                                                     const RepFft* __restrict__ reps) {
@@ -944,7 +952,7 @@ __global__ void __launch_bounds__(kThreads, xi2_lean<R, N, MODE>() ? 4 : 1) k_xi
     for (int o = 0; o < OUTS; ++o) load_old(o);
   }
   constexpr int LOADS = (L * N + kThreads - 1) / kThreads;   // compile-time: loads in flight together
-  constexpr int BATCH = LEAN ? (LOADS + 1) / 2 : LOADS;
+  constexpr int BATCH = LEAN ? (N <= 256 ? (LOADS + 1) / 2 : 8) : LOADS;
   int g0 = 0, ge = 0;
 #pragma unroll
   for (int j0 = 0; j0 < LOADS; j0 += BATCH) {
@@ -1234,9 +1242,9 @@ void fft_y(const FftCtx<R>& f, bool inverse, cudaStream_t st) {
 #define ICM_CASE(N, R1, R2)                                                                                   \
   case N:                                                                                                     \
     if (inverse)                                                                                              \
-      k_ypass2<R, N, R1, R2, true><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3), kThreads, smem_y2<R, N, R2>(), st>>>(f.spec, tw, f.nz, f.kx, f.kxp, nullptr);  \
+      k_ypass2<R, N, R1, R2, true><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(f.spec, tw, f.nz, f.kx, f.kxp, nullptr);  \
     else                                                                                                      \
-      k_ypass2<R, N, R1, R2, false><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3), kThreads, smem_y2<R, N, R2>(), st>>>(f.spec, tw, f.nz, f.kx, f.kxp, nullptr); \
+      k_ypass2<R, N, R1, R2, false><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(f.spec, tw, f.nz, f.kx, f.kxp, nullptr); \
     return;
     ICM_FFT_SIDES(ICM_CASE)
 #undef ICM_CASE
@@ -1516,9 +1524,9 @@ void fft_yz_group(const FftCtx<R>& f, const RepFft* reps, int G, int which, cuda
 #define ICM_CASE(N, R1, R2)                                                                                             \
   case N:                                                                                                               \
     if (which == 2)                                                                                                     \
-      k_ypass2<R, N, R1, R2, true><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3 * G), kThreads, smem_y2<R, N, R2>(), st>>>(nullptr, twy, f.nz, f.kx, f.kxp, reps); \
+      k_ypass2<R, N, R1, R2, true><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3 * G), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(nullptr, twy, f.nz, f.kx, f.kxp, reps); \
     else                                                                                                                \
-      k_ypass2<R, N, R1, R2, false><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3 * G), kThreads, smem_y2<R, N, R2>(), st>>>(nullptr, twy, f.nz, f.kx, f.kxp, reps); \
+      k_ypass2<R, N, R1, R2, false><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3 * G), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(nullptr, twy, f.nz, f.kx, f.kxp, reps); \
     return;
       ICM_FFT_SIDES(ICM_CASE)
 #undef ICM_CASE
