@@ -61,13 +61,8 @@ __device__ __forceinline__ void fft_stage(cplx_t<R>* s, int N, int M, int LS, in
     for (int r = 0; r < RAD; ++r) a[r] = p[r * str];
     if (INV) {
 #pragma unroll
-      for (int r = 0; r < RAD; ++r) {
-        a[r] = cconj(a[r]);
-        if (r > 0) a[r] = cmul(a[r], tw[n1 * r * tws]);
-      }
-      SDft<R, RAD>::run(a);
-#pragma unroll
-      for (int r = 0; r < RAD; ++r) a[r] = cconj(a[r]);
+      for (int r = 1; r < RAD; ++r) a[r] = cmul(a[r], cconj(tw[n1 * r * tws]));
+      sdft_inv<R, RAD>(a);
     } else {
       SDft<R, RAD>::run(a);
 #pragma unroll
@@ -146,8 +141,8 @@ __global__ void __launch_bounds__(kThreads) k_xfwd(const R* __restrict__ src, cp
     const int l = idx / kx, k = idx - l * kx;
     const C zk = lines[pof[k] * kXLS + l];
     const C zm = lines[pof[k == 0 ? 0 : N - k] * kXLS + l];
-    const C x1 = mk((zk.x + zm.x) * R(0.5), (zk.y - zm.y) * R(0.5));
-    const C x2 = cmul_mi(mk((zk.x - zm.x) * R(0.5), (zk.y + zm.y) * R(0.5)));
+    const C x1 = mk(zk.x + zm.x, zk.y - zm.y);   // twice the spectrum (SymParams::inv_ntot)
+    const C x2 = mk(zk.y + zm.y, zm.x - zk.x);
     const long long r1 = row0 + 2 * l;
     if (r1 < nrows) out[r1 * kxp + k] = x1;
     if (r1 + 1 < nrows) out[(r1 + 1) * kxp + k] = x2;
@@ -585,10 +580,12 @@ constexpr int y_planes() {
 }
 
 // Threads of a y-pass block.  FP64 takes one thread per first-stage item: with 256 only 64 of them had one
-// at 128, and what two resident blocks kept active did not fill the FP64 pipe (Y64NOTE).
+// at 128, and what two resident blocks kept active did not fill the FP64 pipe (forward pass on 128^3:
+// 169 us with 256 threads, 153 with 64).
 template <typename R, int N, int R2>
 constexpr int y_threads() {
-  return sizeof(R) == 4 ? kThreads : (R2 * seg_lines<R>() < 64 ? 64 : (R2 * seg_lines<R>() > kThreads ? kThreads : R2 * seg_lines<R>()));
+  constexpr int items = R2 * seg_lines<R>();
+  return sizeof(R) == 4 || items > kThreads ? kThreads : items < 64 ? 64 : items;
 }
 
 template <typename R, int N, int R1, int R2, bool INV>
@@ -755,7 +752,8 @@ __device__ __forceinline__ void x_forward_rows(cplx_t<R>* __restrict__ buf, cons
   __syncthreads();
 }
 
-// The two half spectra of line l at wavenumber k from the transformed lines in buf.
+// Twice the two half spectra of line l at wavenumber k from the transformed lines in buf (the symbol
+// takes the factor back).
 template <typename R, int N, int R1, int R2>
 __device__ __forceinline__ void split_half_spectra(const cplx_t<R>* __restrict__ buf, int l, int k, cplx_t<R>& x1,
                                                    cplx_t<R>& x2) {
@@ -763,8 +761,8 @@ __device__ __forceinline__ void split_half_spectra(const cplx_t<R>* __restrict__
   const int km = k == 0 ? 0 : N - k;
   const C zk = buf[xaddr(l, R2 * (k % R1) + k / R1, N)];
   const C zm = buf[xaddr(l, R2 * (km % R1) + km / R1, N)];
-  x1 = mk((zk.x + zm.x) * R(0.5), (zk.y - zm.y) * R(0.5));
-  x2 = cmul_mi(mk((zk.x - zm.x) * R(0.5), (zk.y + zm.y) * R(0.5)));
+  x1 = mk(zk.x + zm.x, zk.y - zm.y);
+  x2 = mk(zk.y + zm.y, zm.x - zk.x);
 }
 
 // x forward pass: x_forward_rows, then the half spectra of the rows to spec.
@@ -1261,8 +1259,8 @@ void fft_z_symbol(const FftCtx<R>& f, double a, double b, const double* k0sum, d
   SymParams<R> sp;
   sp.a = (R)a;
   sp.b = (R)b;
-  sp.inv_ntot = (R)(1.0 / (double)f.ncell);
-  sp.mean_scale = a > 0.0 ? (R)(1.0 / (a * (double)f.ncell)) : R(0);
+  sp.inv_ntot = (R)(0.5 / (double)f.ncell);
+  sp.mean_scale = a > 0.0 ? (R)(0.5 / (a * (double)f.ncell)) : R(0);
   sp.dx = f.dx; sp.ddx = f.ddx;
   sp.dy = f.dy; sp.ddy = f.ddy;
   sp.dz = f.dz; sp.ddz = f.ddz;
@@ -1481,7 +1479,7 @@ void fft_yz_group(const FftCtx<R>& f, const RepFft* reps, int G, int which, cuda
     SymParams<R> sp;
     sp.a = R(0);
     sp.b = R(0);
-    sp.inv_ntot = (R)(1.0 / (double)f.ncell);
+    sp.inv_ntot = (R)(0.5 / (double)f.ncell);
     sp.mean_scale = R(0);   // per replica, from the table
     sp.dx = f.dx; sp.ddx = f.ddx;
     sp.dy = f.dy; sp.ddy = f.ddy;

@@ -486,8 +486,8 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (NT == 256 ? 3 : 2) : 1)
       if (2 * l + 1 < ny) col0[2 * l + 1] = mk(z0.y, zh.y);
     } else {
       const C zk = p[k], zm = p[nx - k];
-      p[k] = mk((zk.x + zm.x) * R(0.5), (zk.y - zm.y) * R(0.5));
-      p[nx - k] = mk((zk.y + zm.y) * R(0.5), (zm.x - zk.x) * R(0.5));
+      p[k] = mk(zk.x + zm.x, zk.y - zm.y);   // twice the spectrum (SymParams::inv_ntot)
+      p[nx - k] = mk(zk.y + zm.y, zm.x - zk.x);
     }
   }
   __syncthreads();
@@ -508,8 +508,8 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (NT == 256 ? 3 : 2) : 1)
   for (int f = tid; f < ny; f += NT) {   // the two real columns, by Hermitian symmetry along y
     const int p = A.y.pof[f], pm = A.y.pof[f == 0 ? 0 : ny - f];
     const C c = col0[p], d = col0[pm];
-    base[(size_t)p * A.kxp] = mk((c.x + d.x) * R(0.5), (c.y - d.y) * R(0.5));
-    if (nx % 2 == 0) base[(size_t)p * A.kxp + nx / 2] = mk((c.y + d.y) * R(0.5), (d.x - c.x) * R(0.5));
+    base[(size_t)p * A.kxp] = mk(c.x + d.x, c.y - d.y);
+    if (nx % 2 == 0) base[(size_t)p * A.kxp + nx / 2] = mk(c.y + d.y, d.x - c.x);
   }
 }
 

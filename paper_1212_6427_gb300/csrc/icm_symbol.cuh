@@ -8,8 +8,10 @@ namespace icm {
 
 template <typename R>
 struct SymParams {
-  R a, b, inv_ntot;
-  R mean_scale;   // the symbol's scale on the mean mode: 1/(a ncell), 0 when a = 0
+  R a, b;
+  R inv_ntot;     // 1/(2 ncell): the forward passes leave twice the spectrum (they split two packed real
+                  // rows without the factor 1/2)
+  R mean_scale;   // the symbol's scale on the mean mode: 1/(2 a ncell), 0 when a = 0
   const cplx_t<R>* dx; const R* ddx;
   const cplx_t<R>* dy; const R* ddy;
   const cplx_t<R>* dz; const R* ddz;
@@ -40,23 +42,27 @@ template <> __device__ __forceinline__ double recip<double>(double x) {
   return fma(y, fma(e, e, e), y);
 }
 
+// x > 0, in integer arithmetic for FP64 (and for what recip does not flush).
+__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool positive(double x) { return __double2hiint(x) >= 0x00100000; }
+
 template <typename R>
 __device__ __forceinline__ void apply_symbol(cplx_t<R>& c0, cplx_t<R>& c1, cplx_t<R>& c2, cplx_t<R> d0,
                                              cplx_t<R> d1, cplx_t<R> d2, R dd, const SymParams<R>& sp,
                                              bool mean_mode) {
-  const R den = sp.a + sp.b * dd;
-  const R prod = dd * den;
-  const R r = recip<R>(prod > R(0) ? prod : R(1));
-  if (dd > R(0)) {
+  R scale = sp.mean_scale;   // a = 0 (the steady Stokes solve): the mean mode has no solution and is dropped
+  if (!mean_mode) {          // |d|^2 = 0 only there: decided by index, comparisons are FP64 operations too
+    const R den = sp.a + sp.b * dd;
+    const R prod = dd * den;
+    const R r = positive(prod) ? recip<R>(prod) : R(0);
     const cplx_t<R> div = cadd(cadd(cmul(d0, c0), cmul(d1, c1)), cmul(d2, c2));
     const R inv_dd = den * r;
     const cplx_t<R> q = mk(div.x * inv_dd, div.y * inv_dd);
     c0 = csub(c0, cmul(cconj(d0), q));
     c1 = csub(c1, cmul(cconj(d1), q));
     c2 = csub(c2, cmul(cconj(d2), q));
+    scale = sp.inv_ntot * (dd * r);
   }
-  // a = 0 (the steady Stokes solve): the mean mode has no solution and is dropped
-  const R scale = prod > R(0) ? sp.inv_ntot * (dd * r) : (dd > R(0) ? R(0) : sp.mean_scale);
   c0 = cscale(c0, scale);
   c1 = cscale(c1, scale);
   c2 = cscale(c2, scale);
@@ -66,7 +72,6 @@ __device__ __forceinline__ void apply_symbol(cplx_t<R>& c0, cplx_t<R>& c1, cplx_
     c2 = mk((R)(sp.k0sum[2] * sp.k0mul), R(0));
   }
 }
-
 
 }  // namespace
 }  // namespace icm
