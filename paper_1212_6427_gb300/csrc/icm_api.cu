@@ -119,7 +119,7 @@ struct icm_sim {
   AxisPlan pz_alt;
   void *dz_alt = nullptr, *ddz_alt = nullptr;
   int kx = 0, kxp = 0;
-  alignas(64) unsigned char zmap[128];   // TMA descriptor of spec for the z pass
+  alignas(64) unsigned char zmap[kZMapBytes];   // TMA descriptors of spec for the z pass
   bool has_zmap = false;
   // blobs
   long long nb = 0, cap = 0;
@@ -1811,7 +1811,7 @@ bool stages_possible(const icm_batch* b) {
 }
 
 struct alignas(64) ZMap {
-  unsigned char bytes[128];
+  unsigned char bytes[kZMapBytes];
 };
 
 struct SolveGroup {

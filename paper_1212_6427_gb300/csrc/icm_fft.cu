@@ -264,7 +264,6 @@ template <typename R, int N, int MODE> constexpr int xi2_stage() { return xi2_le
 // The z pass holds all three components of its tile, so it takes 8 kx lines
 // (64-byte rows in FP32) to keep two blocks per SM; one thread per first-stage item
 // (3 components x R2 x 8), so the loads of all three components are in flight together.
-constexpr int kZLines = 8;
 template <typename R, int N, int R1, int R2>
 constexpr int zsym2_threads() { return 3 * R2 * kZLines > 1024 ? 1024 : 3 * R2 * kZLines; }
 // Threads of the plain z pass: one first-stage item each, except where the second stage
@@ -275,8 +274,7 @@ constexpr int zplain_threads() {
   return (sizeof(R) == 4 && R2 <= 12 && 2 * R1 < 3 * R2) ? R1 * kZLines : zsym2_threads<R, N, R1, R2>();
 }
 
-// The work of one z tile (3 components x N z x NL kx lines, kx0..kx0+NL-1, storage y
-// position py): forward z FFT, symbol, inverse z FFT.  The first stage reads the tile
+// The work of one z tile (3 components x N z x the NL lines of zt): forward z FFT, symbol, inverse z FFT.  The first stage reads the tile
 // from global memory (FROM_SMEM false) or from `buf`, where a TMA copy has put it.
 // Row of the z tile that holds spectral row R2 blk + n: within each block of R2 rows,
 // odd blocks swap adjacent rows (R2 even).  The second FFT stage reads the same n of
@@ -289,8 +287,8 @@ __device__ __forceinline__ int zrow(int blk, int n) {
 
 template <typename R, int N, int R1, int R2, bool FROM_SMEM, int NT>
 __device__ __forceinline__ void zsym_tile(cplx_t<R>* __restrict__ buf, const cplx_t<R>* __restrict__ tw,
-                                          cplx_t<R>* __restrict__ base, size_t cs, size_t zs, int kx0, int py, int kx,
-                                          const SymParams<R>& sp, const cplx_t<R>* __restrict__ dzt,
+                                          cplx_t<R>* __restrict__ spec, size_t cs, size_t zs, const ZTile<R>& zt, int ny,
+                                          int kx, int kxp, const SymParams<R>& sp, const cplx_t<R>* __restrict__ dzt,
                                           const R* __restrict__ ddzt, int tid) {
   using C = cplx_t<R>;
   constexpr int NL = kZLines;
@@ -310,22 +308,21 @@ __device__ __forceinline__ void zsym_tile(cplx_t<R>* __restrict__ buf, const cpl
   } else {
     for (int it = tid; it < 3 * R2 * NL; it += NT) {
       const int line = it % NL, rest = it / NL, n1 = rest % R2, c = rest / R2;
-      const bool ok = kx0 + line < kx;
+      const bool ok = zt.live(line, kx, ny);
+      const C* base = spec + zt.at(line, kxp);
       C a[R1];
 #pragma unroll
-      for (int r = 0; r < R1; ++r) a[r] = ok ? base[c * cs + (size_t)(n1 + R2 * r) * zs + line] : zero;
+      for (int r = 0; r < R1; ++r) a[r] = ok ? base[c * cs + (size_t)(n1 + R2 * r) * zs] : zero;
       stage_a_fwd<R, R1, R2>(a, tw + n1);
 #pragma unroll
       for (int k2 = 0; k2 < R1; ++k2) buf[(c * N + zrow<R2>(k2, n1)) * NL + line] = a[k2];
     }
   }
   __syncthreads();
-  const C dyv = sp.dy[py];
-  const R ddy = sp.ddy[py];
   if (HOLD3) {
     for (int it = tid; it < R1 * NL; it += NT) {
-      const int line = it % NL, blk = it / NL, k = kx0 + line;
-      if (k >= kx) continue;
+      const int line = it % NL, blk = it / NL, k = zt.k(line), py = zt.row(line);
+      if (k >= kx || py >= ny) continue;
       C b[3][R2];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -333,12 +330,12 @@ __device__ __forceinline__ void zsym_tile(cplx_t<R>* __restrict__ buf, const cpl
         for (int n = 0; n < R2; ++n) b[c][n] = buf[(c * N + zrow<R2>(blk, n)) * NL + line];
         SDft<R, R2>::run(b[c]);
       }
-      const C d0 = sp.dx[k];
-      const R ddx = sp.ddx[k];
+      const C d0 = sp.dx[k], dyv = sp.dy[py];
+      const R dxy = sp.ddx[k] + sp.ddy[py];
 #pragma unroll
       for (int k1 = 0; k1 < R2; ++k1) {
         const int pz = R2 * blk + k1;
-        apply_symbol<R>(b[0][k1], b[1][k1], b[2][k1], d0, dyv, dzt[pz], ddx + ddy + ddzt[pz], sp,
+        apply_symbol<R>(b[0][k1], b[1][k1], b[2][k1], d0, dyv, dzt[pz], dxy + ddzt[pz], sp,
                         k == 0 && py == 0 && pz == 0);
       }
 #pragma unroll
@@ -361,13 +358,14 @@ __device__ __forceinline__ void zsym_tile(cplx_t<R>* __restrict__ buf, const cpl
     __syncthreads();
     // NT is a multiple of NL, so a thread keeps its line (and its x symbol) in every round
     static_assert(NT % NL == 0, "fixed line per thread");
-    const int kt = kx0 + tid % NL;
-    const C dxt = sp.dx[kt < kx ? kt : 0];
-    const R dxy = sp.ddx[kt < kx ? kt : 0] + ddy;
+    const bool ok = zt.live(tid % NL, kx, ny);
+    const int kt = ok ? zt.k(tid % NL) : 0, py = ok ? zt.row(tid % NL) : 0;
+    const C dxt = sp.dx[kt], dyv = sp.dy[py];
+    const R dxy = sp.ddx[kt] + sp.ddy[py];
     for (int it = tid; it < N * NL; it += NT) {
       const int pr = it / NL;                                  // row of the tile
       const int pz = zrow<R2>(pr / R2, pr % R2);               // its spectral row (the swap is an involution)
-      if (kt >= kx) continue;
+      if (!ok) continue;
       C& c0 = buf[it];
       C& c1 = buf[N * NL + it];
       C& c2 = buf[2 * N * NL + it];
@@ -387,13 +385,14 @@ __device__ __forceinline__ void zsym_tile(cplx_t<R>* __restrict__ buf, const cpl
   __syncthreads();
   for (int it = tid; it < 3 * R2 * NL; it += NT) {
     const int line = it % NL, rest = it / NL, n1 = rest % R2, c = rest / R2;
-    if (kx0 + line >= kx) continue;
+    if (!zt.live(line, kx, ny)) continue;
+    C* base = spec + zt.at(line, kxp);
     C a[R1];
 #pragma unroll
     for (int k2 = 0; k2 < R1; ++k2) a[k2] = buf[(c * N + zrow<R2>(k2, n1)) * NL + line];
     stage_a_inv<R, R1, R2>(a, tw + n1);
 #pragma unroll
-    for (int n2 = 0; n2 < R1; ++n2) base[c * cs + (size_t)(n1 + R2 * n2) * zs + line] = a[n2];
+    for (int n2 = 0; n2 < R1; ++n2) base[c * cs + (size_t)(n1 + R2 * n2) * zs] = a[n2];
   }
 }
 
@@ -418,10 +417,10 @@ __global__ void __launch_bounds__(zplain_threads<R, N, R1, R2>(), sizeof(R) == 4
   C* tw = buf + 3 * N * NL;                  // [N] first-stage twiddles, [k2][n1]
   const int tid = threadIdx.x;
   load_stage_twiddles<R, R1, R2>(tw, gtw, tid, NT);
-  const int kx0 = blockIdx.x * NL, py = blockIdx.y;
+  const ZTile<R> zt(blockIdx.x, kx, ny);
   const size_t zs = (size_t)ny * kxp, cs = (size_t)N * zs;
   __syncthreads();
-  zsym_tile<R, N, R1, R2, false, NT>(buf, tw, spec + (size_t)py * kxp + kx0, cs, zs, kx0, py, kx, sp, sp.dz, sp.ddz, tid);
+  zsym_tile<R, N, R1, R2, false, NT>(buf, tw, spec, cs, zs, zt, ny, kx, kxp, sp, sp.dz, sp.ddz, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -473,11 +472,15 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// GRP: tiles of every replica of a group (reps, nrep; the map covers the group buffer).
+struct ZMaps {
+  CUtensorMap row, fold;   // boxes of a tile along a row, of a folded one (FP64)
+};
+
+// GRP: tiles of every replica of a group (reps, nrep; the maps cover the group buffer).
 template <typename R, int N, int R1, int R2, bool GRP = false>
 __global__ void __launch_bounds__(zsym2_threads<R, N, R1, R2>(), sizeof(R) == 4 ? 2 : 1)
-    k_zsym_tma(const __grid_constant__ CUtensorMap zmap, cplx_t<R>* __restrict__ spec,
-               const cplx_t<R>* __restrict__ gtw, int ny, int kx, int kxp, int ntx, SymParams<R> sp, int* err,
+    k_zsym_tma(const __grid_constant__ ZMaps zmap, cplx_t<R>* __restrict__ spec,
+               const cplx_t<R>* __restrict__ gtw, int ny, int kx, int kxp, int tpm, SymParams<R> sp, int* err,
                const RepFft* __restrict__ reps, int nrep) {
   using C = cplx_t<R>;
   constexpr int NL = kZLines;
@@ -505,20 +508,20 @@ __global__ void __launch_bounds__(zsym2_threads<R, N, R1, R2>(), sizeof(R) == 4 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  // tiles: ntx x ny per spectrum; with reps, replica e = t / (ntx ny) of the table, whose
+  // tiles: tpm per spectrum; with reps, replica e = t / tpm of the table, whose
   // spectrum is the slot-th of the group buffer the map covers (components 3 slot ..)
-  const int tpm = ntx * ny;
   const int ntiles = GRP ? tpm * nrep : tpm;
   const size_t zs = (size_t)ny * kxp, cs = (size_t)N * zs;
   auto issue = [&](int t, int st) {
-    const int e = GRP ? t / tpm : 0, tt = t - e * tpm;
-    const int kx0 = (tt % ntx) * NL, py = tt / ntx;
+    const int e = GRP ? t / tpm : 0;
+    const ZTile<R> zt(t - e * tpm, kx, ny);
+    const CUtensorMap* map = zt.folded ? &zmap.fold : &zmap.row;
     const int c0 = GRP ? 3 * reps[e].slot : 0;
     // order this block's earlier generic-proxy writes of the buffer before the copy
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     mbar_expect_tx(&mbar[st], TILE_BYTES);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) tma_load_4d(bufs + st * TILE + c * N * NL, &zmap, 2 * kx0, py, 0, c0 + c, &mbar[st]);
+    for (int c = 0; c < 3; ++c) tma_load_4d(bufs + st * TILE + c * N * NL, map, 2 * zt.k0, zt.row0, 0, c0 + c, &mbar[st]);
   };
   int t = blockIdx.x;
   if (tid == 0 && t < ntiles) issue(t, 0);
@@ -533,8 +536,8 @@ __global__ void __launch_bounds__(zsym2_threads<R, N, R1, R2>(), sizeof(R) == 4 
     }
     __syncthreads();
     if (!s_ok) break;
-    const int e = GRP ? t / tpm : 0, tt = t - e * tpm;
-    const int kx0 = (tt % ntx) * NL, py = tt / ntx;
+    const int e = GRP ? t / tpm : 0;
+    const ZTile<R> zt(t - e * tpm, kx, ny);
     C* sbase = spec;
     SymParams<R> spt = sp;
     if constexpr (GRP) {   // the replica's spectrum and symbol
@@ -547,9 +550,8 @@ __global__ void __launch_bounds__(zsym2_threads<R, N, R1, R2>(), sizeof(R) == 4 
       spt.k0mul = rp.k0mul;
     }
     // (checked build) the tile's row and its last column lie inside the padded spectrum
-    if (index_ok(py, ny, err) && index_ok(kx0 + NL - 1, kxp, err))
-      zsym_tile<R, N, R1, R2, true, NT>(bufs + st * TILE, tw, sbase + (size_t)py * kxp + kx0, cs, zs, kx0, py, kx,
-                                        spt, zdz, zddz, tid);
+    if (index_ok(zt.row0, ny, err) && index_ok(zt.k(NL - 1), kxp, err))
+      zsym_tile<R, N, R1, R2, true, NT>(bufs + st * TILE, tw, sbase, cs, zs, zt, ny, kx, kxp, spt, zdz, zddz, tid);
     __syncthreads();
   }
   if (tid == 0 && !s_ok && t < ntiles) {
@@ -588,6 +590,14 @@ constexpr int y_threads() {
   return sizeof(R) == 4 || items > kThreads ? kThreads : items < 64 ? 64 : items;
 }
 
+// The columns of the y pass go in tiles of seg_lines.  In FP64, where rows are one column longer than whole
+// tiles, the last column of as many planes as a tile has lines makes a tile of its own (see ZTile; y pass of
+// 128^3 146 / 135 us; FP32 on 512 x 384 x 256, bound by memory, 272 / 280).
+template <typename R>
+__host__ __device__ constexpr bool y_folds(int kx) {
+  return sizeof(R) == 8 && kx % seg_lines<R>() == 1 && kx > seg_lines<R>();
+}
+
 template <typename R, int N, int R1, int R2, bool INV>
 __global__ void __launch_bounds__(y_threads<R, N, R2>()) k_ypass2(cplx_t<R>* __restrict__ spec, const cplx_t<R>* __restrict__ gtw,
                                                      int nz, int kx, int kxp, const RepFft* __restrict__ reps) {
@@ -605,19 +615,27 @@ __global__ void __launch_bounds__(y_threads<R, N, R2>()) k_ypass2(cplx_t<R>* __r
   // them in L2.  The inverse pass walks forwards.
   const int bx = INV ? blockIdx.x : gridDim.x - 1 - blockIdx.x;
   const int by = INV ? blockIdx.y : gridDim.y - 1 - blockIdx.y;
-  const int kx0 = bx * NL, z0 = by * ZB, comp = INV ? blockIdx.z % 3 : 2 - blockIdx.z % 3;
-  // plane z0 + zb of the component, columns kx0..
-  C* base0 = spec + ((size_t)(comp * nz + z0) * N) * kxp + kx0;
+  const int comp = INV ? blockIdx.z % 3 : 2 - blockIdx.z % 3;
+  // lines: columns kx0.. of planes z0 + zb, or the last column of planes z0 + zb NL + line (see y_folds)
+  const int zgroups = (nz + ZB - 1) / ZB;
+  const bool folded = sizeof(R) == 8 && by >= zgroups;
+  const int kx0 = folded ? kx - 1 : bx * NL, z0 = folded ? ((by - zgroups) * gridDim.x + bx) * (ZB * NL) : by * ZB;
+  if (z0 >= nz) return;
+  const size_t plane = (size_t)N * kxp, lstep = folded ? plane : 1, zstep = folded ? NL * plane : plane;
+  C* base0 = spec + (comp * nz + z0) * plane + kx0;
+  const auto live = [&](int line, int zb) {
+    return folded ? z0 + zb * NL + line < nz : kx0 + line < kx && z0 + zb < nz;
+  };
   const C zero = mk(R(0), R(0));
   if (!INV) {
     // the loads of this thread's first item go out before the twiddle table is staged
     // (whose barrier they would otherwise wait behind)
     const auto load_item = [&](int it, C (&a)[R1]) {
       const int line = it % NL, rest = it / NL, n1 = rest % R2, zb = rest / R2;
-      const bool ok = kx0 + line < kx && z0 + zb < nz;
-      const C* base = base0 + (size_t)zb * N * kxp;
+      const bool ok = live(line, zb);
+      const C* base = base0 + zb * zstep + line * lstep;
 #pragma unroll
-      for (int r = 0; r < R1; ++r) a[r] = ok ? base[(size_t)(n1 + R2 * r) * kxp + line] : zero;
+      for (int r = 0; r < R1; ++r) a[r] = ok ? base[(size_t)(n1 + R2 * r) * kxp] : zero;
     };
     C a[R1];
     if (tid < ZB * R2 * NL) load_item(tid, a);
@@ -633,25 +651,25 @@ __global__ void __launch_bounds__(y_threads<R, N, R2>()) k_ypass2(cplx_t<R>* __r
     __syncthreads();
     for (int it = tid; it < ZB * R1 * NL; it += NT) {
       const int line = it % NL, rest = it / NL, blk = rest % R1, zb = rest / R1;
-      if (kx0 + line >= kx || z0 + zb >= nz) continue;
-      C* base = base0 + (size_t)zb * N * kxp;
+      if (!live(line, zb)) continue;
+      C* base = base0 + zb * zstep + line * lstep;
       C b[R2];
 #pragma unroll
       for (int n = 0; n < R2; ++n) b[n] = buf[(zb * N + R2 * blk + n) * NL + line];
       SDft<R, R2>::run(b);
 #pragma unroll
-      for (int k1 = 0; k1 < R2; ++k1) base[(size_t)(R2 * blk + k1) * kxp + line] = b[k1];
+      for (int k1 = 0; k1 < R2; ++k1) base[(size_t)(R2 * blk + k1) * kxp] = b[k1];
     }
   } else {
     // the second stage comes first and needs no twiddles: its loads go out first, the
     // table is staged after it, before the barrier the first stage waits at anyway
     for (int it = tid; it < ZB * R1 * NL; it += NT) {
       const int line = it % NL, rest = it / NL, blk = rest % R1, zb = rest / R1;
-      const bool ok = kx0 + line < kx && z0 + zb < nz;
-      const C* base = base0 + (size_t)zb * N * kxp;
+      const bool ok = live(line, zb);
+      const C* base = base0 + zb * zstep + line * lstep;
       C b[R2];
 #pragma unroll
-      for (int k1 = 0; k1 < R2; ++k1) b[k1] = ok ? base[(size_t)(R2 * blk + k1) * kxp + line] : zero;
+      for (int k1 = 0; k1 < R2; ++k1) b[k1] = ok ? base[(size_t)(R2 * blk + k1) * kxp] : zero;
       sdft_inv<R, R2>(b);
 #pragma unroll
       for (int n = 0; n < R2; ++n) buf[(zb * N + R2 * blk + n) * NL + line] = b[n];
@@ -660,14 +678,14 @@ __global__ void __launch_bounds__(y_threads<R, N, R2>()) k_ypass2(cplx_t<R>* __r
     __syncthreads();
     for (int it = tid; it < ZB * R2 * NL; it += NT) {
       const int line = it % NL, rest = it / NL, n1 = rest % R2, zb = rest / R2;
-      if (kx0 + line >= kx || z0 + zb >= nz) continue;
-      C* base = base0 + (size_t)zb * N * kxp;
+      if (!live(line, zb)) continue;
+      C* base = base0 + zb * zstep + line * lstep;
       C a[R1];
 #pragma unroll
       for (int k2 = 0; k2 < R1; ++k2) a[k2] = buf[(zb * N + n1 + R2 * k2) * NL + line];
       stage_a_inv<R, R1, R2>(a, tw + n1);
 #pragma unroll
-      for (int n2 = 0; n2 < R1; ++n2) base[(size_t)(n1 + R2 * n2) * kxp + line] = a[n2];
+      for (int n2 = 0; n2 < R1; ++n2) base[(size_t)(n1 + R2 * n2) * kxp] = a[n2];
     }
   }
 }
@@ -1076,16 +1094,30 @@ template <typename R, int N> size_t smem_z2() { return 3 * (size_t)N * kZLines *
 template <typename R, int N, int R2> size_t smem_y2() {
   return (size_t)y_planes<R, N, R2>() * N * seg_lines<R>() * sizeof(cplx_t<R>) + N * sizeof(cplx_t<R>);
 }
+// Blocks of a y pass over G spectra: tiles along kx by plane groups, and further rows of blocks for the
+// folded last column.
+template <typename R, int N, int R2>
+dim3 y_grid(const FftCtx<R>& f, int G) {
+  constexpr int NL = seg_lines<R>(), ZB = y_planes<R, N, R2>();
+  const int zgroups = (f.nz + ZB - 1) / ZB;
+  if (!y_folds<R>(f.kx)) return dim3((f.kx + NL - 1) / NL, zgroups, 3 * G);
+  const int full = f.kx / NL, folded = (f.nz + ZB * NL - 1) / (ZB * NL);
+  return dim3(full, zgroups + (folded + full - 1) / full, 3 * G);
+}
+
 template <typename R, int N, int R1, int R2, bool GRP>
-void launch_ztma(int grid, const CUtensorMap& map, cplx_t<R>* spec, const cplx_t<R>* tw, const FftCtx<R>& f, int kxz,
-                 const SymParams<R>& sp, const RepFft* reps, int G, cudaStream_t st) {
+void launch_ztma(const void* zmap, cplx_t<R>* spec, const cplx_t<R>* tw, const FftCtx<R>& f, const SymParams<R>& sp,
+                 const RepFft* reps, int G, cudaStream_t st) {
+  const int tpm = z_tiles<R>(f.kx, f.ny);
+  const int grid = std::min(tpm * G, 2 * device_sms());
   k_zsym_tma<R, N, R1, R2, GRP><<<grid, zsym2_threads<R, N, R1, R2>(), smem_ztma<R, N>(), st>>>(
-      map, spec, tw, f.ny, f.kx, f.kxp, kxz, sp, f.err, reps, G);
+      *reinterpret_cast<const ZMaps*>(zmap), spec, tw, f.ny, f.kx, f.kxp, tpm, sp, f.err, reps, G);
 }
 
 template <typename R, int N, int R1, int R2>
-void launch_zplain(dim3 grid, cplx_t<R>* spec, const cplx_t<R>* tw, const FftCtx<R>& f, const SymParams<R>& sp,
-                   const RepFft* reps, cudaStream_t st) {
+void launch_zplain(cplx_t<R>* spec, const cplx_t<R>* tw, const FftCtx<R>& f, const SymParams<R>& sp, const RepFft* reps,
+                   int G, cudaStream_t st) {
+  const dim3 grid(z_tiles<R>(f.kx, f.ny), 1, G);
   k_zsym2<R, N, R1, R2><<<grid, zplain_threads<R, N, R1, R2>(), smem_z2<R, N>(), st>>>(spec, tw, f.ny, f.kx, f.kxp,
                                                                                     sp, reps);
 }
@@ -1240,9 +1272,9 @@ void fft_y(const FftCtx<R>& f, bool inverse, cudaStream_t st) {
 #define ICM_CASE(N, R1, R2)                                                                                   \
   case N:                                                                                                     \
     if (inverse)                                                                                              \
-      k_ypass2<R, N, R1, R2, true><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(f.spec, tw, f.nz, f.kx, f.kxp, nullptr);  \
+      k_ypass2<R, N, R1, R2, true><<<y_grid<R, N, R2>(f, 1), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(f.spec, tw, f.nz, f.kx, f.kxp, nullptr);  \
     else                                                                                                      \
-      k_ypass2<R, N, R1, R2, false><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(f.spec, tw, f.nz, f.kx, f.kxp, nullptr); \
+      k_ypass2<R, N, R1, R2, false><<<y_grid<R, N, R2>(f, 1), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(f.spec, tw, f.nz, f.kx, f.kxp, nullptr); \
     return;
     ICM_FFT_SIDES(ICM_CASE)
 #undef ICM_CASE
@@ -1267,20 +1299,15 @@ void fft_z_symbol(const FftCtx<R>& f, double a, double b, const double* k0sum, d
   sp.k0sum = k0sum;
   sp.k0mul = k0scale / (double)f.ncell;
   const cplx_t<R>* tw = (const cplx_t<R>*)f.pz.tw;
-  const int kxz = (f.kx + kZLines - 1) / kZLines;
   if (f.zmap != nullptr && f.nz <= 256) {
-    const int nsm = device_sms();
-    const int ntiles = kxz * f.ny;
-    const int grid = ntiles < 2 * nsm ? ntiles : 2 * nsm;
-    const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(f.zmap);
     switch (f.nz) {
 #define ICM_CASE(N, R1, R2)                                                                                            \
   case N:                                                                                                              \
     if (N <= 256) {                                                                                                    \
       if (f.zalt)                                                                                                      \
-        launch_ztma<R, N, zalt_r1<N, R1>(), N / zalt_r1<N, R1>(), false>(grid, map, f.spec, tw, f, kxz, sp, nullptr, 1, st); \
+        launch_ztma<R, N, zalt_r1<N, R1>(), N / zalt_r1<N, R1>(), false>(f.zmap, f.spec, tw, f, sp, nullptr, 1, st);     \
       else                                                                                                             \
-        launch_ztma<R, N, R1, R2, false>(grid, map, f.spec, tw, f, kxz, sp, nullptr, 1, st);                         \
+        launch_ztma<R, N, R1, R2, false>(f.zmap, f.spec, tw, f, sp, nullptr, 1, st);                             \
       return;                                                                                                          \
     }                                                                                                                  \
     break;
@@ -1293,9 +1320,9 @@ void fft_z_symbol(const FftCtx<R>& f, double a, double b, const double* k0sum, d
 #define ICM_CASE(N, R1, R2)                                                                                     \
   case N:                                                                                                       \
     if (f.zalt)                                                                                                 \
-      launch_zplain<R, N, zalt_r1<N, R1>(), N / zalt_r1<N, R1>()>(dim3(kxz, f.ny), f.spec, tw, f, sp, nullptr, st); \
+      launch_zplain<R, N, zalt_r1<N, R1>(), N / zalt_r1<N, R1>()>(f.spec, tw, f, sp, nullptr, 1, st); \
     else                                                                                                        \
-      launch_zplain<R, N, R1, R2>(dim3(kxz, f.ny), f.spec, tw, f, sp, nullptr, st);                            \
+      launch_zplain<R, N, R1, R2>(f.spec, tw, f, sp, nullptr, 1, st);                            \
     return;
     ICM_FFT_SIDES(ICM_CASE)
 #undef ICM_CASE
@@ -1472,9 +1499,6 @@ template <typename R>
 void fft_yz_group(const FftCtx<R>& f, const RepFft* reps, int G, int which, cudaStream_t st, const void* gzmap) {
   const cplx_t<R>* twy = (const cplx_t<R>*)f.py.tw;
   const cplx_t<R>* twz = (const cplx_t<R>*)f.pz.tw;
-  constexpr int NL = seg_lines<R>();
-  const int kxt = (f.kx + NL - 1) / NL;
-  const int kxz = (f.kx + kZLines - 1) / kZLines;
   if (which == 1) {   // z FFT, symbol, inverse z FFT
     SymParams<R> sp;
     sp.a = R(0);
@@ -1487,16 +1511,14 @@ void fft_yz_group(const FftCtx<R>& f, const RepFft* reps, int G, int which, cuda
     sp.k0sum = nullptr;
     sp.k0mul = 0.0;
     if (gzmap != nullptr && f.nz <= 256) {
-      const int grid = std::min(kxz * f.ny * G, 2 * device_sms());
-      const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(gzmap);
       switch (f.nz) {
 #define ICM_CASE(N, R1, R2)                                                                                            \
   case N:                                                                                                              \
     if (N <= 256) {                                                                                                    \
       if (f.zalt)                                                                                                      \
-        launch_ztma<R, N, zalt_r1<N, R1>(), N / zalt_r1<N, R1>(), true>(grid, map, nullptr, twz, f, kxz, sp, reps, G, st); \
+        launch_ztma<R, N, zalt_r1<N, R1>(), N / zalt_r1<N, R1>(), true>(gzmap, nullptr, twz, f, sp, reps, G, st); \
       else                                                                                                             \
-        launch_ztma<R, N, R1, R2, true>(grid, map, nullptr, twz, f, kxz, sp, reps, G, st);                           \
+        launch_ztma<R, N, R1, R2, true>(gzmap, nullptr, twz, f, sp, reps, G, st);                           \
       return;                                                                                                          \
     }                                                                                                                  \
     break;
@@ -1509,9 +1531,9 @@ void fft_yz_group(const FftCtx<R>& f, const RepFft* reps, int G, int which, cuda
 #define ICM_CASE(N, R1, R2)                                                                                     \
   case N:                                                                                                       \
     if (f.zalt)                                                                                                 \
-      launch_zplain<R, N, zalt_r1<N, R1>(), N / zalt_r1<N, R1>()>(dim3(kxz, f.ny, G), nullptr, twz, f, sp, reps, st); \
+      launch_zplain<R, N, zalt_r1<N, R1>(), N / zalt_r1<N, R1>()>(nullptr, twz, f, sp, reps, G, st); \
     else                                                                                                        \
-      launch_zplain<R, N, R1, R2>(dim3(kxz, f.ny, G), nullptr, twz, f, sp, reps, st);                          \
+      launch_zplain<R, N, R1, R2>(nullptr, twz, f, sp, reps, G, st);                          \
     return;
       ICM_FFT_SIDES(ICM_CASE)
 #undef ICM_CASE
@@ -1522,9 +1544,9 @@ void fft_yz_group(const FftCtx<R>& f, const RepFft* reps, int G, int which, cuda
 #define ICM_CASE(N, R1, R2)                                                                                             \
   case N:                                                                                                               \
     if (which == 2)                                                                                                     \
-      k_ypass2<R, N, R1, R2, true><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3 * G), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(nullptr, twy, f.nz, f.kx, f.kxp, reps); \
+      k_ypass2<R, N, R1, R2, true><<<y_grid<R, N, R2>(f, G), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(nullptr, twy, f.nz, f.kx, f.kxp, reps); \
     else                                                                                                                \
-      k_ypass2<R, N, R1, R2, false><<<dim3(kxt, (f.nz + y_planes<R, N, R2>() - 1) / y_planes<R, N, R2>(), 3 * G), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(nullptr, twy, f.nz, f.kx, f.kxp, reps); \
+      k_ypass2<R, N, R1, R2, false><<<y_grid<R, N, R2>(f, G), y_threads<R, N, R2>(), smem_y2<R, N, R2>(), st>>>(nullptr, twy, f.nz, f.kx, f.kxp, reps); \
     return;
       ICM_FFT_SIDES(ICM_CASE)
 #undef ICM_CASE
@@ -1598,9 +1620,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// The spectrum as a 4-D tensor (floats along kx, y, z, component) and the box one z
-// tile of one component occupies: 2 kZLines floats x 1 x nz x 1.  Wave numbers past
-// kx read as zeros.
+// The spectrum as a 4-D tensor (floats along kx, y, z, component) and the boxes one z
+// tile of one component occupies (ZMaps): 2 kZLines floats x 1 x nz x 1 or, in FP64, 2 x
+// kZLines x nz x 1.  Wave numbers past kx and rows past ny read as zeros.
 bool make_zmap(void* map, const void* spec, int precision, int kx, int kxp, int ny, int nz, int ncomp) {
   int r1 = 0, r2 = 0;
   if (nz > 256 || !fft_split(nz, r1, r2)) return false;
@@ -1619,14 +1641,17 @@ bool make_zmap(void* map, const void* spec, int precision, int kx, int kxp, int 
   const cuuint64_t dims[4] = {(cuuint64_t)(2 * kx), (cuuint64_t)ny, (cuuint64_t)nz, (cuuint64_t)ncomp};
   const cuuint64_t strides[3] = {2 * (cuuint64_t)kxp * es, 2 * (cuuint64_t)kxp * es * ny,
                                  2 * (cuuint64_t)kxp * es * ny * nz};
-  const cuuint32_t box[4] = {2 * kZLines, 1, (cuuint32_t)nz, 1};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
-  const CUresult r = fn(reinterpret_cast<CUtensorMap*>(map),
-                        precision == 32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4,
-                        const_cast<void*>(spec), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
+  const auto encode = [&](CUtensorMap* m, int cols) {
+    const cuuint32_t box[4] = {(cuuint32_t)(2 * cols), (cuuint32_t)(kZLines / cols), (cuuint32_t)nz, 1};
+    return fn(m, precision == 32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4,
+              const_cast<void*>(spec), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  static_assert(sizeof(ZMaps) == kZMapBytes, "the callers' storage");
+  ZMaps* m = reinterpret_cast<ZMaps*>(map);
+  return encode(&m->row, kZLines) && (precision == 32 || encode(&m->fold, 1));
 }
 
 #endif

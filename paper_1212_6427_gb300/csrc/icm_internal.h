@@ -88,13 +88,14 @@ struct FftCtx {
   const cplx_t<R>* dy; const R* ddy;
   const cplx_t<R>* dz; const R* ddz;
   cplx_t<R>* spec;   // 3 * nz * ny * kxp complex scratch
-  const void* zmap;  // host copy of the TMA descriptor of spec for the z pass (or null)
+  const void* zmap;  // host copy of the TMA descriptors of spec for the z pass (or null)
   int* err;          // device error bits (bounded waits report here)
   int zalt;          // 1: the z pass uses the other split of fft_split_z_alt (pz, dz, ddz follow it)
 };
 
 // Fill `map` (a 128-byte CUtensorMap) with the descriptor the TMA z pass uses for a
 // spectrum buffer; returns false if TMA is unavailable for this shape.
+constexpr int kZMapBytes = 256;   // two tensor maps
 bool make_zmap(void* map, const void* spec, int precision, int kx, int kxp, int ny, int nz, int ncomp = 3);
 
 enum OutMode : int { OUT_STORE = 0, OUT_ADD_AND_STORE2 = 1, OUT_ADD = 2, OUT_NONE = 3 };

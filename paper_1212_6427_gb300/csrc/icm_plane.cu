@@ -644,12 +644,12 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (NT == 256 ? 3 : 2) : 1)
 // The first stage reads global memory into registers, the last one writes it, and the middle stage
 // keeps the three components of its wave numbers in registers through the symbol.
 // ---------------------------------------------------------------------------
-constexpr int kZAny = 8;
+constexpr int kZAny = kZLines;
 
 template <typename R, int RAD, bool INV, bool GLOBAL, int NT>
 __device__ __forceinline__ void z_stage(cplx_t<R>* __restrict__ buf, const StageAxis& Z, int s,
                                         const cplx_t<R>* __restrict__ tw, cplx_t<R>* __restrict__ base, size_t zs,
-                                        size_t cs, int live, int tid) {
+                                        size_t cs, bool live, int tid) {
   using C = cplx_t<R>;
   const int M = Z.M[s], mr = M / RAD, tws = Z.n / M, nbf = Z.n / RAD;
   for (int it = tid; it < 3 * nbf * kZAny; it += NT) {
@@ -657,18 +657,18 @@ __device__ __forceinline__ void z_stage(cplx_t<R>* __restrict__ buf, const Stage
     const int comp = rest < nbf ? 0 : (rest < 2 * nbf ? 1 : 2), bf = rest - comp * nbf;
     const int blk = GLOBAL ? 0 : (int)Z.dmr[s].div(bf), n1 = GLOBAL ? bf : bf - blk * mr;
     C* p = buf + (comp * Z.n + blk * M + n1) * kZAny + line;
-    C* g = base + comp * cs + n1 * zs + line;
+    C* g = base + comp * cs + n1 * zs;
     C a[RAD];
     if (GLOBAL && !INV) {
 #pragma unroll
-      for (int r = 0; r < RAD; ++r) a[r] = line < live ? g[(size_t)(r * mr) * zs] : mk(R(0), R(0));
+      for (int r = 0; r < RAD; ++r) a[r] = live ? g[(size_t)(r * mr) * zs] : mk(R(0), R(0));
     } else {
 #pragma unroll
       for (int r = 0; r < RAD; ++r) a[r] = p[r * mr * kZAny];
     }
     butterfly<R, RAD, INV, INV>(a, tw, n1 * tws, true);
     if (GLOBAL && INV) {
-      if (line < live) {
+      if (live) {
 #pragma unroll
         for (int r = 0; r < RAD; ++r) g[(size_t)(r * mr) * zs] = a[r];
       }
@@ -684,7 +684,7 @@ __device__ __forceinline__ void z_stage(cplx_t<R>* __restrict__ buf, const Stage
 // are a serial chain of FP64 operations (18.4 us against 12.2 per pass on 16^3).
 template <typename R, int RAD, int NT>
 __device__ __forceinline__ void z_symbol_apart(cplx_t<R>* __restrict__ buf, const StageAxis& Z, const SymParams<R>& sp,
-                                               int kx0, int py, int live, int tid) {
+                                               int k, int py, bool live, int tid) {
   using C = cplx_t<R>;
   const int cs = Z.n * kZAny, nbf = Z.n / RAD;
   const auto dft = [&](bool inv) {
@@ -706,8 +706,8 @@ __device__ __forceinline__ void z_symbol_apart(cplx_t<R>* __restrict__ buf, cons
   const C dyv = sp.dy[py];
   const R ddy = sp.ddy[py];
   for (int it = tid; it < cs; it += NT) {
-    const int line = it % kZAny, pz = it / kZAny, k = kx0 + line;
-    if (line < live)
+    const int pz = it / kZAny;
+    if (live)
       apply_symbol<R>(buf[it], buf[cs + it], buf[2 * cs + it], sp.dx[k], dyv, sp.dz[pz], sp.ddx[k] + ddy + sp.ddz[pz], sp,
                       k == 0 && py == 0 && pz == 0);
   }
@@ -717,13 +717,13 @@ __device__ __forceinline__ void z_symbol_apart(cplx_t<R>* __restrict__ buf, cons
 
 template <typename R, int RAD, int NT>
 __device__ __forceinline__ void z_symbol_stage(cplx_t<R>* __restrict__ buf, const StageAxis& Z, const SymParams<R>& sp,
-                                               int kx0, int py, int live, int tid) {
+                                               int k, int py, bool live, int tid) {
   using C = cplx_t<R>;
   const C dyv = sp.dy[py];
   const R ddy = sp.ddy[py];
   for (int it = tid; it < (Z.n / RAD) * kZAny; it += NT) {
-    const int line = it % kZAny, blk = it / kZAny, k = kx0 + line;
-    if (line >= live) continue;
+    const int line = it % kZAny, blk = it / kZAny;
+    if (!live) continue;
     C b[3][RAD];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -757,10 +757,14 @@ __global__ void __launch_bounds__(kZAnyThreads, sizeof(R) == 4 ? 4 : 2)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
   C* tw = buf + 3 * Z.n * kZAny;
-  const int tid = threadIdx.x, kx0 = blockIdx.x * kZAny, py = blockIdx.y;
-  const int live = min(kZAny, kx - kx0);
+  const int tid = threadIdx.x;
+  // NT is a multiple of kZAny: a thread keeps its line in every loop
+  static_assert(NT % kZAny == 0, "fixed line per thread");
+  const ZTile<R> zt(blockIdx.x, kx, ny);
+  const bool live = zt.live(tid % kZAny, kx, ny);
+  const int k = live ? zt.k(tid % kZAny) : 0, py = live ? zt.row(tid % kZAny) : 0;
   const size_t zs = (size_t)ny * kxp, cs = (size_t)Z.n * zs;
-  C* base = spec + (size_t)py * kxp + kx0;
+  C* base = spec + (size_t)py * kxp + k;
   for (int i = tid; i < Z.n; i += NT) tw[i] = ((const C*)Z.tw)[i];
   __syncthreads();
 #define ICM_Z(RAD) z_stage<R, RAD, false, true, NT>(buf, Z, 0, tw, base, zs, cs, live, tid)
@@ -775,9 +779,9 @@ __global__ void __launch_bounds__(kZAnyThreads, sizeof(R) == 4 ? 4 : 2)
   }
 #define ICM_Z(RAD)                                              \
   if constexpr (sizeof(R) == 4)                                 \
-    z_symbol_stage<R, RAD, NT>(buf, Z, sp, kx0, py, live, tid); \
+    z_symbol_stage<R, RAD, NT>(buf, Z, sp, k, py, live, tid); \
   else                                                          \
-    z_symbol_apart<R, RAD, NT>(buf, Z, sp, kx0, py, live, tid)
+    z_symbol_apart<R, RAD, NT>(buf, Z, sp, k, py, live, tid)
   switch (Z.rad[Z.ns - 1]) {   // the last factor of a general side (general_factors)
     case 2: ICM_Z(2); break;
     case 3: ICM_Z(3); break;
@@ -935,7 +939,7 @@ template <typename R>
 void fft_z_any(const FftCtx<R>& f, const SymParams<R>& sp, cudaStream_t st) {
   const StageAxis Z = stage_axis(f.pz);
   const size_t sm = (size_t)(3 * f.nz * kZAny + f.nz) * sizeof(cplx_t<R>);
-  k_zsym_any<R><<<dim3((f.kx + kZAny - 1) / kZAny, f.ny), kZAnyThreads, sm, st>>>(Z, f.spec, f.ny, f.kx, f.kxp, sp);
+  k_zsym_any<R><<<z_tiles<R>(f.kx, f.ny), kZAnyThreads, sm, st>>>(Z, f.spec, f.ny, f.kx, f.kxp, sp);
 }
 
 // This file is compiled once per precision (-DICM_PLANE_PREC=32 or 64).

@@ -42,6 +42,36 @@ template <> __device__ __forceinline__ double recip<double>(double x) {
   return fma(y, fma(e, e, e), y);
 }
 
+// The lines of a z tile: kZLines wave numbers k0.. of one row.  In FP64, where rows are one wave number
+// longer than whole tiles (every nx = 16 m), the last wave number of kZLines rows makes a tile instead: one
+// of its own per row would be seven eighths idle, a ninth of the blocks at nx = 128.  z pass of 128^3, last
+// column alone / folded: FP64, bound by its operations, 424 / 375 us; FP32, bound by latency, which the
+// scattered column makes longer, 21.7 / 23.4 us (and 310 / 325 us on 512 x 384 x 256).
+constexpr int kZLines = 8;
+template <typename R>
+__host__ __device__ constexpr bool z_folds(int kx) { return sizeof(R) == 8 && kx % kZLines == 1 && kx > kZLines; }
+template <typename R>
+__host__ __device__ constexpr int z_tiles_x(int kx) { return z_folds<R>(kx) ? kx / kZLines : (kx + kZLines - 1) / kZLines; }
+template <typename R>
+__host__ __device__ constexpr int z_tiles(int kx, int ny) {
+  return z_tiles_x<R>(kx) * ny + (z_folds<R>(kx) ? (ny + kZLines - 1) / kZLines : 0);
+}
+template <typename R>
+struct ZTile {
+  int k0, row0;     // wave number and row of line 0
+  bool folded;      // lines are rows
+  __device__ __forceinline__ ZTile(int t, int kx, int ny) {
+    const int ntx = z_tiles_x<R>(kx), full = ntx * ny;
+    folded = sizeof(R) == 8 && t >= full;
+    row0 = folded ? (t - full) * kZLines : t / ntx;
+    k0 = folded ? kx - 1 : (t - row0 * ntx) * kZLines;
+  }
+  __device__ __forceinline__ int k(int line) const { return folded ? k0 : k0 + line; }
+  __device__ __forceinline__ int row(int line) const { return folded ? row0 + line : row0; }
+  __device__ __forceinline__ bool live(int line, int kx, int ny) const { return k(line) < kx && row(line) < ny; }
+  __device__ __forceinline__ size_t at(int line, int kxp) const { return (size_t)row(line) * kxp + k(line); }
+};
+
 // x > 0, in integer arithmetic for FP64 (and for what recip does not flush).
 __device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool positive(double x) { return __double2hiint(x) >= 0x00100000; }
