@@ -100,8 +100,13 @@ template <> struct BoxMuller<float> {
     // -2 ln u1 = -2 ln(2) log2(u1); the hardware log2 and reciprocal square root are
     // accurate to ~2^-22 relative, far inside the FP32 path's tolerance.  u1 may round
     // to 1, where the radius is 0: the floor keeps x * rsqrt(x) finite.
-    const float x = fmaxf(-1.38629436111989061f * __log2f(u1), 1e-30f);
-    const float rad = x * rsqrtf(x);
+    // Neither argument is subnormal, so the .ftz forms give the same values without the
+    // scaling around the others.
+    float l, y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(u1));
+    const float x = fmaxf(-1.38629436111989061f * l, 1e-30f);
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    const float rad = x * y;
     float s, c;
     __sincosf(6.28318530717958648f * u2, &s, &c);
     z0 = rad * c;

@@ -229,6 +229,51 @@ __device__ __forceinline__ void gen_own(RhsSmem<R>& sm, int slot, R (&z)[6], uin
   sm.z[slot][4][ly][lx] = z[5];
 }
 
+// The velocities around a cell that its right-hand side takes: component c at the cell and its six
+// neighbours, and x_xpym = v_x at (+x, -y) and so on.
+template <typename R>
+struct RhsStencil {
+  R c[3], xp[3], xm[3], yp[3], ym[3], zp[3], zm[3];
+  R x_xpym, x_xpzm, y_ypxm, y_ypzm, z_zpxm, z_zpym;
+};
+
+// Divergence of the momentum flux.  Products ut_a ut_b at the edges, ut_a = (v_a[e] + v_a[e-e_b])/2 and
+// ut_b = (v_b[e] + v_b[e-e_a])/2, and squared cell-centre averages, each without its factor 1/4 (in aq);
+// the difference of two squares as difference times sum, and every product inside a
+// multiply-add: 44 operations per cell where the plain sums take 57 (right-hand side of 128^3 with noise, both
+// launches: FP64 702 -> 685 us; FP32 45.7 -> 43.6, with the two planes per turn of the march's loop).
+template <typename R>
+__device__ __forceinline__ void advection(const RhsStencil<R>& q, R aq, R (&a)[3]) {
+  const R axy = q.c[0] + q.ym[0], bxy = q.c[1] + q.xm[1], axz = q.c[0] + q.zm[0], bxz = q.c[2] + q.xm[2];
+  const R exy = axy * bxy, eyz = (q.c[1] + q.zm[1]) * (q.c[2] + q.ym[2]);
+  const R sx = fma(axz, bxz, exy), sy = exy + eyz, sz = fma(axz, bxz, eyz);
+  const R tx = fma(R(2), q.c[0], q.xp[0] + q.xm[0]), dx = q.xp[0] - q.xm[0];
+  const R ty = fma(R(2), q.c[1], q.yp[1] + q.ym[1]), dy = q.yp[1] - q.ym[1];
+  const R tz = fma(R(2), q.c[2], q.zp[2] + q.zm[2]), dz = q.zp[2] - q.zm[2];
+  a[0] = aq * fma(dx, tx, fma(q.yp[0] + q.c[0], q.yp[1] + q.y_ypxm, fma(q.zp[0] + q.c[0], q.zp[2] + q.z_zpxm, -sx)));
+  a[1] = aq * fma(dy, ty, fma(q.xp[0] + q.x_xpym, q.xp[1] + q.c[1], fma(q.zp[1] + q.c[1], q.zp[2] + q.z_zpym, -sy)));
+  a[2] = aq * fma(dz, tz, fma(q.xp[0] + q.x_xpzm, q.xp[2] + q.c[2], fma(q.yp[1] + q.y_ypzm, q.yp[2] + q.c[2], -sz)));
+}
+
+// Advection and right-hand side of cell o: zd, ze are the differences of the diagonal and the off-diagonal
+// stress normals, ao the advection of the step before (unless this is the first).
+template <typename R, bool NOISE>
+__device__ __forceinline__ void rhs_out(const GridParams& g, const RhsStencil<R>& q, const R (&a)[3], const R (&zd)[3],
+                                        const R (&ze)[3], R (&ao)[3], bool hist, R* __restrict__ adv,
+                                        R* __restrict__ rhs, uint32_t o) {
+  const uint32_t nc = (uint32_t)g.ncell;
+  const R ce = rhs_c<R>(g).ce, cc = rhs_c<R>(g).cc, sd = rhs_c<R>(g).sd, so = rhs_c<R>(g).so;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    if (!hist) ao[c] = a[c];
+    const R nb = (q.xp[c] + q.xm[c]) + (q.yp[c] + q.ym[c]) + (q.zp[c] + q.zm[c]);
+    R s = fma(R(-1.5), a[c], R(0.5) * ao[c]);
+    if (NOISE) s = fma(sd, zd[c], fma(so, ze[c], s));
+    adv[o + c * nc] = a[c];
+    rhs[o + c * nc] = fma(cc, q.c[c], fma(ce, nb, s));
+  }
+}
+
 // Marching block of TX x TY cells.  A block takes a contiguous range of planes: with
 // g.kz > 0 the kz planes of one tile (grid = tiles x ceil(nz / kz)); with g.kz == 0 the
 // blocks are persistent (about two per SM) in groups of one block per tile of a tile
@@ -247,7 +292,6 @@ __device__ __forceinline__ void rhs_run(RhsSmem<R>& sm, const R* __restrict__ v,
   // offsets in 32 bits: 3 ncell <= 3 x 512^3 < 2^32
   const uint32_t nc = (uint32_t)g.ncell;
   const uint32_t plane = (uint32_t)g.nx * (uint32_t)g.ny;
-  const R ce = rhs_c<R>(g).ce, cc = rhs_c<R>(g).cc, aq = rhs_c<R>(g).aq, sd = rhs_c<R>(g).sd, so = rhs_c<R>(g).so;
   const int lx = tx + 1, ly = ty + 1;
   {
     const int i0 = (int)(tile % ntx) * TX, j0 = (int)(tile / ntx) * TY;
@@ -307,10 +351,13 @@ __device__ __forceinline__ void rhs_run(RhsSmem<R>& sm, const R* __restrict__ v,
       gen_own<R, RK>(sm, 1, zn, own + plane * (uint32_t)k0, k0, plane, g, step, lx, ly, next, nvalid);
       if (hnoise) gen_halo<R, RK>(sm, 1, ht, ncell + plane * (uint32_t)k0, plane, (k0 & 1) != 0, g, step);
     }
+    int zs = 1, zsn = 2;   // slots of the normals of planes k, k+1
+    // two planes per turn where normals are drawn: the registers that pass from plane to plane are renamed
+    // instead of copied (256^3: 269 -> 259 us with noise; without, 171 -> 188)
+#pragma unroll(NOISE ? 2 : 1)
     for (int k = k0; k < kend; ++k) {
       const int kk = k - k0;
       const int sp = kk % kRing, sc = (kk + 1) % kRing, sn = (kk + 2) % kRing;
-      const int zs = (kk + 1) % kZRing, zsn = (kk + 2) % kZRing;   // normals of planes k, k+1
       put(sn, vn, hq);                                         // plane k+1
       const uint32_t o = own + plane * (uint32_t)k;
       R ao[3] = {R(0), R(0), R(0)};
@@ -333,61 +380,32 @@ __device__ __forceinline__ void rhs_run(RhsSmem<R>& sm, const R* __restrict__ v,
         const auto P = sm.v[sp];
         const auto C = sm.v[sc];
         const auto N = sm.v[sn];
-        // component x
-        const R x_c = vc[0], x_xp = C[0][ly][lx + 1], x_xm = C[0][ly][lx - 1];
-        const R x_yp = C[0][ly + 1][lx], x_ym = C[0][ly - 1][lx], x_zp = vn[0], x_zm = vp[0];
-        const R x_xpym = C[0][ly - 1][lx + 1], x_xpzm = P[0][ly][lx + 1];
-        // component y
-        const R y_c = vc[1], y_xp = C[1][ly][lx + 1], y_xm = C[1][ly][lx - 1];
-        const R y_yp = C[1][ly + 1][lx], y_ym = C[1][ly - 1][lx], y_zp = vn[1], y_zm = vp[1];
-        const R y_ypxm = C[1][ly + 1][lx - 1], y_ypzm = P[1][ly + 1][lx];
-        // component z
-        const R z_c = vc[2], z_xp = C[2][ly][lx + 1], z_xm = C[2][ly][lx - 1];
-        const R z_yp = C[2][ly + 1][lx], z_ym = C[2][ly - 1][lx], z_zp = vn[2], z_zm = vp[2];
-        const R z_zpxm = N[2][ly][lx - 1], z_zpym = N[2][ly - 1][lx];
-
-        // edge products ut_a ut_b at edge index e, ut_a = (v_a[e] + v_a[e-e_b])/2 and
-        // ut_b = (v_b[e] + v_b[e-e_a])/2, and the squared cell-centre averages, each
-        // without its factor 1/4 (in aq)
-        const R exy_c = (x_c + x_ym) * (y_c + y_xm);
-        const R exy_yp = (x_yp + x_c) * (y_yp + y_ypxm);
-        const R exy_xp = (x_xp + x_xpym) * (y_xp + y_c);
-        const R exz_c = (x_c + x_zm) * (z_c + z_xm);
-        const R exz_zp = (x_zp + x_c) * (z_zp + z_zpxm);
-        const R exz_xp = (x_xp + x_xpzm) * (z_xp + z_c);
-        const R eyz_c = (y_c + y_zm) * (z_c + z_ym);
-        const R eyz_zp = (y_zp + y_c) * (z_zp + z_zpym);
-        const R eyz_yp = (y_yp + y_ypzm) * (z_yp + z_c);
-        const R ubx_c = x_xp + x_c, ubx_m = x_c + x_xm;
-        const R uby_c = y_yp + y_c, uby_m = y_c + y_ym;
-        const R ubz_c = z_zp + z_c, ubz_m = z_c + z_zm;
-        const R ax = aq * (ubx_c * ubx_c - ubx_m * ubx_m + exy_yp - exy_c + exz_zp - exz_c);
-        const R ay = aq * (uby_c * uby_c - uby_m * uby_m + exy_xp - exy_c + eyz_zp - eyz_c);
-        const R az = aq * (ubz_c * ubz_c - ubz_m * ubz_m + exz_xp - exz_c + eyz_yp - eyz_c);
-        const R nbx = x_xp + x_xm + x_yp + x_ym + x_zp + x_zm;
-        const R nby = y_xp + y_xm + y_yp + y_ym + y_zp + y_zm;
-        const R nbz = z_xp + z_xm + z_yp + z_ym + z_zp + z_zm;
-        R fx = R(0), fy = R(0), fz = R(0);
+        RhsStencil<R> q;
+        q.c[0] = vc[0]; q.c[1] = vc[1]; q.c[2] = vc[2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          q.xp[c] = C[c][ly][lx + 1]; q.xm[c] = C[c][ly][lx - 1];
+          q.yp[c] = C[c][ly + 1][lx]; q.ym[c] = C[c][ly - 1][lx];
+          q.zp[c] = vn[c]; q.zm[c] = vp[c];
+        }
+        q.x_xpym = C[0][ly - 1][lx + 1]; q.x_xpzm = P[0][ly][lx + 1];
+        q.y_ypxm = C[1][ly + 1][lx - 1]; q.y_ypzm = P[1][ly + 1][lx];
+        q.z_zpxm = N[2][ly][lx - 1]; q.z_zpym = N[2][ly - 1][lx];
+        R zd[3], ze[3];
         if (NOISE) {
           const auto Z = sm.z[zs];   // plane k: [0] xx, [1] yy, [2] xy, [3] xz, [4] yz
           // divergence of the stress at the faces: Sigma_aa at cells, Sigma_ab on edges
-          fx = sd * (zc[0] - Z[0][ly][lx - 1]) + so * (Z[2][ly + 1][lx] - zc[3]) + so * (zn[4] - zc[4]);
-          fy = sd * (zc[1] - Z[1][ly - 1][lx]) + so * (Z[2][ly][lx + 1] - zc[3]) + so * (zn[5] - zc[5]);
-          fz = sd * (zc[2] - zzp) + so * (Z[3][ly][lx + 1] - zc[4]) + so * (Z[4][ly + 1][lx] - zc[5]);
+          zd[0] = zc[0] - Z[0][ly][lx - 1]; ze[0] = (Z[2][ly + 1][lx] - zc[3]) + (zn[4] - zc[4]);
+          zd[1] = zc[1] - Z[1][ly - 1][lx]; ze[1] = (Z[2][ly][lx + 1] - zc[3]) + (zn[5] - zc[5]);
+          zd[2] = zc[2] - zzp; ze[2] = (Z[3][ly][lx + 1] - zc[4]) + (Z[4][ly + 1][lx] - zc[5]);
         }
-        if (!hist) {
-          ao[0] = ax;
-          ao[1] = ay;
-          ao[2] = az;
-        }
-        adv[o] = ax;
-        adv[o + nc] = ay;
-        adv[o + 2 * nc] = az;
-        rhs[o] = cc * x_c + ce * nbx + fx - (R(1.5) * ax - R(0.5) * ao[0]);
-        rhs[o + nc] = cc * y_c + ce * nby + fy - (R(1.5) * ay - R(0.5) * ao[1]);
-        rhs[o + 2 * nc] = cc * z_c + ce * nbz + fz - (R(1.5) * az - R(0.5) * ao[2]);
+        R a[3];
+        advection<R>(q, rhs_c<R>(g).aq, a);
+        rhs_out<R, NOISE>(g, q, a, zd, ze, ao, hist, adv, rhs, o);
       }
       if (NOISE) zzp = zc[2];
+      zs = zsn;
+      zsn = zsn == kZRing - 1 ? 0 : zsn + 1;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         vp[c] = vc[c];
@@ -482,9 +500,9 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 2 : 1) k_rhs_batch(const 
 //    normals twice, for halos;
 //  * in FP32, up to kFlatCells: what the march saves (48 bytes per cell of stored normals)
 //    only pays where every SM marches many planes.
-// Measured with noise, both launches (us), march against stored normals: FP32 19.0 / 11.0 on
-// 32^3, 29.8 / 15.1 on 64^3, 29.9 / 25.3 on 96^3, 45.3 / 56.3 on 128^3, 275 / 386 on 256^3;
-// FP64 449 / 24 on 32^3 (eight marching blocks) and 1422 / 702 on 128^3, where half of the
+// Measured with noise, both launches (us), march against stored normals: FP32 19.0 / 10.5 on
+// 32^3, 29.8 / 15.1 on 64^3, 29.9 / 25.4 on 96^3, 43.6 / 56.3 on 128^3, 259 / 386 on 256^3;
+// FP64 449 / 24 on 32^3 (eight marching blocks) and 1422 / 685 on 128^3, where half of the
 // gain is the cheaper normals above.
 // ---------------------------------------------------------------------------
 constexpr int kFlatThreads = 128;
@@ -536,7 +554,6 @@ __device__ __forceinline__ void rhs_cell(const GridParams& g, uint32_t o, bool h
   const auto above = [&](uint32_t c) { return kl ? c - sz : c + plane; };
   const auto below = [&](uint32_t c) { return kf ? c + sz : c - plane; };
   const uint32_t yp = up(o), ym = down(o), zp = above(o), zm = below(o);
-  const R ce = rhs_c<R>(g).ce, cc = rhs_c<R>(g).cc, aq = rhs_c<R>(g).aq;
   R ao[3] = {R(0), R(0), R(0)};
   if (hist) {
     ao[0] = adv[o];
@@ -544,46 +561,32 @@ __device__ __forceinline__ void rhs_cell(const GridParams& g, uint32_t o, bool h
     ao[2] = adv[o + 2 * nc];
   }
   const R *vx = v, *vy = v + nc, *vz = v + 2 * (size_t)nc;
-  const R x_c = vx[o], x_xp = vx[xp], x_xm = vx[xm], x_yp = vx[yp], x_ym = vx[ym], x_zp = vx[zp], x_zm = vx[zm];
-  const R y_c = vy[o], y_xp = vy[xp], y_xm = vy[xm], y_yp = vy[yp], y_ym = vy[ym], y_zp = vy[zp], y_zm = vy[zm];
-  const R z_c = vz[o], z_xp = vz[xp], z_xm = vz[xm], z_yp = vz[yp], z_ym = vz[ym], z_zp = vz[zp], z_zm = vz[zm];
-  R a[3] = {R(0), R(0), R(0)};
-  if (g.advection) {
-    const R x_xpym = vx[down(xp)], x_xpzm = vx[below(xp)], y_ypxm = vy[up(xm)], y_ypzm = vy[below(yp)];
-    const R z_zpxm = vz[above(xm)], z_zpym = vz[above(ym)];
-    const R exy_c = (x_c + x_ym) * (y_c + y_xm), exz_c = (x_c + x_zm) * (z_c + z_xm), eyz_c = (y_c + y_zm) * (z_c + z_ym);
-    const R ubx_c = x_xp + x_c, ubx_m = x_c + x_xm, uby_c = y_yp + y_c, uby_m = y_c + y_ym;
-    const R ubz_c = z_zp + z_c, ubz_m = z_c + z_zm;
-    // differences of products: (ubx_c^2 - ubx_m^2) + (exy(+y) - exy) + (exz(+z) - exz), ...
-    a[0] = aq * (fma(ubx_c, ubx_c, -ubx_m * ubx_m) + fma(x_yp + x_c, y_yp + y_ypxm, -exy_c) +
-                 fma(x_zp + x_c, z_zp + z_zpxm, -exz_c));
-    a[1] = aq * (fma(uby_c, uby_c, -uby_m * uby_m) + fma(x_xp + x_xpym, y_xp + y_c, -exy_c) +
-                 fma(y_zp + y_c, z_zp + z_zpym, -eyz_c));
-    a[2] = aq * (fma(ubz_c, ubz_c, -ubz_m * ubz_m) + fma(x_xp + x_xpzm, z_xp + z_c, -exz_c) +
-                 fma(y_yp + y_ypzm, z_yp + z_c, -eyz_c));
+  RhsStencil<R> q;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const R* u = v + c * (size_t)nc;
+    q.c[c] = u[o];
+    q.xp[c] = u[xp]; q.xm[c] = u[xm];
+    q.yp[c] = u[yp]; q.ym[c] = u[ym];
+    q.zp[c] = u[zp]; q.zm[c] = u[zm];
   }
-  R f[3] = {R(0), R(0), R(0)};
+  // every load before the first branch, so that all are in flight together
+  const bool adv_on = g.advection != 0;
+  q.x_xpym = adv_on ? vx[down(xp)] : R(0); q.x_xpzm = adv_on ? vx[below(xp)] : R(0);
+  q.y_ypxm = adv_on ? vy[up(xm)] : R(0); q.y_ypzm = adv_on ? vy[below(yp)] : R(0);
+  q.z_zpxm = adv_on ? vz[above(xm)] : R(0); q.z_zpym = adv_on ? vz[above(ym)] : R(0);
+  R zd[3], ze[3];
   if (NOISE) {
-    const R sd = rhs_c<R>(g).sd, so = rhs_c<R>(g).so;
     const R *zxx = z, *zyy = z + nc, *zzz = z + 2 * (size_t)nc, *zxy = z + 3 * (size_t)nc, *zxz = z + 4 * (size_t)nc,
             *zyz = z + 5 * (size_t)nc;
     const R xy = zxy[o], xz = zxz[o], yz = zyz[o];
-    f[0] = fma(sd, zxx[o] - zxx[xm], so * ((zxy[yp] - xy) + (zxz[zp] - xz)));
-    f[1] = fma(sd, zyy[o] - zyy[ym], so * ((zxy[xp] - xy) + (zyz[zp] - yz)));
-    f[2] = fma(sd, zzz[o] - zzz[zm], so * ((zxz[xp] - xz) + (zyz[yp] - yz)));
+    zd[0] = zxx[o] - zxx[xm]; ze[0] = (zxy[yp] - xy) + (zxz[zp] - xz);
+    zd[1] = zyy[o] - zyy[ym]; ze[1] = (zxy[xp] - xy) + (zyz[zp] - yz);
+    zd[2] = zzz[o] - zzz[zm]; ze[2] = (zxz[xp] - xz) + (zyz[yp] - yz);
   }
-  if (!hist) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) ao[c] = a[c];
-  }
-  const R nb[3] = {x_xp + x_xm + x_yp + x_ym + x_zp + x_zm, y_xp + y_xm + y_yp + y_ym + y_zp + y_zm,
-                   z_xp + z_xm + z_yp + z_ym + z_zp + z_zm};
-  const R own[3] = {x_c, y_c, z_c};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    adv[o + c * nc] = a[c];
-    rhs[o + c * nc] = fma(cc, own[c], fma(ce, nb[c], fma(R(0.5), ao[c], fma(R(-1.5), a[c], f[c]))));
-  }
+  R a[3] = {R(0), R(0), R(0)};
+  if (adv_on) advection<R>(q, rhs_c<R>(g).aq, a);
+  rhs_out<R, NOISE>(g, q, a, zd, ze, ao, hist, adv, rhs, o);
 }
 
 template <typename R>
