@@ -251,15 +251,22 @@ template <typename R, int N> constexpr int xf2_min_blocks() { return sizeof(R) =
 template <typename R, int N, int R2> constexpr int x_plain_lines() {
   return sizeof(R) != 4 || N > 128 ? kXLines : (kThreads / R2 >= 64 ? 64 : 32);
 }
-// The inverse x pass of FP32 sides up to 256 runs lean at four blocks per SM: its
-// spectrum loads go in two batches, the old values of the adding modes are loaded
-// just before the output, and 128 records are staged.  Otherwise (and for the
-// two-output mode, which would spill) all loads are in flight at once and one record
-// per thread is staged.
+// The inverse x pass of FP32 runs lean: its spectrum loads go in batches, the old values of
+// the adding modes are loaded just before the output, and 128 records or fewer are staged.
+// Otherwise (and for the two-output mode, which would spill) all loads are in flight at once
+// and one record per thread is staged.
 template <typename R, int N, int MODE> constexpr bool xi2_lean() {
   return sizeof(R) == 4 && MODE != OUT_ADD_AND_STORE2;
 }
-template <typename R, int N, int MODE> constexpr int xi2_stage() { return xi2_lean<R, N, MODE>() ? 128 : kThreads; }
+// Blocks per SM: four up to 256; above, three where nothing is added (sixteen lines of 512 leave three
+// blocks room for 32 records each), two with the old values to hold (512 x 384 x 256, two / three blocks: store
+// 289 / 275 us, gather only 226 / 199, add 364 / 419).
+template <typename R, int N, int MODE> constexpr int xi2_min_blocks() {
+  return !xi2_lean<R, N, MODE>() ? 1 : N <= 256 ? 4 : MODE == OUT_ADD ? 2 : 3;
+}
+template <typename R, int N, int MODE> constexpr int xi2_stage() {
+  return !xi2_lean<R, N, MODE>() ? kThreads : xi2_min_blocks<R, N, MODE>() == 3 ? 32 : 128;
+}
 
 // The z pass holds all three components of its tile, so it takes 8 kx lines
 // (64-byte rows in FP32) to keep two blocks per SM; one thread per first-stage item
@@ -590,6 +597,10 @@ constexpr int y_threads() {
   return sizeof(R) == 4 || items > kThreads ? kThreads : items < 64 ? 64 : items;
 }
 
+// FP32 sides above 256: registers capped so that three blocks share an SM instead of two, 80 instead of 84 to
+// 116 (512 x 384 x 256, y forward / inverse: 242 / 235 us with two, 188 / 227 with three).  0: no floor.
+template <typename R, int N> constexpr int y_min_blocks() { return sizeof(R) == 4 && N > 256 ? 3 : 0; }
+
 // The columns of the y pass go in tiles of seg_lines.  In FP64, where rows are one column longer than whole
 // tiles, the last column of as many planes as a tile has lines makes a tile of its own (see ZTile; y pass of
 // 128^3 146 / 135 us; FP32 on 512 x 384 x 256, bound by memory, 272 / 280).
@@ -599,7 +610,7 @@ __host__ __device__ constexpr bool y_folds(int kx) {
 }
 
 template <typename R, int N, int R1, int R2, bool INV>
-__global__ void __launch_bounds__(y_threads<R, N, R2>()) k_ypass2(cplx_t<R>* __restrict__ spec, const cplx_t<R>* __restrict__ gtw,
+__global__ void __launch_bounds__(y_threads<R, N, R2>(), y_min_blocks<R, N>()) k_ypass2(cplx_t<R>* __restrict__ spec, const cplx_t<R>* __restrict__ gtw,
                                                      int nz, int kx, int kxp, const RepFft* __restrict__ reps) {
   using C = cplx_t<R>;
   constexpr int NL = seg_lines<R>();
@@ -919,7 +930,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_xyf(const float* __restrict__ s
 // (without 1/h^2) to rb.acc_lap.  x stays in shared memory for the gathers.
 // GRP: a group solve whose replicas gather into their own accumulators (reps[i].rb).
 template <typename R, int N, int R1, int R2, int MODE, int GATHER, bool GRP = false>
-__global__ void __launch_bounds__(kThreads, xi2_lean<R, N, MODE>() ? (N <= 256 ? 4 : 2) : 1) k_xinv2(const cplx_t<R>* __restrict__ spec, R* __restrict__ dst,
+__global__ void __launch_bounds__(kThreads, xi2_min_blocks<R, N, MODE>()) k_xinv2(const cplx_t<R>* __restrict__ spec, R* __restrict__ dst,
                                                     R* __restrict__ dst2, const cplx_t<R>* __restrict__ gtw,
                                                     int nrows, long long ncell, int kxp, RowBlobs rb0,
                                                     const RepFft* __restrict__ reps) {

@@ -264,25 +264,26 @@ template <typename R> struct SDft<R, 2> {
     a[1] = csub(t, a[1]);
   }
 };
+// Differences that are used after a quarter turn are formed turned, -i (a - b), component by component, so
+// that the additions they enter are whole complex ones.
+template <typename C> __device__ __forceinline__ C csub_mi(C a, C b) { return mk(a.y - b.y, b.x - a.x); }
 template <typename R> struct SDft<R, 3> {
   __device__ __forceinline__ static void run(cplx_t<R>* a) {
     const R s = R(0.86602540378443864676);
-    const cplx_t<R> t1 = cadd(a[1], a[2]);
-    const cplx_t<R> t2 = mk(a[0].x - R(0.5) * t1.x, a[0].y - R(0.5) * t1.y);
-    const cplx_t<R> d = csub(a[1], a[2]);
-    const cplx_t<R> t3 = mk(s * d.x, s * d.y);
+    const cplx_t<R> t1 = cadd(a[1], a[2]), e = csub_mi(a[1], a[2]);
+    const cplx_t<R> t2 = cfmar<R>(R(-0.5), t1, a[0]);
     a[0] = cadd(a[0], t1);
-    a[1] = cadd(t2, cmul_mi(t3));
-    a[2] = cadd(t2, cmul_pi(t3));
+    a[1] = cfmar<R>(s, e, t2);
+    a[2] = cfmar<R>(-s, e, t2);
   }
 };
 template <typename R> struct SDft<R, 4> {
   __device__ __forceinline__ static void run(cplx_t<R>* a) {
-    const cplx_t<R> s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]), s13 = cadd(a[1], a[3]), d13 = csub(a[1], a[3]);
+    const cplx_t<R> s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]), s13 = cadd(a[1], a[3]), e13 = csub_mi(a[1], a[3]);
     a[0] = cadd(s02, s13);
     a[2] = csub(s02, s13);
-    a[1] = cadd(d02, cmul_mi(d13));
-    a[3] = cadd(d02, cmul_pi(d13));
+    a[1] = cadd(d02, e13);
+    a[3] = csub(d02, e13);
   }
 };
 // 9 = 3 x 3 with W_9^(n1 k2), n1 k2 in {1, 2, 4} (cos and sin of 40, 80 and 160 degrees).
@@ -312,21 +313,21 @@ template <typename R> struct SDft<R, 9> {
   }
 };
 template <typename R> struct SDft<R, 6> : SDftComp<R, 2, 3> {};
-// DFT_4 of u_0, W_8 u_1, -i u_2, W_8^3 u_3.  The factor sqrt(1/2) common to the two eighth turns rides
+// DFT_4 of u_0, W_8 u_1, e_2 = -i u_2, W_8^3 u_3.  The factor sqrt(1/2) common to the two eighth turns rides
 // on the last additions as a fused multiply-add: 20 operations where rotating first takes 24.  The FP64
-// passes are bound by their operations; with this, the inverses by exchange and the spectra kept doubled,
+// passes are bound by their operations; with this, inverses free of negations and the spectra kept doubled,
 // x / y / z / y / x of the 128^3 solve take 148 / 146 / 424 / 145 / 164 us (165 / 153 / 451 / 153 / 180 before).
 template <typename R>
-__device__ __forceinline__ void eighth_column(cplx_t<R> u0, cplx_t<R> u1, cplx_t<R> u2, cplx_t<R> u3, cplx_t<R>& o0,
+__device__ __forceinline__ void eighth_column(cplx_t<R> u0, cplx_t<R> u1, cplx_t<R> e2, cplx_t<R> u3, cplx_t<R>& o0,
                                               cplx_t<R>& o1, cplx_t<R>& o2, cplx_t<R>& o3) {
   const R r = R(0.70710678118654752440);
-  const cplx_t<R> s = mk(u0.x + u2.y, u0.y - u2.x), d = mk(u0.x - u2.y, u0.y + u2.x);
+  const cplx_t<R> s = cadd(u0, e2), d = csub(u0, e2);
   const R px = u1.x + u1.y, py = u1.y - u1.x, qx = u3.y - u3.x, qy = u3.x + u3.y;
-  const R sx = px + qx, sy = py - qy, dx = px - qx, dy = py + qy;
-  o0 = mk(fma(r, sx, s.x), fma(r, sy, s.y));
-  o2 = mk(fma(-r, sx, s.x), fma(-r, sy, s.y));
-  o1 = mk(fma(r, dy, d.x), fma(-r, dx, d.y));
-  o3 = mk(fma(-r, dy, d.x), fma(r, dx, d.y));
+  const cplx_t<R> p = mk(px + qx, py - qy), m = mk(py + qy, qx - px);
+  o0 = cfmar<R>(r, p, s);
+  o2 = cfmar<R>(-r, p, s);
+  o1 = cfmar<R>(r, m, d);
+  o3 = cfmar<R>(-r, m, d);
 }
 template <typename R> struct SDft<R, 8> {
   // 8 = 2 x 4: even outputs DFT_4 of the sums, odd ones the eighth-turn column of the differences
@@ -335,7 +336,7 @@ template <typename R> struct SDft<R, 8> {
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
       b[n] = cadd(a[n], a[n + 4]);
-      u[n] = csub(a[n], a[n + 4]);
+      u[n] = n == 2 ? csub_mi(a[n], a[n + 4]) : csub(a[n], a[n + 4]);
     }
     SDft<R, 4>::run(b);
 #pragma unroll
@@ -360,18 +361,18 @@ template <typename R> struct SDft<R, 16> {
 #pragma unroll
       for (int k = 0; k < 4; ++k) a[4 * k] = z[k];
     }
-    eighth_column<R>(y[0][2], y[1][2], y[2][2], y[3][2], a[2], a[6], a[10], a[14]);
+    eighth_column<R>(y[0][2], y[1][2], cmul_mi(y[2][2]), y[3][2], a[2], a[6], a[10], a[14]);
 #pragma unroll
     for (int k2 = 1; k2 <= 3; k2 += 2) {   // W^2 or W^6 on the third input: its sqrt(1/2) in the sums too
       const cplx_t<R> z1 = mulw96<R>(y[1][k2], 6 * k2), z3 = mulw96<R>(y[3][k2], (18 * k2) % 96);
       const cplx_t<R> u = y[2][k2], z0 = y[0][k2];
-      const R px = k2 == 1 ? u.x + u.y : u.y - u.x, py = k2 == 1 ? u.y - u.x : -u.x - u.y;
-      const cplx_t<R> s = mk(fma(r, px, z0.x), fma(r, py, z0.y)), d = mk(fma(-r, px, z0.x), fma(-r, py, z0.y));
-      const cplx_t<R> t = cadd(z1, z3), e = csub(z1, z3);
+      const cplx_t<R> p = k2 == 1 ? mk(u.x + u.y, u.y - u.x) : mk(u.y - u.x, -u.x - u.y);
+      const cplx_t<R> s = cfmar<R>(r, p, z0), d = cfmar<R>(-r, p, z0);
+      const cplx_t<R> t = cadd(z1, z3), e = csub_mi(z1, z3);
       a[k2] = cadd(s, t);
       a[8 + k2] = csub(s, t);
-      a[4 + k2] = cadd(d, cmul_mi(e));
-      a[12 + k2] = cadd(d, cmul_pi(e));
+      a[4 + k2] = cadd(d, e);
+      a[12 + k2] = csub(d, e);
     }
   }
 };
@@ -379,15 +380,17 @@ template <typename R> struct SDft<R, 12> : SDftComp<R, 4, 3> {};
 template <typename R> struct SDft<R, 24> : SDftComp<R, 8, 3> {};
 template <typename R> struct SDft<R, 32> : SDftComp<R, 4, 8> {};
 
-// Inverse (unnormalised) small DFT: exchanging real and imaginary parts before and after the
-// forward one conjugates its roots, and costs nothing (negations are FP64 operations).
+// Inverse (unnormalised) small DFT: the forward one with its outputs in reverse order, which costs
+// nothing.
 template <typename R, int M>
 __device__ __forceinline__ void sdft_inv(cplx_t<R>* a) {
-#pragma unroll
-  for (int i = 0; i < M; ++i) a[i] = mk(a[i].y, a[i].x);
   SDft<R, M>::run(a);
 #pragma unroll
-  for (int i = 0; i < M; ++i) a[i] = mk(a[i].y, a[i].x);
+  for (int i = 1; 2 * i < M; ++i) {
+    const cplx_t<R> t = a[i];
+    a[i] = a[M - i];
+    a[M - i] = t;
+  }
 }
 
 // First-stage twiddles laid out as tw2[k2 * R2 + n1] = W_N^(n1 k2) (N entries), so
