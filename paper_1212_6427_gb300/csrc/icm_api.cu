@@ -331,18 +331,41 @@ WcaParams wca_params(const icm_sim* s) {
   return w;
 }
 
+// Sines and cosines of the axis tables, once per different side of a simulation: long double is done in
+// software on some hosts, and half of the circle gives the other half.
+struct AxisTrig {
+  int n = 0;
+  std::vector<long double> c, s, h;   // cos, sin of 2 pi m / n and sin of pi m / n, m = 0 .. n/2
+  void make(int side) {
+    if (side == n) return;
+    n = side;
+    c.resize(n / 2 + 1);
+    s.resize(n / 2 + 1);
+    h.resize(n / 2 + 1);
+    const long double pi = 3.141592653589793238462643383279502884L;
+    for (int m = 0; m <= n / 2; ++m) {
+      const long double th = 2.0L * pi * (long double)m / (long double)n;
+      c[m] = cosl(th);
+      s[m] = sinl(th);
+      h[m] = sinl(0.5L * th);
+    }
+  }
+  long double cos_of(int m) const { return c[2 * m <= n ? m : n - m]; }
+  long double sin_of(int m) const { return 2 * m <= n ? s[m] : -s[n - m]; }
+  long double half_sin_of(int m) const { return h[2 * m <= n ? m : n - m]; }
+};
+
 // Build one axis plan: radices, twiddles (long double), digit-reversed order, and
 // the symbol d = (exp(i theta) - 1)/h, |d|^2 = 4 sin^2(theta/2)/h^2 by storage position
 // (x: by natural wavenumber, only nx/2+1 of them).
-icm_status build_axis(icm_sim* s, int n, bool natural, int count, AxisPlan& P, void*& dtab, void*& ddtab,
-                      bool z_alt = false) {
+icm_status build_axis(icm_sim* s, AxisTrig& trig, int n, bool natural, int count, AxisPlan& P, void*& dtab,
+                      void*& ddtab, bool z_alt = false) {
   int r1 = 0, r2 = 0;
   const bool two = z_alt ? fft_split_z_alt(n, r1, r2) : fft_split(n, r1, r2);
   const std::vector<int> rad = two ? std::vector<int>{r1, r2} : factor_radices(n);
   P.n = n;
   P.nstages = (int)rad.size();
   for (size_t i = 0; i < rad.size(); ++i) P.radix[i] = rad[i];
-  const long double pi = 3.141592653589793238462643383279502884L;
   std::vector<int> pof(n), fop(n);
   for (int k = 0; k < n; ++k) {
     int pos = 0, M = n, rem = k;
@@ -365,18 +388,17 @@ icm_status build_axis(icm_sim* s, int n, bool natural, int count, AxisPlan& P, v
       memcpy(&buf[idx * 8], &x, 8);
     }
   };
+  trig.make(n);
   for (int m = 0; m < n; ++m) {
-    const long double th = 2.0L * pi * (long double)m / (long double)n;
-    put(tw, 2 * m, cosl(th));
-    put(tw, 2 * m + 1, -sinl(th));
+    put(tw, 2 * m, trig.cos_of(m));
+    put(tw, 2 * m + 1, -trig.sin_of(m));
   }
   for (int i = 0; i < count; ++i) {
     const int k = natural ? i : fop[i];
-    const long double th = 2.0L * pi * (long double)k / (long double)n;
     const long double h = s->h;
-    put(dt, 2 * i, (cosl(th) - 1.0L) / h);
-    put(dt, 2 * i + 1, sinl(th) / h);
-    const long double sn = sinl(0.5L * th);
+    put(dt, 2 * i, (trig.cos_of(k) - 1.0L) / h);
+    put(dt, 2 * i + 1, trig.sin_of(k) / h);
+    const long double sn = trig.half_sin_of(k);
     put(dd, i, 4.0L * sn * sn / (h * h));
   }
   void* dtw = dalloc(s, tw.size());
@@ -1057,8 +1079,8 @@ icm_status icm_create(const int32_t grid[3], double h, double rho, double eta, d
     icm_destroy(s);
     return fail(ICM_ECUDA, "creation of the auxiliary stream failed");
   }
-  fft_prepare();
-  if (!grid_prepare(s->stream)) {
+  const bool fresh = !fft_prepare();   // the first simulation of this context
+  if (!grid_prepare(s->stream, fresh)) {
     cudaGetLastError();
     icm_destroy(s);
     return fail(ICM_ECUDA, "upload of the noise tables failed");
@@ -1084,9 +1106,10 @@ icm_status icm_create(const int32_t grid[3], double h, double rho, double eta, d
     return fail(ICM_ENOMEM, "device allocation of %.1f MB of grid state failed", (4.0 * fbytes) / 1e6);
   }
   icm_status st = ICM_OK;
-  if ((st = build_axis(s, s->nx, true, s->kx, s->px, s->dx, s->ddx)) != ICM_OK ||
-      (st = build_axis(s, s->ny, false, s->ny, s->py, s->dy, s->ddy)) != ICM_OK ||
-      (st = build_axis(s, s->nz, false, s->nz, s->pz, s->dz, s->ddz)) != ICM_OK) {
+  AxisTrig trig;
+  if ((st = build_axis(s, trig, s->nx, true, s->kx, s->px, s->dx, s->ddx)) != ICM_OK ||
+      (st = build_axis(s, trig, s->ny, false, s->ny, s->py, s->dy, s->ddy)) != ICM_OK ||
+      (st = build_axis(s, trig, s->nz, false, s->nz, s->pz, s->dz, s->ddz)) != ICM_OK) {
     const std::string msg = g_err;
     icm_destroy(s);
     return fail(st, "%s", msg.c_str());
@@ -1095,7 +1118,7 @@ icm_status icm_create(const int32_t grid[3], double h, double rho, double eta, d
     int r1 = 0, r2 = 0;
     s->has_zalt = fft_split_z_alt(s->nz, r1, r2);
   }
-  if (s->has_zalt && (st = build_axis(s, s->nz, false, s->nz, s->pz_alt, s->dz_alt, s->ddz_alt, true)) != ICM_OK) {
+  if (s->has_zalt && (st = build_axis(s, trig, s->nz, false, s->nz, s->pz_alt, s->dz_alt, s->ddz_alt, true)) != ICM_OK) {
     const std::string msg = g_err;
     icm_destroy(s);
     return fail(st, "%s", msg.c_str());

@@ -1716,7 +1716,8 @@ ICM_INST_XI(double, extern)
 #endif
 
 #if ICM_SHARD(0)
-void fft_prepare() {
+bool fft_prepare() {
+  if (plane_prepared()) return true;
   fft_prepare_xf<float>();
   fft_prepare_yz<float>();
   fft_prepare_xi<float>();
@@ -1724,7 +1725,8 @@ void fft_prepare() {
   fft_prepare_yz<double>();
   fft_prepare_xi<double>();
   plane_prepare<float>();
-  plane_prepare<double>();
+  plane_prepare<double>();   // last: plane_prepared looks for it
+  return false;
 }
 
 template void spectral_solve<float>(const FftCtx<float>&, const float*, float*, float*, int, double, double,

@@ -914,12 +914,13 @@ struct NormalTables {
 };
 }  // namespace
 
-bool grid_prepare(cudaStream_t st) {
+bool grid_prepare(cudaStream_t st, bool fresh) {
   cudaFuncSetAttribute(k_rhs<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<float>());
   cudaFuncSetAttribute(k_rhs<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<float>());
   cudaFuncSetAttribute(k_rhs_batch<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<float>());
   cudaFuncSetAttribute(k_rhs_batch<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rhs_smem<float>());
   const int dev = current_device();
+  if (fresh && dev >= 0) g_tables_ready[dev].store(false);   // a context after a device reset has none
   if (dev >= 0 && g_tables_ready[dev].load()) return true;
   static const NormalTables tables;   // outlives the copies below
   return cudaMemcpyToSymbolAsync(g_log_tab, tables.log_tab, sizeof(tables.log_tab), 0, cudaMemcpyHostToDevice, st) ==

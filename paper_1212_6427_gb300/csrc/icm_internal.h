@@ -150,11 +150,12 @@ void debug_wait_timeout(int* err, long long limit_ns, cudaStream_t st);
 // per chain, the second of two launches timed with CUDA events on st.  -1 on error.
 double fma_rate(int precision, int iters, int blocks_per_sm, cudaStream_t st, double* seconds);
 
-// Raise the dynamic shared-memory limits of the kernels (call once, outside capture).
-void fft_prepare();
-// (grid_prepare also queues the upload of the FP64 Box-Muller tables on st, once per device;
-// false if that fails.  grid_ready records that it has landed.)
-bool grid_prepare(cudaStream_t st);
+// Raise the dynamic shared-memory limits of the kernels (outside capture).  fft_prepare's some 300
+// calls are made once per context: true if they had been.
+bool fft_prepare();
+// (grid_prepare also queues the upload of the FP64 Box-Muller tables on st, once per device and
+// for the first simulation of a context; false if that fails.  grid_ready records that it has landed.)
+bool grid_prepare(cudaStream_t st, bool fresh);
 void grid_ready();
 
 // ---------------------------------------------------------------------------
@@ -374,6 +375,7 @@ __device__ __forceinline__ double plane_sum(const double* __restrict__ part, lon
 // Whether a grid's planes fit in shared memory (and are worth it).
 bool plane_has_passes(int precision, int nx, int ny, int nz);
 template <typename R> void plane_prepare();
+bool plane_prepared();
 // The spectrum fft_x_forward + fft_y leave, with the blobs' spread (pb, or null); src may be null
 // with blobs.  reps: the G replicas of a group solve (no blobs), or null.
 template <typename R>

@@ -885,6 +885,16 @@ void plane_prepare() {
 #undef ICM_ATTR
 }
 
+#if ICM_PLANE_PREC == 64
+// Whether this context has the attributes of fft_prepare, whose last call is the one above for FP64.
+bool plane_prepared() {
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, k_zsym_any<double>) == cudaSuccess) return a.maxDynamicSharedSizeBytes == 226 * 1024;
+  cudaGetLastError();
+  return false;
+}
+#endif
+
 template <typename R>
 void plane_forward(const FftCtx<R>& f, const R* src, const PlaneBlobs* pb, const RepFft* reps, int G, cudaStream_t st) {
   const PlaneArgs A = plane_args(f);
