@@ -139,8 +139,10 @@ icm_status icm_set_blob_wca(icm_sim* sim, double epsilon, double sigma);
  * result beyond rounding (no counterpart in the paper).  Defaults: every choice on
  * except fused_xy, rhs_kz as below. */
 typedef struct icm_plan {
-  int32_t fused_blobs; /* 1: spreading and interpolation inside the x FFT passes through row-block
-                          bins (sides 32, 48, 64, 96, 128, 192, 256, 384, 512); 0: separate kernels */
+  int32_t fused_blobs; /* 1: spreading and interpolation inside the plane passes, where a z plane fits
+                          in shared memory (see fused_xy), else inside the x FFT passes through
+                          row-block bins (sides 32, 48, 64, 96, 128, 192, 256, 384, 512); 0: separate
+                          kernels                                                                  */
   int32_t tma_z;       /* 1: persistent z pass fed by TMA (z sides <= 256 with register kernels);
                           0: one block per z tile                                                  */
   int32_t rhs_kz;      /* right-hand-side kernel of FP32 grids above 2^20 cells: 4..64 z planes marched
@@ -151,10 +153,11 @@ typedef struct icm_plan {
                           normals in a pass of their own and do not march                          */
   int32_t fork;        /* 1: the blob-side prologue runs on a second stream beside the RHS          */
   int32_t fused_xy;    /* 1: forward x and y FFT passes fused on thread-block clusters (FP32,
-                          Nx = Ny in 32, 64, 128, 256); 0 (default): two passes                    */
+                          Nx = Ny in 32, 64, 128, 256); 0 (default): whole z planes in one launch
+                          per direction where they fit in shared memory, else two passes           */
   int32_t z_split;     /* 1: the z transform with its other two-stage split (Nz = 32: 4 x 8, 48:
                           12 x 4, 64: 16 x 4, 96: 8 x 12, 128: 8 x 16, 192: 12 x 16, 256: 32 x 8);
-                          0 (default): the axis split (8 x 4, 16 x 3, 8 x 8, 16 x 6, 16 x 8,
+                          0 (default but FP32 Nz = 256): the axis split (8 x 4, 16 x 3, 8 x 8, 16 x 6, 16 x 8,
                           16 x 12, 16 x 16)                                                        */
 } icm_plan;
 
