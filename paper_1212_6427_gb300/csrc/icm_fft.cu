@@ -240,8 +240,7 @@ template <typename R, int N> constexpr size_t stage_offset() {
 }
 // Blob task records staged per block (the rest are read in place).  The forward x
 // pass stages 128, which keeps its FP32 blocks of sides up to 256 at four per SM
-// (registers capped to match); the inverse pass, which holds its loads in flight in
-// registers and would spill under that cap, stages one per thread.
+// (registers capped to match); the inverse pass: xi2_stage.
 constexpr int kStageF = 128;
 template <typename R, int N, int S> size_t smem_x2b() { return stage_offset<R, N>() + S * sizeof(StagedTask<R>); }
 template <typename R, int N> constexpr int xf2_min_blocks() { return sizeof(R) == 4 && N <= 256 ? 4 : 1; }
