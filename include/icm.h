@@ -140,9 +140,10 @@ icm_status icm_set_blob_wca(icm_sim* sim, double epsilon, double sigma);
  * except fused_xy, rhs_kz as below. */
 typedef struct icm_plan {
   int32_t fused_blobs; /* 1: spreading and interpolation inside the plane passes, where a z plane fits
-                          in shared memory (see fused_xy), else inside the x FFT passes through
-                          row-block bins (sides 32, 48, 64, 96, 128, 192, 256, 384, 512); 0: separate
-                          kernels                                                                  */
+                          in shared memory (see fused_xy) and the blobs are few enough for it to pay
+                          (about 40 per plane in FP32), else inside the x FFT passes through
+                          row-block bins (sides 32, 48, 64, 96, 128, 192, 256, 384, 512) or, on the
+                          other sides and in between, in separate kernels; 0: separate kernels     */
   int32_t tma_z;       /* 1: persistent z pass fed by TMA (z sides <= 256 with register kernels);
                           0: one block per z tile                                                  */
   int32_t rhs_kz;      /* right-hand-side kernel of FP32 grids above 2^20 cells: 4..64 z planes marched

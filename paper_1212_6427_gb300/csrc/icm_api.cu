@@ -521,6 +521,44 @@ RowBins row_bins(const icm_sim* s) {
   return bins;
 }
 
+// Who does the blob work of a step whose planes have passes of their own.
+enum BlobWork : int { BLOBS_IN_PLANES, BLOBS_IN_ROWS, BLOBS_APART };
+
+// Every block of a plane pass looks through all blobs for those of its plane (icm_plane.cu), so the
+// plane passes' blob work grows with blobs times planes, that of the row-block bins and of the
+// separate kernels with the blobs only.  Steps with excess mass make five passes with blob work,
+// steps without one or two.  Measured step times (us), planes / row blocks / separate kernels:
+//   FP32, excess mass: 64^3, 1024 blobs 97 / 111 / 105, 4096 blobs 154 / 136 / 133, 16384 blobs 341 /
+//   221 / 242; 96^3, 4000 blobs 198 / 213 / 196; 128^3, 4096 blobs 278 / 285 / 307, 32768 blobs
+//   666 / 466 / 563; 81^3, 2592 blobs 162 / - / 169, 5184 blobs 203 / - / 191: lines at 40
+//   blobs per plane, 32 on planes of 128 x 128 and above, and 4096 in all.  More planes than three
+//   blocks per SM take turns: 64 x 64 x 256, 2048 blobs 215 / 210 / 232, 8192 blobs 312 / 235 / 287.
+//   Large planes that leave SMs idle lose with any number: 128 x 128 x 32, one blob 127 / 114 / 145.
+//   FP32, neutral blobs: 128^3, 4096 blobs 131 / 158 / 129, 32768 blobs 258 / 285 / 248; 64 x 64 x 256,
+//   4096 blobs 108 / 119 / 107, 16384 blobs 181 / 170 / 156: 64 blobs per plane and 8192 in all.
+//   FP64, where the separate kernels' atomics cost most: 96^3, 16000 blobs 2224 / 2237 / 2665, 256000
+//   blobs 10608 / 8271 / 16438; 64 x 64 x 48, 6144 blobs 594 / 600 / 794; 48^3, 32000 blobs 1394 / 1793 /
+//   2177 (row blocks across planes); neutral, 96^3, 153600 blobs 3448 / 3660 / 4731; 32 x 32 x 256,
+//   65536 blobs 1918 / 1495 / 2026.
+// Past the FP32 lines row blocks win over the separate kernels on large planes, with many blobs or many
+// planes: 96^3, 8000 blobs 252 / 228, 32000 blobs 436 / 451; 128^3 and 64 x 64 x 256 as above.
+BlobWork plane_blob_work(const icm_sim* s) {
+  int r1, r2;
+  const bool rows = s->fused && s->ny % 32 == 0 && fft_split(s->ny, r1, r2);   // (row blocks inside a plane)
+  const bool turns = s->nz > device_sms();   // 3 nz planes, at most three blocks per SM
+  const long long nz = s->nz, cells = (long long)s->nx * s->ny;
+  if (s->prec == 64) {
+    if (!rows || (!s->any_me && !turns)) return BLOBS_IN_PLANES;
+    return s->nb <= (turns ? 16384 : std::min(160 * nz, 16384LL)) ? BLOBS_IN_PLANES : BLOBS_IN_ROWS;
+  }
+  if (!s->any_me) return s->nb <= (s->fused ? std::min(64 * nz, 8192LL) : 64 * nz) ? BLOBS_IN_PLANES : BLOBS_APART;
+  if (!s->fused) return s->nb <= 40 * nz ? BLOBS_IN_PLANES : BLOBS_APART;
+  if (rows && 3 * nz < device_sms() && s->nx >= 128 && s->ny >= 96) return BLOBS_IN_ROWS;
+  const bool large = cells >= 128 * 128;
+  if (s->nb <= (turns ? 2048 : std::min((large ? 32 : 40) * nz, 4096LL))) return BLOBS_IN_PLANES;
+  return rows && (turns || large || s->nb > 6000) ? BLOBS_IN_ROWS : BLOBS_APART;
+}
+
 // The nine steps of Sec. III.C for one time level, enqueued on s->stream.  With a
 // segment index (batched group solves) only the blob and stencil work between two
 // solves is enqueued: segment 0 ends before the first solve, segments 1 and 2 after
@@ -577,8 +615,10 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
   const bool drift = (s->flags & ICM_FLAG_THERMAL_DRIFT) && s->kT > 0.0 && s->nb > 0;
   const double geob = (double)(12 * sizeof(int) + 36 * sizeof(R));   // stencil record per blob
   // blob work inside the plane passes or the x passes
-  const bool in_plane = plane && s->plan.fused_blobs && s->nb > 0 && segment < 0;
-  const bool fused = !in_plane && s->fused && s->plan.fused_blobs && s->nb > 0 && segment < 0;
+  const bool inside = s->plan.fused_blobs && s->nb > 0 && segment < 0;
+  const BlobWork who = plane ? plane_blob_work(s) : BLOBS_IN_ROWS;
+  const bool in_plane = inside && plane && who == BLOBS_IN_PLANES;
+  const bool fused = inside && s->fused && who == BLOBS_IN_ROWS;
   const RowBins bins = row_bins(s);
 
   // The blob-side prologue (scalars, predictor, pair forces, bins) reads only v and the

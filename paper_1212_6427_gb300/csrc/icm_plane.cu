@@ -231,8 +231,8 @@ __device__ __forceinline__ void load_plane_tables(const PlaneSmem<R>& S, const P
 // Calls f(blob, c, r) with four lanes r = 0 .. 3 for every blob whose support along z covers plane z,
 // c the plane's index in it (from -1 to K with EXT, where the Laplacian reaches one plane
 // further).  The block scans the blobs' first nodes, a few coalesced bytes each, and compacts
-// the hits, up to kPlaneList at a time: cheaper than building bins in three launches up to tens
-// of thousands of blobs.  Few enough hits are put in ascending order and served by one warp, so that
+// the hits, up to kPlaneList at a time: cheaper than building bins in three launches while the blobs
+// are few (plane_blob_work in icm_api.cu draws the line).  Few enough hits are put in ascending order and served by one warp, so that
 // what they add up to does not depend on the warps' timing.
 constexpr int kOrdered = 16;
 template <int NT, bool EXT, typename F>
