@@ -1730,24 +1730,30 @@ icm_status icm_op_coupling(icm_sim* s, int64_t n, const double* qi, const double
     return fail(ICM_EINVAL, "need a >= 0, b >= 0, a + b > 0");
   if (n == 0) return ICM_OK;
   if (!finite_all(qi, 3 * n) || !finite_all(qj, 3 * n)) return fail(ICM_EINVAL, "non-finite position");
-  // chunks of pairs bound the scratch (tables of at most 41 KB per position)
-  const long long chunk = std::min<long long>(n, 512);
-  std::vector<double> q(6 * (size_t)chunk);
-  Tmp tq(s, sizeof(double) * 6 * chunk), to(s, sizeof(double) * 9 * chunk);
-  Tmp ts(s, sizeof(double) * couple_scratch_doubles(s->nx, s->ny, s->nz, (int)chunk));
-  if (!tq.p || !to.p || !ts.p) return fail(ICM_ENOMEM, "allocation failed");
-  for (long long p0 = 0; p0 < n; p0 += chunk) {
-    const long long m = std::min(chunk, (long long)n - p0);
-    memcpy(q.data(), qi + 3 * p0, sizeof(double) * 3 * m);
-    memcpy(q.data() + 3 * m, qj + 3 * p0, sizeof(double) * 3 * m);
-    wrap_host(q.data(), 2 * m, s);
-    ICM_CK(cudaMemcpyAsync(tq.p, q.data(), sizeof(double) * 6 * m, cudaMemcpyHostToDevice, s->stream));
-    couple_pairs(s->nx, s->ny, s->nz, s->h, s->kernel, (int)m, (const double*)tq.p, a, b, (double*)ts.p, (double*)to.p,
-                 s->stream);
-    ICM_CK(cudaGetLastError());
-    ICM_CK(cudaMemcpyAsync(out + 9 * p0, to.p, sizeof(double) * 9 * m, cudaMemcpyDeviceToHost, s->stream));
-    ICM_CK(cudaStreamSynchronize(s->stream));
-  }
+  // Positions and results of all pairs on the device; the tables and partial sums of a chunk of pairs in
+  // the spectrum scratch where they fit, else in memory of their own, and if there is none, in
+  // smaller chunks in the spectrum scratch (a pair takes at most a sixth of it).
+  const size_t room = 3 * (size_t)s->nz * s->ny * s->kxp * 2 * s->rsize() / sizeof(double);
+  const auto need = [&](long long m) { return couple_scratch_doubles(s->nx, s->ny, s->nz, (int)m); };
+  long long chunk = std::min<long long>(n, 512);
+  std::vector<double> q(6 * (size_t)n);
+  memcpy(q.data(), qi, sizeof(double) * 3 * n);
+  memcpy(q.data() + 3 * n, qj, sizeof(double) * 3 * n);
+  wrap_host(q.data(), 2 * n, s);
+  Tmp tq(s, sizeof(double) * 6 * n), to(s, sizeof(double) * 9 * n);
+  if (!tq.p || !to.p) return fail(ICM_ENOMEM, "allocation failed");
+  std::unique_ptr<Tmp> own;
+  if (need(chunk) > room) own.reset(new Tmp(s, sizeof(double) * need(chunk)));
+  double* scratch = own && own->p ? (double*)own->p : (double*)s->spec;
+  while (scratch == s->spec && chunk > 1 && need(chunk) > room) chunk = (chunk + 1) / 2;
+  const double* dq = (const double*)tq.p;
+  ICM_CK(cudaMemcpyAsync(tq.p, q.data(), sizeof(double) * q.size(), cudaMemcpyHostToDevice, s->stream));
+  for (long long p0 = 0; p0 < n; p0 += chunk)
+    couple_pairs(s->nx, s->ny, s->nz, s->h, s->kernel, (int)std::min(chunk, (long long)n - p0), dq + 3 * p0,
+                 dq + 3 * (n + p0), a, b, scratch, (double*)to.p + 9 * p0, s->stream);
+  ICM_CK(cudaGetLastError());
+  ICM_CK(cudaMemcpyAsync(out, to.p, sizeof(double) * 9 * n, cudaMemcpyDeviceToHost, s->stream));
+  ICM_CK(cudaStreamSynchronize(s->stream));
   return ICM_OK;
 }
 

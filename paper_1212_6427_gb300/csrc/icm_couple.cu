@@ -39,14 +39,15 @@ struct CoupleDims {
   __host__ __device__ int symbol_base(int ax) const { return ax == 0 ? 0 : count[0] + (ax == 2 ? count[1] : 0); }
 };
 
-// Blocks 0 .. npos-1: the stencil sums of one position (the roots of one axis at a time
-// in shared memory).  Block npos: the symbols.
-__global__ void __launch_bounds__(128) k_couple_tables(CoupleDims d, double h, int kernel, int npos,
-                                                       const double* __restrict__ q, double2* __restrict__ tab,
+// Blocks 0 .. 2 npair - 1: the stencil sums of one position, qi first (the roots of one axis at a time
+// in shared memory).  Block 2 npair: the symbols.
+__global__ void __launch_bounds__(128) k_couple_tables(CoupleDims d, double h, int kernel, int npair,
+                                                       const double* __restrict__ qi, const double* __restrict__ qj,
+                                                       double2* __restrict__ tab,
                                                        double2* __restrict__ sym, double* __restrict__ symdd) {
   __shared__ double2 roots[kMaxSide];
   const int p = blockIdx.x;
-  if (p == npos) {
+  if (p == 2 * npair) {
     for (int ax = 0; ax < 3; ++ax)
       for (int k = threadIdx.x; k < d.count[ax]; k += blockDim.x) {
         double s, c, sf;
@@ -57,6 +58,7 @@ __global__ void __launch_bounds__(128) k_couple_tables(CoupleDims d, double h, i
       }
     return;
   }
+  const double* q = p < npair ? qi + 3 * p : qj + 3 * (p - npair);
   double2* out = tab + (size_t)p * d.per_position();
   for (int ax = 0; ax < 3; ++ax) {
     const int n = d.n[ax];
@@ -64,7 +66,7 @@ __global__ void __launch_bounds__(128) k_couple_tables(CoupleDims d, double h, i
     for (int k = threadIdx.x; k < n; k += blockDim.x) roots[k] = unit_root(k, n);
     __syncthreads();
     for (int off = 0; off < 2; ++off) {
-      const double s = q[3 * p + ax] / h - (off ? 0.5 : 0.0);
+      const double s = q[ax] / h - (off ? 0.5 : 0.0);
       const double anchor = kernel == 3 ? Peskin<double, 3>::anchor(s) : Peskin<double, 4>::anchor(s);
       const double frac = s - anchor;
       double w[4];
@@ -200,15 +202,15 @@ size_t couple_scratch_doubles(int nx, int ny, int nz, int npair) {
   return 2 * (size_t)(2 * npair) * d.per_position() + 3 * (size_t)d.symbols() + 9 * (size_t)npair * couple_blocks(d);
 }
 
-void couple_pairs(int nx, int ny, int nz, double h, int kernel, int npair, const double* q_dev, double a, double b,
-                  double* scratch, double* out_dev, cudaStream_t st) {
+void couple_pairs(int nx, int ny, int nz, double h, int kernel, int npair, const double* qi_dev, const double* qj_dev,
+                  double a, double b, double* scratch, double* out_dev, cudaStream_t st) {
   const CoupleDims d = couple_dims(nx, ny, nz);
   const int nblk = couple_blocks(d);
   double2* tab = reinterpret_cast<double2*>(scratch);
   double2* sym = tab + (size_t)(2 * npair) * d.per_position();
   double* symdd = reinterpret_cast<double*>(sym + d.symbols());
   double* partial = symdd + d.symbols();
-  k_couple_tables<<<2 * npair + 1, 128, 0, st>>>(d, h, kernel, 2 * npair, q_dev, tab, sym, symdd);
+  k_couple_tables<<<2 * npair + 1, 128, 0, st>>>(d, h, kernel, npair, qi_dev, qj_dev, tab, sym, symdd);
   k_couple_modes<<<dim3(nblk, npair), kCoupleThreads, 6 * (size_t)d.count[0] * sizeof(double2), st>>>(
       d, npair, a, b, tab, sym, symdd, partial);
   const double scale = 1.0 / ((double)nx * ny * nz * h * h * h);

@@ -394,11 +394,11 @@ void blob_finish_plane(const BlobParams& p, BlobState s, const double* parts, bo
                        int* hist_dev, cudaStream_t st);
 
 // Coupling matrices J(qi) (a - b L)^-1 P S(qj) (row-major 3 x 3 each) of npair pairs of
-// positions as sums over wave vectors (icm_couple.cu).  q_dev: the npair positions qi, then
-// the npair positions qj, wrapped into the box; scratch: couple_scratch_doubles of them.
+// positions as sums over wave vectors (icm_couple.cu).  qi_dev, qj_dev: npair positions each,
+// wrapped into the box; scratch: couple_scratch_doubles of them, 16-byte aligned.
 size_t couple_scratch_doubles(int nx, int ny, int nz, int npair);
-void couple_pairs(int nx, int ny, int nz, double h, int kernel, int npair, const double* q_dev, double a, double b,
-                  double* scratch, double* out_dev, cudaStream_t st);
+void couple_pairs(int nx, int ny, int nz, double h, int kernel, int npair, const double* qi_dev, const double* qj_dev,
+                  double a, double b, double* scratch, double* out_dev, cudaStream_t st);
 
 // WCA pair forces (Sec. IV.A, Eq. WCA) at q^{n+1/2} through a cell list of cells at
 // least the cut-off wide: count, scan (k_bin_scan on the cell arrays), fill, forces.
