@@ -5,17 +5,18 @@
 // product of three 1-D sums of at most four terms, f(k) = sum_n phi_n exp(-2 pi i k n/N),
 // and the solve is the symbol P^(k)/(a + b |d|^2).  By Parseval's identity
 //   M_ab = (1/(h^3 N)) sum_k conj(J_a) (delta_ab - conj(d_a) d_b / |d|^2) S_b / (a + b|d|^2),
-// so a pair of positions costs one pass over the half spectrum (about 100 operations per
+// so a pair of positions costs one pass over the half spectrum (17 operations per
 // wave vector and pair, everything in registers) where solving for the three unit forces
 // costs three round trips of the 3-D transform, memory passes and launches included.
 //
 // Bound by FP64 operations (an FP64 FMA issues at 1/64 of the FP32 rate on this chip), in
 // both precisions: the sum is formed in FP64 for FP32 simulations too.  16 pairs on 32^3 in
-// FP64, the whole call: 3.49 ms with the transforms (48 solves of eight launches), 0.148 ms
+// FP64, the whole call: 3.49 ms with the transforms (48 solves of eight launches), 0.087 ms
 // with the sums.
 #include <algorithm>
 
 #include "icm_internal.h"
+#include "icm_symbol.cuh"
 
 namespace icm {
 namespace {
@@ -91,74 +92,117 @@ __global__ void __launch_bounds__(128) k_couple_tables(CoupleDims d, double h, i
   }
 }
 
-// A thread takes one (ky, kz) column and sums over kx: the y-z products, the symbols and
-// the nine sums stay in registers, and the x sums of the pair (the same for every thread
-// at a time) are read as broadcasts from shared memory.  128 columns per block keep the
-// FP64 pipe of an SM busy with one block; partial[pair][block][9] is summed by
-// k_couple_final.
+// A thread takes one (ky, kz) column and one segment of kx.  With u = conj(J_x) S_x products of the x
+// sums and c = 1/(|d|^2 (a + b|d|^2)), every entry of M is the real part of a y-z factor times one of five
+// sums over kx, the same for every pair of components that shares their stagger offsets:
+//   s0 = sum c u00,  s1 = sum c u11,  s2 = sum c |d_x|^2 u11,  s3 = sum c conj(d_x) u01,  s4 = sum c d_x u10,
+// (u_ij: J of offset i, S of offset j), as the diagonal's 1/(a + b|d|^2) - c |d_a|^2 is c times the other
+// two |d|^2.  So a wave vector costs ten multiply-adds and one reciprocal, 17 FP64 operations, where
+// forming J, S and their nine products cost 96; the y-z factors are formed once per column and segment.
+// Segments of at most 64 wave numbers spread one pair over the whole device; with 16, where the y-z factors
+// weigh as much as the sums, one pair on 64^3 and 128^3 takes 85 and 135 us instead of 97 and 121, 64
+// pairs 554 and 3476 instead of 400 and 2552.  One pair
+// in an FP32 simulation, the whole call: 128^3 120 us, 256^3 409 us; with one sum per entry on at
+// most 64 blocks 507 and 3431, with three FP32 solves 305 and 1388.
 constexpr int kCoupleThreads = 128;
-__global__ void __launch_bounds__(kCoupleThreads) k_couple_modes(CoupleDims d, int npair, double a, double b,
-                                                                 const double2* __restrict__ tab,
+constexpr int kCoupleSegment = 64;      // wave numbers
+constexpr int kCoupleBlocks = 1216;     // blocks per pair at most: eight per SM
+struct CoupleShape {
+  int nseg, seglen, colblocks;
+  __host__ __device__ int blocks() const { return nseg * colblocks; }
+};
+CoupleShape couple_shape(const CoupleDims& d) {
+  const int cols = d.count[1] * d.count[2];
+  CoupleShape s;
+  s.nseg = (d.count[0] + kCoupleSegment - 1) / kCoupleSegment;
+  s.seglen = (d.count[0] + s.nseg - 1) / s.nseg;
+  const int full = (cols + kCoupleThreads - 1) / kCoupleThreads;
+  const int rounds = (full * s.nseg + kCoupleBlocks - 1) / kCoupleBlocks;   // columns per thread
+  s.colblocks = (full + rounds - 1) / rounds;
+  return s;
+}
+
+__device__ __forceinline__ double2 conj_mul(double2 a, double2 b) {   // conj(a) b
+  return make_double2(fma(a.y, b.y, a.x * b.x), fma(a.x, b.y, -a.y * b.x));
+}
+__device__ __forceinline__ double re_mul(double2 a, double2 b) { return fma(a.x, b.x, -a.y * b.y); }
+
+struct CoupleX {
+  double2 u00, u11, u11dd, u01, u10;
+  double dd, pad;
+};
+
+__global__ void __launch_bounds__(kCoupleThreads) k_couple_modes(CoupleDims d, CoupleShape sh, int npair, double a,
+                                                                 double b, const double2* __restrict__ tab,
                                                                  const double2* __restrict__ sym,
                                                                  const double* __restrict__ symdd,
                                                                  double* __restrict__ partial) {
-  extern __shared__ __align__(16) double2 xs[];   // J off 0, J off 1, S off 0, S off 1, d_x, (|d_x|^2, weight)
+  __shared__ CoupleX xs[kCoupleSegment];
   __shared__ double red[kCoupleThreads / 32][9];
   const int pair = blockIdx.y, kx = d.count[0], tid = threadIdx.x;
+  const int seg = blockIdx.x % sh.nseg, cb = blockIdx.x / sh.nseg;
+  const int k0 = seg * sh.seglen, len = min(sh.seglen, kx - k0);
   const double2* ti = tab + (size_t)pair * d.per_position();
   const double2* tj = tab + (size_t)(npair + pair) * d.per_position();
-  for (int k = tid; k < kx; k += kCoupleThreads) {
-    xs[k] = ti[k];
-    xs[kx + k] = ti[kx + k];
-    xs[2 * kx + k] = tj[k];
-    xs[3 * kx + k] = tj[kx + k];
-    xs[4 * kx + k] = sym[k];
+  for (int i = tid; i < len; i += kCoupleThreads) {
+    const int k = k0 + i;
     // every wave vector but those of kx = 0 and the Nyquist plane stands for its conjugate too
-    xs[5 * kx + k] = make_double2(symdd[k], k == 0 || 2 * k == d.n[0] ? 1.0 : 2.0);
+    const double w = k == 0 || 2 * k == d.n[0] ? 1.0 : 2.0, dd = symdd[k];
+    const double2 i0 = make_double2(w * ti[k].x, w * ti[k].y), i1 = make_double2(w * ti[kx + k].x, w * ti[kx + k].y);
+    const double2 j0 = tj[k], j1 = tj[kx + k], dx = sym[k];
+    CoupleX x;
+    x.u00 = conj_mul(i0, j0);
+    x.u11 = conj_mul(i1, j1);
+    x.u11dd = make_double2(dd * x.u11.x, dd * x.u11.y);
+    x.u01 = conj_mul(cmul(dx, i0), j1);
+    x.u10 = conj_mul(i1, cmul(dx, j0));
+    x.dd = dd;
+    xs[i] = x;
   }
   __syncthreads();
   double m[9];
 #pragma unroll
   for (int i = 0; i < 9; ++i) m[i] = 0.0;
-  const long long cols = (long long)d.count[1] * d.count[2];
-  for (long long c = (long long)blockIdx.x * kCoupleThreads + tid; c < cols; c += (long long)gridDim.x * kCoupleThreads) {
-    const int ky = (int)(c % d.count[1]), kz = (int)(c / d.count[1]);
+  const int cols = d.count[1] * d.count[2], cy = d.count[1], cz = d.count[2];
+  for (int c = cb * kCoupleThreads + tid; c < cols; c += sh.colblocks * kCoupleThreads) {
+    const int kz = c / cy, ky = c - kz * cy;
+    const double ddy = symdd[d.symbol_base(1) + ky], ddz = symdd[d.symbol_base(2) + kz], ddyz = ddy + ddz;
+    double2 s0 = make_double2(0.0, 0.0), s1 = s0, s2 = s0, s3 = s0, s4 = s0;
+#pragma unroll 4
+    for (int k = 0; k < len; ++k) {
+      const CoupleX& x = xs[k];
+      const double dd = x.dd + ddyz, prod = dd * fma(b, dd, a);
+      const double w = positive(prod) ? recip<double>(prod) : 0.0;
+      s0 = cfmar<double>(w, x.u00, s0);
+      s1 = cfmar<double>(w, x.u11, s1);
+      s2 = cfmar<double>(w, x.u11dd, s2);
+      s3 = cfmar<double>(w, x.u01, s3);
+      s4 = cfmar<double>(w, x.u10, s4);
+    }
     const double2* iy = ti + d.base(1) + ky;
     const double2* iz = ti + d.base(2) + kz;
     const double2* jy = tj + d.base(1) + ky;
     const double2* jz = tj + d.base(2) + kz;
     const double2 dy = sym[d.symbol_base(1) + ky], dz = sym[d.symbol_base(2) + kz];
-    const double ddyz = symdd[d.symbol_base(1) + ky] + symdd[d.symbol_base(2) + kz];
-    const int cy = d.count[1], cz = d.count[2];
     // y-z factors of the components x, y, z (a component's own axis has offset 0)
     const double2 Jx = cmul(iy[cy], iz[cz]), Jy = cmul(iy[0], iz[cz]), Jz = cmul(iy[cy], iz[0]);
     const double2 Sx = cmul(jy[cy], jz[cz]), Sy = cmul(jy[0], jz[cz]), Sz = cmul(jy[cy], jz[0]);
-#pragma unroll 2
-    for (int k = 0; k < kx; ++k) {
-      const double2 dx = xs[4 * kx + k], wd = xs[5 * kx + k];
-      const double2 i0 = xs[k], i1 = xs[kx + k], j0 = xs[2 * kx + k], j1 = xs[3 * kx + k];
-      const double dd = wd.x + ddyz;
-      const double den = a + b * dd;
-      // c1 = 1/(a + b|d|^2), c2 = c1/|d|^2; the mean mode is not projected, and dropped at a = 0
-      const double prod = dd * den;
-      const double r = wd.y / (prod > 0.0 ? prod : 1.0);
-      const double c1 = prod > 0.0 ? dd * r : (dd == 0.0 && a > 0.0 ? wd.y / a : 0.0);
-      const double c2 = prod > 0.0 ? r : 0.0;
-      const double2 J[3] = {cmul(i0, Jx), cmul(i1, Jy), cmul(i1, Jz)};
-      const double2 S[3] = {cmul(j0, Sx), cmul(j1, Sy), cmul(j1, Sz)};
-      const double2 dv[3] = {dx, dy, dz};
-      double2 A[3], B[3];   // d_a J_a and c2 d_b S_b
-#pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        A[t] = cmul(dv[t], J[t]);
-        B[t] = cmul(dv[t], S[t]);
-        B[t] = make_double2(c2 * B[t].x, c2 * B[t].y);
-        m[4 * t] = fma(c1, fma(J[t].x, S[t].x, J[t].y * S[t].y), m[4 * t]);   // Re conj(J) S
-      }
-#pragma unroll
-      for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int s = 0; s < 3; ++s) m[3 * p + s] = fma(-A[p].x, B[s].x, fma(-A[p].y, B[s].y, m[3 * p + s]));
+    const double2 xx = conj_mul(Jx, Sx), yy = conj_mul(Jy, Sy), zz = conj_mul(Jz, Sz);
+    const double2 dJy = cmul(dy, Jy), dJz = cmul(dz, Jz), dSy = cmul(dy, Sy), dSz = cmul(dz, Sz);
+    m[0] += ddyz * re_mul(xx, s0);
+    m[1] -= re_mul(conj_mul(Jx, dSy), s3);
+    m[2] -= re_mul(conj_mul(Jx, dSz), s3);
+    m[3] -= re_mul(conj_mul(dJy, Sx), s4);
+    m[4] += re_mul(yy, cfmar<double>(ddz, s1, s2));
+    m[5] -= re_mul(conj_mul(dJy, dSz), s1);
+    m[6] -= re_mul(conj_mul(dJz, Sx), s4);
+    m[7] -= re_mul(conj_mul(dJz, dSy), s1);
+    m[8] += re_mul(zz, cfmar<double>(ddy, s1, s2));
+    // the mean mode (weight 0 above) is not projected, and dropped at a = 0
+    if (c == 0 && k0 == 0 && a > 0.0) {
+      m[0] += re_mul(xx, xs[0].u00) / a;
+      m[4] += re_mul(yy, xs[0].u11) / a;
+      m[8] += re_mul(zz, xs[0].u11) / a;
     }
   }
 #pragma unroll
@@ -176,45 +220,39 @@ __global__ void __launch_bounds__(kCoupleThreads) k_couple_modes(CoupleDims d, i
   }
 }
 
-__global__ void k_couple_final(const double* __restrict__ partial, int nblk, int npair, double scale,
-                               double* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 9 * npair) return;
-  const int pair = i / 9, e = i - 9 * pair;
+// One block per pair, one warp per entry.
+__global__ void __launch_bounds__(9 * 32) k_couple_final(const double* __restrict__ partial, int nblk, double scale,
+                                                         double* __restrict__ out) {
+  const int e = threadIdx.x >> 5, lane = threadIdx.x & 31, pair = blockIdx.x;
   double x = 0.0;
-  for (int b = 0; b < nblk; ++b) x += partial[((size_t)pair * nblk + b) * 9 + e];
-  out[i] = x * scale;
+  for (int b = lane; b < nblk; b += 32) x += partial[((size_t)pair * nblk + b) * 9 + e];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if (lane == 0) out[9 * pair + e] = x * scale;
 }
 
 CoupleDims couple_dims(int nx, int ny, int nz) { return CoupleDims{{nx, ny, nz}, {nx / 2 + 1, ny, nz}}; }
-
-// Blocks per pair: one per 128 columns, at most 64 (the pairs fill the device; a grid of one
-// pair still spreads over 64 SMs, which bounds the final sum's serial chain).
-int couple_blocks(const CoupleDims& d) {
-  const long long cols = (long long)d.count[1] * d.count[2];
-  return (int)std::min<long long>((cols + kCoupleThreads - 1) / kCoupleThreads, 64);
-}
 
 }  // namespace
 
 size_t couple_scratch_doubles(int nx, int ny, int nz, int npair) {
   const CoupleDims d = couple_dims(nx, ny, nz);
-  return 2 * (size_t)(2 * npair) * d.per_position() + 3 * (size_t)d.symbols() + 9 * (size_t)npair * couple_blocks(d);
+  return 2 * (size_t)(2 * npair) * d.per_position() + 3 * (size_t)d.symbols() + 9 * (size_t)npair * couple_shape(d).blocks();
 }
 
 void couple_pairs(int nx, int ny, int nz, double h, int kernel, int npair, const double* qi_dev, const double* qj_dev,
                   double a, double b, double* scratch, double* out_dev, cudaStream_t st) {
   const CoupleDims d = couple_dims(nx, ny, nz);
-  const int nblk = couple_blocks(d);
+  const CoupleShape sh = couple_shape(d);
+  const int nblk = sh.blocks();
   double2* tab = reinterpret_cast<double2*>(scratch);
   double2* sym = tab + (size_t)(2 * npair) * d.per_position();
   double* symdd = reinterpret_cast<double*>(sym + d.symbols());
   double* partial = symdd + d.symbols();
   k_couple_tables<<<2 * npair + 1, 128, 0, st>>>(d, h, kernel, npair, qi_dev, qj_dev, tab, sym, symdd);
-  k_couple_modes<<<dim3(nblk, npair), kCoupleThreads, 6 * (size_t)d.count[0] * sizeof(double2), st>>>(
-      d, npair, a, b, tab, sym, symdd, partial);
+  k_couple_modes<<<dim3(nblk, npair), kCoupleThreads, 0, st>>>(d, sh, npair, a, b, tab, sym, symdd, partial);
   const double scale = 1.0 / ((double)nx * ny * nz * h * h * h);
-  k_couple_final<<<(9 * npair + 127) / 128, 128, 0, st>>>(partial, nblk, npair, scale, out_dev);
+  k_couple_final<<<npair, 9 * 32, 0, st>>>(partial, nblk, scale, out_dev);
 }
 
 }  // namespace icm
