@@ -237,6 +237,7 @@ FftCtx<R> fft_ctx(const icm_sim* s) {
   FftCtx<R> f;
   f.nx = s->nx; f.ny = s->ny; f.nz = s->nz;
   f.kx = s->kx; f.kxp = s->kxp;
+  f.h = s->h;
   f.ncell = s->ncell;
   f.px = s->px; f.py = s->py; f.pz = s->pz;
   f.dx = (const cplx_t<R>*)s->dx; f.ddx = (const R*)s->ddx;
@@ -356,8 +357,9 @@ struct AxisTrig {
 };
 
 // Build one axis plan: radices, twiddles (long double), digit-reversed order, and
-// the symbol d = (exp(i theta) - 1)/h, |d|^2 = 4 sin^2(theta/2)/h^2 by storage position
-// (x: by natural wavenumber, only nx/2+1 of them).
+// the symbol for unit spacing, d = exp(i theta) - 1, |d|^2 = 4 sin^2(theta/2), by storage position
+// (x: by natural wavenumber, only nx/2+1 of them).  The spacing enters with b (SymParams): the projection
+// does not depend on it, and |d|^2 (a + b |d|^2) stays in range whatever the units.
 icm_status build_axis(icm_sim* s, AxisTrig& trig, int n, bool natural, int count, AxisPlan& P, void*& dtab,
                       void*& ddtab, bool z_alt = false) {
   int r1 = 0, r2 = 0;
@@ -395,11 +397,10 @@ icm_status build_axis(icm_sim* s, AxisTrig& trig, int n, bool natural, int count
   }
   for (int i = 0; i < count; ++i) {
     const int k = natural ? i : fop[i];
-    const long double h = s->h;
-    put(dt, 2 * i, (trig.cos_of(k) - 1.0L) / h);
-    put(dt, 2 * i + 1, trig.sin_of(k) / h);
+    put(dt, 2 * i, trig.cos_of(k) - 1.0L);
+    put(dt, 2 * i + 1, trig.sin_of(k));
     const long double sn = trig.half_sin_of(k);
-    put(dd, i, 4.0L * sn * sn / (h * h));
+    put(dd, i, 4.0L * sn * sn);
   }
   void* dtw = dalloc(s, tw.size());
   void* dpof = dalloc(s, sizeof(int) * n);
@@ -1911,7 +1912,7 @@ RepFft rep_entry(const icm_sim* s, int rt) {
     r.dst = s->v;
     r.k0sum = s->scal + SC_K0;
     r.a = s->rho / s->dt;
-    r.b = 0.5 * s->eta;
+    r.b = unit_b(0.5 * s->eta, s->h);
     r.k0mul = k0mul;
   } else if (rt == 1) { // P S dp
     r.dst = s->work;
@@ -1924,7 +1925,7 @@ RepFft rep_entry(const icm_sim* s, int rt) {
     r.dst2 = s->work;
     r.k0sum = s->scal + SC_SUMSRC;
     r.a = s->rho;
-    r.b = 0.5 * s->dt * s->eta;
+    r.b = unit_b(0.5 * s->dt * s->eta, s->h);
     r.k0mul = k0mul;
   }
   return r;

@@ -54,8 +54,8 @@ __global__ void __launch_bounds__(128) k_couple_tables(CoupleDims d, double h, i
         double s, c, sf;
         sincospi((double)k / (double)d.n[ax], &s, &c);
         sf = sinpi(2.0 * (double)k / (double)d.n[ax]);
-        sym[d.symbol_base(ax) + k] = make_double2(-2.0 * s * s / h, sf / h);   // (exp(i theta) - 1)/h
-        symdd[d.symbol_base(ax) + k] = 4.0 * s * s / (h * h);
+        sym[d.symbol_base(ax) + k] = make_double2(-2.0 * s * s, sf);   // exp(i theta) - 1: unit spacing
+        symdd[d.symbol_base(ax) + k] = 4.0 * s * s;
       }
     return;
   }
@@ -250,7 +250,8 @@ void couple_pairs(int nx, int ny, int nz, double h, int kernel, int npair, const
   double* symdd = reinterpret_cast<double*>(sym + d.symbols());
   double* partial = symdd + d.symbols();
   k_couple_tables<<<2 * npair + 1, 128, 0, st>>>(d, h, kernel, npair, qi_dev, qj_dev, tab, sym, symdd);
-  k_couple_modes<<<dim3(nblk, npair), kCoupleThreads, 0, st>>>(d, sh, npair, a, b, tab, sym, symdd, partial);
+  k_couple_modes<<<dim3(nblk, npair), kCoupleThreads, 0, st>>>(d, sh, npair, a, unit_b(b, h), tab, sym,
+                                                                symdd, partial);
   const double scale = 1.0 / ((double)nx * ny * nz * h * h * h);
   k_couple_final<<<npair, 9 * 32, 0, st>>>(partial, nblk, scale, out_dev);
 }

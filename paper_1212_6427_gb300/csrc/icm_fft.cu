@@ -1300,7 +1300,7 @@ template <typename R>
 void fft_z_symbol(const FftCtx<R>& f, double a, double b, const double* k0sum, double k0scale, cudaStream_t st) {
   SymParams<R> sp;
   sp.a = (R)a;
-  sp.b = (R)b;
+  sp.b = (R)unit_b(b, f.h);
   sp.inv_ntot = (R)(0.5 / (double)f.ncell);
   sp.mean_scale = a > 0.0 ? (R)(0.5 / (a * (double)f.ncell)) : R(0);
   sp.dx = f.dx; sp.ddx = f.ddx;

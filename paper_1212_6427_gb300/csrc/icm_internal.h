@@ -74,6 +74,9 @@ struct AxisPlan {
   const int* pos_of_freq = nullptr;  // device: n ints
 };
 
+// b of a symbol a + b |d|^2 whose |d|^2 is for unit spacing.
+inline double unit_b(double b, double h) { return b / h / h; }
+
 // Everything the FFT passes need for one grid.
 template <typename R>
 struct FftCtx {
@@ -82,11 +85,12 @@ struct FftCtx {
   int kxp;       // padded row length of the spectrum (multiple of 16)
   long long ncell;
   AxisPlan px, py, pz;
-  // Discrete symbols d_a = (exp(i theta_a) - 1)/h and |d_a|^2: x by natural kx,
+  // Discrete symbols for unit spacing d_a = exp(i theta_a) - 1 and |d_a|^2: x by natural kx,
   // y and z by storage position of the forward pass.
   const cplx_t<R>* dx; const R* ddx;
   const cplx_t<R>* dy; const R* ddy;
   const cplx_t<R>* dz; const R* ddz;
+  double h;          // the spacing
   cplx_t<R>* spec;   // 3 * nz * ny * kxp complex scratch
   const void* zmap;  // host copy of the TMA descriptors of spec for the z pass (or null)
   int* err;          // device error bits (bounded waits report here)
@@ -124,7 +128,7 @@ struct RepFft {
   void* dst;            // output field
   void* dst2;           // second output (OUT_ADD_AND_STORE2)
   const double* k0sum;  // prescribed grid sums of the mean mode (or null)
-  double a, b, k0mul;   // symbol a + b |d|^2 and k0sum scale (k0scale / ncell)
+  double a, b, k0mul;   // symbol a + b |d|^2 for unit spacing and k0sum scale (k0scale / ncell)
   int slot;             // spec = slot-th spectrum of a contiguous group buffer (tensor-map z pass)
   const RowBlobs* rb;   // the replica's blob work in the x passes (blob solves), or null
 };

@@ -8,7 +8,7 @@ namespace icm {
 
 template <typename R>
 struct SymParams {
-  R a, b;
+  R a, b;         // of a + b|d|^2 with d for unit spacing (unit_b)
   R inv_ntot;     // 1/(2 ncell): the forward passes leave twice the spectrum (they split two packed real
                   // rows without the factor 1/2)
   R mean_scale;   // the symbol's scale on the mean mode: 1/(2 a ncell), 0 when a = 0
@@ -24,7 +24,8 @@ namespace {
 // identity on the mean mode, whose value is replaced by the FP64 bookkeeping if given
 // (and which is zero when a = 0).
 // One reciprocal r = 1/(|d|^2 (a + b|d|^2)) serves both divisions; |d|^2 = 0 only on the mean mode,
-// whose scale is precomputed.
+// whose scale is precomputed.  |d|^2 is between 4 sin^2(pi/512) = 1.5e-4 and 12, so the product is in range where
+// a + b|d|^2 and its reciprocal are.
 // 1/x, x normal and positive: the hardware reciprocal in FP32 (within one ulp); in FP64 the
 // approximate reciprocal instruction and one step of third order, y (1 + e + e^2) with
 // e = 1 - x y, three FP64 operations where a division takes about ten (FP64 operations bound
