@@ -1595,7 +1595,7 @@ void fft_x_inverse_group(const FftCtx<R>& f, const RepFft* reps, int G, int mode
 template <typename R>
 void spectral_solve_group(const FftCtx<R>& f, const RepFft* reps, int G, int mode, cudaStream_t st,
                           const void* gzmap, bool blobs) {
-  if (!blobs && plane_has_passes(8 * sizeof(R), f.nx, f.ny, f.nz)) {
+  if (!blobs && plane_has_group_passes(8 * sizeof(R), f.nx, f.ny, f.nz, G)) {
     plane_forward<R>(f, nullptr, nullptr, reps, G, st);
     fft_yz_group<R>(f, reps, G, 1, st, gzmap);
     plane_inverse<R>(f, nullptr, nullptr, mode, nullptr, reps, G, st);

@@ -378,6 +378,8 @@ __device__ __forceinline__ double plane_sum(const double* __restrict__ part, lon
 }
 // Whether a grid's planes fit in shared memory (and are worth it).
 bool plane_has_passes(int precision, int nx, int ny, int nz);
+// The same for a group solve of that many members on the grid.
+bool plane_has_group_passes(int precision, int nx, int ny, int nz, int members);
 template <typename R> void plane_prepare();
 bool plane_prepared();
 // The spectrum fft_x_forward + fft_y leave, with the blobs' spread (pb, or null); src may be null

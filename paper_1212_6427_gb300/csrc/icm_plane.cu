@@ -864,6 +864,21 @@ bool plane_has_passes(int precision, int nx, int ny, int nz) {
   const int nsm = device_sms(), planes = 3 * nz, waves = (planes + nsm - 1) / nsm;
   return precision == 32 || waves == 1 || 10 * planes >= 8 * waves * nsm;
 }
+
+// A launch over many members keeps the device full whichever way, and then the separate passes' cheaper
+// butterflies count.  In FP64 that is so from two members on: planes / separate, a step of the batch (us):
+// 32^3, two members 299 / 248, 32 members 2226 / 1574; 48^3 583 / 570 and 7561 / 6693; 96^3 3427 / 3441
+// and (16) 25729 / 25749.  In FP32 planes win up to one round of three blocks per SM, or two full ones,
+// and from 96 x 96 on: 32^3, four members 99 / 103, 16 members 187 / 159; 48^3, three 127 / 155, six 185 /
+// 203, 16 members 393 / 375; 64^3, two 140 / 141, 16 members 609 / 563; 96^3, 16 members 1643 / 1898;
+// 128^3, two 540 / 497, eight 1749 / 1796.
+bool plane_has_group_passes(int precision, int nx, int ny, int nz, int members) {
+  if (!plane_has_passes(precision, nx, ny, nz)) return false;
+  if (members == 1) return true;
+  if (precision == 64) return false;
+  const long long planes = 3LL * nz * members, round = 3LL * device_sms();
+  return planes <= round || nx * ny >= 96 * 96 || (planes <= 2 * round && 10 * planes >= 18 * round);
+}
 #endif
 
 template <typename R>
