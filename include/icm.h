@@ -146,12 +146,13 @@ typedef struct icm_plan {
                           other sides and in between, in separate kernels; 0: separate kernels     */
   int32_t tma_z;       /* 1: persistent z pass fed by TMA (z sides <= 256 with register kernels);
                           0: one block per z tile                                                  */
-  int32_t rhs_kz;      /* right-hand-side kernel of FP32 grids above 2^20 cells: 4..64 z planes marched
-                          by each block, or 0 for persistent blocks (as many as the SMs hold)
-                          marching even shares of all tile-planes (default 0 when each of two
-                          blocks per SM gets at least 8 tile-planes of 32 x 16 cells, else 8 for
-                          Nz <= 48 and 16 otherwise).  Smaller grids and FP64 draw the stress
-                          normals in a pass of their own and do not march                          */
+  int32_t rhs_kz;      /* right-hand-side kernel of FP32 grids (but up to 2^20 cells at kT = 0, or with Nx
+                          up to 16, or 32): 4..64 z planes marched by each block, or 0 for persistent blocks (as
+                          many as the SMs hold) marching even shares of all tile-planes (default 0
+                          when each of two blocks per SM gets at least 8 tile-planes of 32 x 16
+                          cells, else the fewest planes that give every SM one or two blocks).
+                          Those grids and FP64 draw the stress normals in a pass of their own and
+                          do not march                                                             */
   int32_t fork;        /* 1: the blob-side prologue runs on a second stream beside the RHS          */
   int32_t fused_xy;    /* 1: forward x and y FFT passes fused on thread-block clusters (FP32,
                           Nx = Ny in 32, 64, 128, 256); 0 (default): whole z planes in one launch
@@ -397,7 +398,9 @@ icm_status icm_batch_step(icm_batch* batch, int64_t nsteps);
  * along every axis of every grid, and no WCA pair forces or thermal drift; otherwise
  * the batch runs as with grouped = 1.  Groups on z sides from 96 whose plan takes the
  * tensor-map z pass put their members' spectra in one buffer of the batch (the members'
- * own spectra stay unused meanwhile).  The batch's device tables and these buffers come
+ * own spectra stay unused meanwhile).  FP64 members with noise whose spectra are too small for
+ * all of their stress normals share a buffer of the batch for them; without room for it the
+ * batch runs as with grouped = 1.  The batch's device tables and these buffers come
  * from cudaMalloc, not from the members' allocator, and are freed at the next capture
  * or by icm_batch_destroy.  Batched stages with the blob work in the group
  * x passes (grouped = 3): as 2, but where every member has blobs and a register x side

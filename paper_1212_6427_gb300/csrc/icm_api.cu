@@ -109,8 +109,7 @@ struct icm_sim {
   void* v = nullptr;     // face velocities
   void* adv = nullptr;   // A^{n-1}, overwritten by A^n
   void* work = nullptr;  // right-hand side / spread sources / dv~ / dv
-  void* spec = nullptr;  // spectrum scratch
-  void* normals = nullptr;   // stress normals of the step (grids whose right-hand side stores them), 6 ncell
+  void* spec = nullptr;  // spectrum scratch; the stress normals before the first solve
   // FFT plans and symbol tables
   AxisPlan px, py, pz;
   void *dx = nullptr, *ddx = nullptr, *dy = nullptr, *ddy = nullptr, *dz = nullptr, *ddz = nullptr;
@@ -175,6 +174,7 @@ struct icm_sim {
   bool graph_ok = false;
   long long version = 0;     // bumped whenever the step sequence changes (batch graphs recapture)
 
+  long long spec_reals() const { return 6LL * nz * ny * kxp; }   // of the precision
   size_t rsize() const { return prec == 32 ? sizeof(float) : sizeof(double); }
 };
 
@@ -649,7 +649,7 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
     ICM_STAGE("bins", nb * (24.0 + 2 * geob + 8.0 * kAccPerBlob), build_row_bins<R>(bp, s->nb, s->qh, bins, sb));
   if (fork) cudaEventRecord(s->ev_join, sb);
   // step 2: unperturbed fluid solve (Eq. provisional_step-1)
-  ICM_STAGE("rhs", 4 * F, explicit_rhs<R>(gp, v, adv, work, (R*)s->normals, s->step_dev, s->hist_dev, st));
+  ICM_STAGE("rhs", 4 * F, explicit_rhs<R>(gp, v, adv, work, (R*)s->spec, s->spec_reals(), s->step_dev, s->hist_dev, st));
   if (fork) cudaStreamWaitEvent(st, s->ev_join, 0);
   if (drift) ICM_STAGE("drift", 2 * gath + nb * 32, blob_spread_drift<R>(bp, bs, work, st));
   if (in_plane) {
@@ -795,15 +795,20 @@ std::string plan_key(const icm_sim* s) {
 // The plan of a simulation nobody tuned: everything on (the 32 x 8 z split on FP32 z
 // sides of 256).  The RHS blocks are persistent
 // when every block of a full GPU (two per SM) gets at least 8 tile-planes of 32 x 16
-// cells, which the single-simulation sweeps found fastest from 128^3 up; on smaller
-// grids they march 8 z planes on short z sides, else 16.
+// cells, which the single-simulation sweeps found fastest from 128^3 up; smaller
+// grids march as few planes per block as give every SM one block, or two at half as much again per plane (a march
+// starts with two planes): 64^3, 4 / 8 / 16 planes 13.9 / 18.8 / 29.0 us; 96^3, 4 / 6 / 8 / 16 planes 26.0 /
+// 23.9 / 28.3 / 29.2; 64 x 64 x 96, 4 / 6 / 8 planes 19.1 / 16.8 / 19.0.
 icm_plan default_plan(const icm_sim* s) {
-  int dev = 0, nsm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) !=
-                                                cudaSuccess)
-    nsm = 1;
-  const long long tile_planes = (long long)((s->nx + 31) / 32) * ((s->ny + 15) / 16) * s->nz;
-  const int kz = tile_planes >= 16LL * std::max(nsm, 1) ? 0 : (s->nz <= 48 ? 8 : 16);
+  const int nsm = device_sms();
+  const long long tiles = (long long)((s->nx + 31) / 32) * ((s->ny + 15) / 16);
+  const auto march = [&](int blocks) {   // planes per block that give at most so many blocks
+    int kz = 4;
+    while (kz < 64 && tiles * ((s->nz + kz - 1) / kz) > blocks) ++kz;
+    return kz;
+  };
+  const int one = march(nsm), two = march(2 * nsm);
+  const int kz = tiles * s->nz >= 16LL * nsm ? 0 : (2 * (one + 2) <= 3 * (two + 2) ? one : two);
   // the 32 x 8 z split measured 5% faster than 16 x 16 in the FP32 tensor-map z pass at 256
   const int zs = s->prec == 32 && s->nz == 256 ? 1 : 0;
   return icm_plan{1, 1, kz, 1, 0, zs};
@@ -1134,14 +1139,12 @@ icm_status icm_create(const int32_t grid[3], double h, double rho, double eta, d
   s->adv = dalloc(s, fbytes);
   s->work = dalloc(s, fbytes);
   s->spec = dalloc(s, 3 * (size_t)s->nz * s->ny * s->kxp * 2 * rs);
-  const bool stored = kT > 0.0 && rhs_stored_normals(s->prec, s->ncell);
-  if (stored) s->normals = dalloc(s, 2 * fbytes);
   s->scal = (double*)dalloc(s, sizeof(double) * SC_COUNT);
   s->step_dev = (long long*)dalloc(s, 256);
   s->hist_dev = (int*)dalloc(s, 256);
   s->err_dev = (int*)dalloc(s, 256);
   s->partial = (double*)dalloc(s, sizeof(double) * 3 * icm_sim::kPartials);
-  if (!s->v || !s->adv || !s->work || !s->spec || (stored && !s->normals) || !s->scal || !s->step_dev || !s->hist_dev || !s->err_dev ||
+  if (!s->v || !s->adv || !s->work || !s->spec || !s->scal || !s->step_dev || !s->hist_dev || !s->err_dev ||
       !s->partial) {
     icm_destroy(s);
     return fail(ICM_ENOMEM, "device allocation of %.1f MB of grid state failed", (4.0 * fbytes) / 1e6);
@@ -1777,10 +1780,10 @@ icm_status icm_op_explicit_rhs(icm_sim* s, const double* fluid_v, const double* 
   ICM_CK(cudaMemcpyAsync((char*)tc.p + 64, &hist, sizeof(int), cudaMemcpyHostToDevice, s->stream));
   const GridParams gp = grid_params(s);
   if (s->prec == 32)
-    explicit_rhs<float>(gp, (const float*)tv.p, (float*)ta.p, (float*)s->work, (float*)s->normals, (const long long*)tc.p,
+    explicit_rhs<float>(gp, (const float*)tv.p, (float*)ta.p, (float*)s->work, (float*)s->spec, s->spec_reals(), (const long long*)tc.p,
                         (const int*)((char*)tc.p + 64), s->stream);
   else
-    explicit_rhs<double>(gp, (const double*)tv.p, (double*)ta.p, (double*)s->work, (double*)s->normals, (const long long*)tc.p,
+    explicit_rhs<double>(gp, (const double*)tv.p, (double*)ta.p, (double*)s->work, (double*)s->spec, s->spec_reals(), (const long long*)tc.p,
                          (const int*)((char*)tc.p + 64), s->stream);
   ICM_CK(cudaGetLastError());
   if ((st = download_field(s, s->work, out_rhs)) != ICM_OK) return st;
@@ -1848,7 +1851,7 @@ struct icm_batch {
   std::vector<cudaStream_t> gstreams;  // one per group of the last capture
   void* reps = nullptr;                // device tables of the group solves
   void* stage_tables = nullptr;        // device member tables of the batched stages
-  std::vector<void*> group_specs;      // spectra of the groups with the tensor-map z pass
+  std::vector<void*> group_specs;      // spectra of the groups with the tensor-map z pass, normals of FP64 members
 };
 
 namespace {
@@ -2057,6 +2060,27 @@ icm_status batch_capture_stages(icm_batch* b) {
       zero_prefix.push_back(zero_prefix.back() + 3 * s->ncell * (long long)sizeof(R) / 16);
     }
   }
+  // FP64: one launch draws the normals of all members, so members whose spectrum scratch does not hold theirs
+  // (explicit_rhs goes through it in slabs) share a buffer of the batch; without room for
+  // it the batch runs as with group solves only
+  size_t extra = 0;
+  for (const icm_sim* s : b->sims)
+    if (sizeof(R) == 8 && s->kT > 0.0 && s->spec_reals() < 6 * s->ncell) extra += 6 * (size_t)s->ncell * sizeof(R);
+  unsigned char* normals_at = nullptr;
+  if (extra > 0) {
+    void* buf = nullptr;
+    if (cudaMalloc(&buf, extra) != cudaSuccess) {
+      cudaGetLastError();
+      return ICM_ENOMEM;
+    }
+    b->group_specs.push_back(buf);
+    normals_at = (unsigned char*)buf;
+  }
+  auto normals_room = [&](long long reals) {
+    unsigned char* p = normals_at;
+    normals_at += reals * sizeof(R);
+    return p;
+  };
   std::vector<RhsMember<R>> rhs_noise, rhs_quiet;
   long long tot_noise = 0, tot_quiet = 0;
   for (icm_sim* s : b->sims) {
@@ -2066,7 +2090,8 @@ icm_status batch_capture_stages(icm_batch* b) {
     r.v = (const R*)s->v;
     r.adv = (R*)s->adv;
     r.rhs = (R*)s->work;
-    r.normals = (R*)s->normals;
+    r.normals = (R*)s->spec;
+    if (sizeof(R) == 8 && s->kT > 0.0 && s->spec_reals() < 6 * s->ncell) r.normals = (R*)normals_room(6 * s->ncell);
     r.step_dev = s->step_dev;
     r.hist_dev = s->hist_dev;
     long long& tot = s->kT > 0.0 ? tot_noise : tot_quiet;
@@ -2203,8 +2228,11 @@ icm_status batch_capture_stages(icm_batch* b) {
 
 icm_status batch_capture(icm_batch* b) {
   batch_clear_graph(b);
-  if (b->grouped >= 2 && stages_possible(b))
-    return b->sims[0]->prec == 32 ? batch_capture_stages<float>(b) : batch_capture_stages<double>(b);
+  if (b->grouped >= 2 && stages_possible(b)) {
+    const icm_status st = b->sims[0]->prec == 32 ? batch_capture_stages<float>(b) : batch_capture_stages<double>(b);
+    if (st != ICM_ENOMEM) return st;
+    batch_clear_graph(b);
+  }
   const size_t n = b->sims.size();
   // groups of two or more members on a grid with register FFT passes
   std::vector<SolveGroup> groups;
@@ -2374,8 +2402,7 @@ int64_t icm_estimate_device_bytes(const int32_t grid[3], int32_t precision, int6
   const int64_t kxp = (grid[0] / 2 + 1 + 15) / 16 * 16;
   int64_t cap = 64;
   while (cap < nblobs) cap *= 2;
-  // velocities, advective fluxes, work, and the stress normals where they are stored
-  const int64_t fields = 3 * (3 * ncell * rs) + (rhs_stored_normals(precision, ncell) ? 6 * ncell * rs : 0);
+  const int64_t fields = 3 * (3 * ncell * rs);   // velocities, advective fluxes, work
   const int64_t spec = 3 * (int64_t)grid[2] * grid[1] * kxp * 2 * rs;
   const int64_t tables = 3 * (int64_t)kMaxSide * (3 * 2 * rs + 4) + 16 * 256;
   const int64_t blobs = nblobs > 0 ? 41 * cap * 8 + (int64_t)bin_blob_bytes(cap) : 0;

@@ -498,11 +498,12 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 2 : 1) k_rhs_batch(const 
 // threads' worth of cells per plane and a prologue of two planes.  Used
 //  * in FP64, always: the work is bound by the FP64 pipe, and the march draws 9% of its
 //    normals twice, for halos;
-//  * in FP32, up to kFlatCells: what the march saves (48 bytes per cell of stored normals)
-//    only pays where every SM marches many planes.
-// Measured with noise, both launches (us), march against stored normals: FP32 19.0 / 10.5 on
-// 32^3, 29.8 / 15.1 on 64^3, 29.9 / 25.4 on 96^3, 43.6 / 56.3 on 128^3, 259 / 386 on 256^3;
-// FP64 449 / 24 on 32^3 (eight marching blocks) and 1422 / 685 on 128^3, where half of the
+//  * in FP32, on at most kFlatCells cells where the normals of all fit in the scratch (x sides up to 16, and
+//    32) or there are none: elsewhere the march, in runs short enough for every SM (default_plan),
+//    takes as long without storing anything.
+// Measured with noise, both launches (us), march against stored normals: FP32 18.1 / 10.7 on 32^3, 13.9 /
+// 15.3 on 64^3, 23.9 / 26.0 on 96^3, 25.7 / 19.4 on 81^3 (ragged tiles), 43.6 / 56.3 on 128^3, 259 / 386 on
+// 256^3; FP64 449 / 24 on 32^3 (eight marching blocks) and 1422 / 700 on 128^3, where half of the
 // gain is the cheaper normals above.
 // ---------------------------------------------------------------------------
 constexpr int kFlatThreads = 128;
@@ -539,10 +540,46 @@ __device__ __forceinline__ void noise_pair(const GridParams& g, uint32_t t, uint
   put(c1, 4, 5);
 }
 
-// The right-hand side of one cell, the same sums as rhs_run's (its comments apply).
+// The normals live in the spectrum scratch, which no one needs before the first solve and which
+// holds 3.2 to 6 reals per cell, so the right-hand side takes no memory of its own (a buffer for them was
+// 40% more device memory in FP64).  Where the 6 of every cell do not fit, slab after slab of planes does: the
+// normals of planes k0 - 1 .. k0 + n, then the right-hand sides of planes k0 .. k0 + n - 1.  All at once / in two
+// slabs: 298 / 313 us on 96^3 in FP64, 685 / 707 on 128^3.
+struct NormalSlabs {
+  int n, count;   // planes per slab (all of them: no halo), slabs
+  bool whole() const { return count == 1; }
+};
+NormalSlabs normal_slabs(long long plane, int nz, long long room) {
+  const long long fit = room / (6 * plane);   // planes
+  if (fit >= nz) return NormalSlabs{nz, 1};
+  const int count = (int)((nz + fit - 3) / (fit - 2));
+  return NormalSlabs{(nz + count - 1) / count, count};
+}
+
+// Normals of cell `t` of the slab of planes k0 - 1 .. k0 + n (periodic).  One cell per thread: two that share a Philox
+// call are no faster on large grids (96^3 in FP64 315 us against 313) and slower where a thread's chain of
+// operations is what takes the time (24^3 39.8 against 31.8).
+template <typename R>
+__device__ __forceinline__ void noise_slab_cell(const GridParams& g, uint32_t t, int k0, int n, uint32_t step,
+                                                R* __restrict__ z) {
+  const uint32_t plane = (uint32_t)g.nx * (uint32_t)g.ny, nc = plane * (uint32_t)(n + 2);
+  if (t >= nc) return;
+  const int slot = (int)g.dny.div(g.dnx.div(t));
+  int k = k0 - 1 + slot;
+  k = k < 0 ? k + g.nz : (k >= g.nz ? k - g.nz : k);
+  const uint32_t cell = t - (uint32_t)slot * plane + (uint32_t)k * plane;
+  R w[6];
+  cell_normals<R>(cell, plane, (k & 1) != 0, step, PhiloxKey{g.key0, g.key1}, w);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) z[(size_t)c * nc + t] = w[c];
+}
+
+// The right-hand side of one cell, the same sums as rhs_run's (its comments apply).  z holds the normals of all
+// cells or, with slab, those of `slots` planes from plane k0 - 1 on.
 template <typename R, bool NOISE>
 __device__ __forceinline__ void rhs_cell(const GridParams& g, uint32_t o, bool hist, const R* __restrict__ v,
-                                         R* __restrict__ adv, R* __restrict__ rhs, const R* __restrict__ z) {
+                                         R* __restrict__ adv, R* __restrict__ rhs, const R* __restrict__ z,
+                                         bool slab = false, int k0 = 0, int slots = 0) {
   const uint32_t nc = (uint32_t)g.ncell, nx = g.nx, plane = nx * (uint32_t)g.ny;
   const uint32_t row = g.dnx.div(o), i = o - row * nx;
   const uint32_t k = g.dny.div(row), j = row - k * (uint32_t)g.ny;
@@ -577,12 +614,16 @@ __device__ __forceinline__ void rhs_cell(const GridParams& g, uint32_t o, bool h
   q.z_zpxm = adv_on ? vz[above(xm)] : R(0); q.z_zpym = adv_on ? vz[above(ym)] : R(0);
   R zd[3], ze[3];
   if (NOISE) {
-    const R *zxx = z, *zyy = z + nc, *zzz = z + 2 * (size_t)nc, *zxy = z + 3 * (size_t)nc, *zxz = z + 4 * (size_t)nc,
-            *zyz = z + 5 * (size_t)nc;
-    const R xy = zxy[o], xz = zxz[o], yz = zyz[o];
-    zd[0] = zxx[o] - zxx[xm]; ze[0] = (zxy[yp] - xy) + (zxz[zp] - xz);
-    zd[1] = zyy[o] - zyy[ym]; ze[1] = (zxy[xp] - xy) + (zyz[zp] - yz);
-    zd[2] = zzz[o] - zzz[zm]; ze[2] = (zxz[xp] - xz) + (zyz[yp] - yz);
+    // the cell in z (o, or o - (k0 - 1) plane), and its neighbours there: a slab does not wrap along z
+    const uint32_t zo = slab ? o + plane - (uint32_t)k0 * plane : o, zc = slab ? plane * (uint32_t)slots : nc;
+    const uint32_t zd1 = slab ? zo - plane : zm, zu = slab ? zo + plane : zp;
+    const uint32_t zxm = zo + (xm - o), zxp = zo + (xp - o), zym = zo + (ym - o), zyp = zo + (yp - o);
+    const R *zxx = z, *zyy = z + zc, *zzz = z + 2 * (size_t)zc, *zxy = z + 3 * (size_t)zc, *zxz = z + 4 * (size_t)zc,
+            *zyz = z + 5 * (size_t)zc;
+    const R xy = zxy[zo], xz = zxz[zo], yz = zyz[zo];
+    zd[0] = zxx[zo] - zxx[zxm]; ze[0] = (zxy[zyp] - xy) + (zxz[zu] - xz);
+    zd[1] = zyy[zo] - zyy[zym]; ze[1] = (zxy[zxp] - xy) + (zyz[zu] - yz);
+    zd[2] = zzz[zo] - zzz[zd1]; ze[2] = (zxz[zxp] - xz) + (zyz[zyp] - yz);
   }
   R a[3] = {R(0), R(0), R(0)};
   if (adv_on) advection<R>(q, rhs_c<R>(g).aq, a);
@@ -601,6 +642,21 @@ __global__ void __launch_bounds__(kFlatThreads) k_rhs_flat(GridParams g, const R
                                                          const int* __restrict__ hist_dev) {
   const uint32_t o = blockIdx.x * kFlatThreads + threadIdx.x;
   if (o < (uint32_t)g.ncell) rhs_cell<R, NOISE>(g, o, *hist_dev != 0, v, adv, rhs, z);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kFlatThreads / 2) k_noise_slab(GridParams g, int k0, int n, R* __restrict__ z,
+                                                                const long long* __restrict__ step_dev) {
+  noise_slab_cell<R>(g, blockIdx.x * (kFlatThreads / 2) + threadIdx.x, k0, n, (uint32_t)(*step_dev), z);
+}
+template <typename R>
+__global__ void __launch_bounds__(kFlatThreads) k_rhs_slab(GridParams g, int k0, int n,
+                                                         const R* __restrict__ v, R* __restrict__ adv,
+                                                         R* __restrict__ rhs, const R* __restrict__ z,
+                                                         const int* __restrict__ hist_dev) {
+  const uint32_t plane = (uint32_t)g.nx * (uint32_t)g.ny, t = blockIdx.x * kFlatThreads + threadIdx.x;
+  if (t < plane * (uint32_t)n)
+    rhs_cell<R, true>(g, t + (uint32_t)k0 * plane, *hist_dev != 0, v, adv, rhs, z, true, k0, n + 2);
 }
 
 // The same over every member of a batch: block u of a member (units of 128 cells or 64 pairs).
@@ -746,19 +802,34 @@ size_t rhs_smem() { return sizeof(RhsSmem<R>); }
 
 }  // namespace
 
-bool rhs_stored_normals(int precision, long long ncell) { return precision == 64 || ncell <= kFlatCells; }
+bool rhs_marches(int precision, int nx, int ny, int nz, bool noise) {
+  if (precision == 64) return false;
+  const bool whole = (nx / 2 + 1 + 15) / 16 * 16 >= nx;   // the row length of the spectrum
+  return (long long)nx * ny * nz > kFlatCells || (noise && !whole);
+}
 
 template <typename R>
-void explicit_rhs(const GridParams& g, const R* v, R* adv, R* rhs, R* normals, const long long* step_dev,
+void explicit_rhs(const GridParams& g, const R* v, R* adv, R* rhs, R* normals, long long room, const long long* step_dev,
                   const int* hist_dev, cudaStream_t st) {
-  if (rhs_stored_normals(8 * sizeof(R), g.ncell)) {
-    const unsigned cells = (unsigned)((g.ncell + kFlatThreads - 1) / kFlatThreads);
-    if (g.kT > 0.0) {
-      const long long pairs = (long long)g.nx * g.ny * ((g.nz + 1) / 2);
-      k_noise<R><<<(unsigned)((2 * pairs + kFlatThreads - 1) / kFlatThreads), kFlatThreads / 2, 0, st>>>(g, normals, step_dev);
-      k_rhs_flat<R, true><<<cells, kFlatThreads, 0, st>>>(g, v, adv, rhs, normals, hist_dev);
-    } else {
-      k_rhs_flat<R, false><<<cells, kFlatThreads, 0, st>>>(g, v, adv, rhs, normals, hist_dev);
+  if (!rhs_marches(8 * sizeof(R), g.nx, g.ny, g.nz, g.kT > 0.0)) {
+    const long long plane = (long long)g.nx * g.ny;
+    const auto blocks = [](long long threads, int nt) { return (unsigned)((threads + nt - 1) / nt); };
+    if (!(g.kT > 0.0)) {
+      k_rhs_flat<R, false><<<blocks(g.ncell, kFlatThreads), kFlatThreads, 0, st>>>(g, v, adv, rhs, normals, hist_dev);
+      return;
+    }
+    const NormalSlabs ns = normal_slabs(plane, g.nz, room);
+    if (ns.whole()) {
+      k_noise<R><<<blocks(plane * ((g.nz + 1) / 2), kFlatThreads / 2), kFlatThreads / 2, 0, st>>>(g, normals, step_dev);
+      k_rhs_flat<R, true><<<blocks(g.ncell, kFlatThreads), kFlatThreads, 0, st>>>(g, v, adv, rhs, normals, hist_dev);
+      return;
+    }
+    if constexpr (sizeof(R) == 8) {   // (FP32: whole, see rhs_marches)
+      for (int k0 = 0; k0 < g.nz; k0 += ns.n) {
+        const int n = std::min(ns.n, g.nz - k0);
+        k_noise_slab<R><<<blocks(plane * (n + 2), kFlatThreads / 2), kFlatThreads / 2, 0, st>>>(g, k0, n, normals, step_dev);
+        k_rhs_slab<R><<<blocks(plane * n, kFlatThreads), kFlatThreads, 0, st>>>(g, k0, n, v, adv, rhs, normals, hist_dev);
+      }
     }
     return;
   }
@@ -945,7 +1016,7 @@ void scalars_after_step(double* scal, double, double, double, bool inertial, lon
 }
 
 #define ICM_INST(R)                                                                                          \
-  template void explicit_rhs<R>(const GridParams&, const R*, R*, R*, R*, const long long*, const int*, cudaStream_t); \
+  template void explicit_rhs<R>(const GridParams&, const R*, R*, R*, R*, long long, const long long*, const int*, cudaStream_t); \
   template void batch_rhs<R>(const RhsMember<R>*, int, long long, bool, cudaStream_t);                        \
   template void stress_normals<R>(const GridParams&, long long, R*, cudaStream_t);                           \
   template void field_sums<R>(const R*, long long, double*, double*, int, cudaStream_t);                      \

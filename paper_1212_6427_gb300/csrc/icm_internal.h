@@ -200,12 +200,14 @@ template <> __host__ __device__ inline const RhsConst<double>& rhs_c<double>(con
 // r = (rho/dt) v + (eta/2) L v + div Sigma^n - (3/2 A^n - 1/2 A^{n-1}); adv <- A^n.
 // step_dev: device int64 time level (Philox counter word 1).  has_hist_dev: device
 // int, 0 = no history (A^{n-1} := A^n); set to 1 by the kernel launch sequence.
-// normals: scratch for the stress normals, 6 ncell values, where rhs_stored_normals says so.
+// normals: scratch of `room` values for the stress normals, where the right-hand side does not march: at least those of
+// three planes, 6 per cell (the spectrum scratch is that large on every grid).
 template <typename R>
-void explicit_rhs(const GridParams& g, const R* v, R* adv, R* rhs, R* normals, const long long* step_dev,
+void explicit_rhs(const GridParams& g, const R* v, R* adv, R* rhs, R* normals, long long room, const long long* step_dev,
                   const int* has_hist_dev, cudaStream_t st);
-// Whether the right-hand side of a grid draws its normals in a pass of its own.
-bool rhs_stored_normals(int precision, long long ncell);
+// Whether the right-hand side of a grid marches through it (with the plan's rhs_kz); otherwise it draws its normals in
+// a pass of its own.
+bool rhs_marches(int precision, int nx, int ny, int nz, bool noise);
 
 template <typename R>
 void stress_normals(const GridParams& g, long long step, R* out, cudaStream_t st);
@@ -482,7 +484,7 @@ struct RhsMember {
   const R* v;
   R* adv;
   R* rhs;
-  R* normals;             // the member's scratch for its stress normals (FP64)
+  R* normals;             // scratch for all of the member's stress normals, 6 ncell (FP64)
   const long long* step_dev;
   const int* hist_dev;
   long long w0;           // first global work unit of the member: tile-planes (FP32), blocks of
