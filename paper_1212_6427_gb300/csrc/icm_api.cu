@@ -137,8 +137,9 @@ struct icm_sim {
   bool plane = false;         // the grid's planes have passes of their own (plane_has_passes)
   int nrowblk = 0;
   int* bin_idx = nullptr;     // count [nrowblk], start [nrowblk + 1], cursor [nrowblk]
-  void* bin_blob = nullptr;   // list [kBinsPerBlob cap] ints, geometry [cap], accumulators [12 cap]
+  void* bin_blob = nullptr;   // records [cap], accumulators [12 cap], list [kBinsPerBlob cap] ints; or see kPlaneBytes
   int* bin_list = nullptr;
+  int* plane_first = nullptr;   // first z nodes of the plane passes' blobs
   void* geo = nullptr;
   double* acc = nullptr;
   // scalars
@@ -180,13 +181,14 @@ struct icm_sim {
 
 namespace {
 
-// Per blob slot: the bin list (kBinsPerBlob ints), the stencil record and 4 (n,3)
-// FP64 accumulators.
+// Per blob slot: the stencil record, then for the x passes 4 (n,3) FP64 accumulators and the bin list
+// (kBinsPerBlob ints), for the plane passes in the same place the partial sums and two first nodes.
 constexpr size_t kGeoBytes = kStencilBytes;
-constexpr int kAccPerBlob = 12;       // accumulators of the x passes
-constexpr int kPartsPerBlob = 3 * kPlaneParts;   // or the partial sums of the plane passes, in the same place
+constexpr int kAccPerBlob = 12;
 size_t bin_list_bytes(long long cap) { return ((size_t)kBinsPerBlob * 4 * cap + 255) / 256 * 256; }
-size_t bin_blob_bytes(long long cap) { return bin_list_bytes(cap) + (kGeoBytes + 8 * kPartsPerBlob) * cap; }
+size_t bin_blob_bytes(long long cap) { return (kGeoBytes + 8 * kAccPerBlob) * cap + bin_list_bytes(cap); }
+constexpr size_t kPlaneBytes = 3 * 8 * kPlaneParts + 2 * 4;   // of a blob in the plane passes, beside the record
+static_assert(kPlaneBytes <= 8 * kAccPerBlob + 4 * kBinsPerBlob, "the plane passes' share fits in the bins'");
 
 void* dalloc(icm_sim* s, size_t bytes) {
   void* p = nullptr;
@@ -544,6 +546,7 @@ enum BlobWork : int { BLOBS_IN_PLANES, BLOBS_IN_ROWS, BLOBS_APART };
 // Past the FP32 lines row blocks win over the separate kernels on large planes, with many blobs or many
 // planes: 96^3, 8000 blobs 252 / 228, 32000 blobs 436 / 451; 128^3 and 64 x 64 x 256 as above.
 BlobWork plane_blob_work(const icm_sim* s) {
+  if (s->geo == nullptr) return BLOBS_APART;   // no memory for the records (grow_blobs)
   int r1, r2;
   const bool rows = s->fused && s->ny % 32 == 0 && fft_split(s->ny, r1, r2);   // (row blocks inside a plane)
   const bool turns = s->nz > device_sms();   // 3 nz planes, at most three blocks per SM
@@ -640,7 +643,7 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
   ICM_STAGE("scalars", 0, scalars_before_step(s->scal, s->dt, s->rho, dvf, sb));
   // step 1: midpoint predictor (Eq. particle_pred)
   PlaneRecords rec{};
-  if (in_plane) rec = PlaneRecords{s->geo, s->bin_list, (int)s->cap};
+  if (in_plane) rec = PlaneRecords{s->geo, s->plane_first, (int)s->cap};
   ICM_STAGE("predict", 2 * gath + nb * (72 + (in_plane ? geob + 8.0 : 0.0)),
             blob_predict<R>(bp, bs, v, sb, rec));
   // pair forces at q^{n+1/2} (four kernels: cell count, scan, fill, forces)
@@ -660,7 +663,7 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
     pb.p = bp;
     pb.s = bs;
     pb.geo = s->geo;
-    pb.zfirst = s->bin_list;
+    pb.zfirst = s->plane_first;
     pb.zstride = (int)s->cap;
     const long long n3 = 3 * s->nb;
     pb.jvt = s->acc;
@@ -687,7 +690,7 @@ void enqueue_step(icm_sim* s, Prof* prof, int segment = -1) {
       passes("rt2", nullptr, PLANE_CDP, nullptr, 1.0, 0.0, nullptr, v, OUT_NONE, s->acc + 4 * n3, nullptr);
       // steps 6 and 7: (rho - dt/2 eta L) dv + dt grad dpi = S (dp - m_e J dv~); v = v~ + dv
       passes("rt3", nullptr, PLANE_SRC, nullptr, s->rho, 0.5 * s->dt * s->eta, s->scal + SC_SUMSRC, v, OUT_ADD,
-             s->acc + 8 * n3, s->acc + 12 * n3);
+             s->acc, s->acc + 4 * n3);   // (the forward pass has summed up the parts that were there)
     }
     // steps 8 and 9, the lagged slip term and the end-of-step scalars
     ICM_STAGE("finish", nb * (s->any_me ? 264 : 144),
@@ -869,8 +872,8 @@ icm_status grow_blobs(icm_sim* s, long long need) {
   }
   void* nbin = nullptr;
   if (s->fused || s->plane) {
-    nbin = dalloc(s, bin_blob_bytes(cap));
-    if (!nbin) {
+    nbin = dalloc(s, s->fused ? bin_blob_bytes(cap) : (kGeoBytes + kPlaneBytes) * cap);
+    if (!nbin && s->fused) {   // (grids that only have plane passes run the blob work apart without it)
       ICM_CK(cudaStreamSynchronize(s->stream));
       dfree(s, nbuf);
       return fail(ICM_ENOMEM, "device allocation of the bins of %lld blob slots failed", cap);
@@ -879,13 +882,12 @@ icm_status grow_blobs(icm_sim* s, long long need) {
   ICM_CK(cudaStreamSynchronize(s->stream));
   if (s->blob) dfree(s, s->blob);
   s->blob = nbuf;
-  if (s->fused || s->plane) {
-    if (s->bin_blob) dfree(s, s->bin_blob);
-    s->bin_blob = nbin;
-    s->bin_list = (int*)nbin;
-    s->geo = (unsigned char*)nbin + bin_list_bytes(cap);
-    s->acc = (double*)((unsigned char*)s->geo + kGeoBytes * cap);
-  }
+  if (s->bin_blob) dfree(s, s->bin_blob);
+  s->bin_blob = nbin;
+  s->geo = nbin;
+  s->acc = nbin ? (double*)((unsigned char*)nbin + kGeoBytes * cap) : nullptr;
+  s->bin_list = nbin && s->fused ? (int*)(s->acc + kAccPerBlob * cap) : nullptr;
+  s->plane_first = nbin ? (int*)(s->acc + 3 * kPlaneParts * cap) : nullptr;
   s->cap = cap;
   s->q = arrs[0]; s->qh = arrs[1]; s->u = arrs[2]; s->f = arrs[3]; s->g = arrs[4]; s->w0 = arrs[5];
   s->w1 = arrs[6]; s->jvt = arrs[7]; s->du = arrs[8]; s->dp = arrs[9]; s->cdp = arrs[10]; s->src = arrs[11];

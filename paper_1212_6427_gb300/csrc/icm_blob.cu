@@ -750,14 +750,14 @@ __global__ void k_finish_plane(BlobParams p, BlobState s, const double* __restri
   if (i < n3) {
     const int a = (int)(i % 3);
     const int K = p.kernel;
-    const double jvt = plane_sum(parts, n3, i, K);
+    const double jvt = inertial ? s.jvt[i] : plane_sum(parts, n3, i, K);
     double u = jvt, jv = jvt, g = 0.0;
     if (inertial) {
       double du = p.slip == 1 ? 0.0 : 0.5 * (p.eta / p.rho) * p.dt * s.g[i];
       if (p.slip == 2) du += s.w1[i] - s.w0[i];
-      u = jvt + plane_sum(parts + 4 * n3, n3, i, K) + du;
-      jv = jvt + plane_sum(parts + 8 * n3, n3, i, K);
-      g = plane_sum(parts + 12 * n3, n3, i, K + 2) * (p.inv_h * p.inv_h);
+      u = jvt + s.cdp[i] + du;
+      jv = jvt + plane_sum(parts, n3, i, K);
+      g = plane_sum(parts + 4 * n3, n3, i, K + 2) * (p.inv_h * p.inv_h);
     }
     const double qn = wrap_pos(fma(0.5 * p.dt, jv + s.w1[i], s.q[i]), p.box[a], p.inv_box[a]);
     s.q[i] = qn;

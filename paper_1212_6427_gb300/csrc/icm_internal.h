@@ -364,14 +364,17 @@ struct PlaneBlobs {
   int source;           // PlaneSource of a forward pass
   const double* vec;    // PLANE_VEC: the vectors
   const double* jvt;    // partial sums of J v~ (PLANE_CDP, PLANE_SRC)
-  const double* jdvt;   // and of J dv~ (PLANE_SRC, which also adds up the source's grid sum)
+  const double* jdvt;   // and of J dv~ (PLANE_SRC, which also adds up the source's grid sum and leaves the values of
+                        // J v~ and J dv~ in s.jvt and s.cdp)
   // An inverse pass gathers J x, and J L x (without 1/h^2), plane by plane: the part of blob b
   // and component a that plane c of its support holds goes to part[c (3 nb) + 3 b + a], one
   // writer each, and whoever needs the value adds the planes in order (plane_sum).
   double* part;         // kernel planes
   double* part_lap;     // kernel + 2 planes
 };
-constexpr int kPlaneParts = 4 + 4 + 4 + 6;   // J v~, J dv~, J dv, J L dv: doubles per blob component
+// Room for partial sums, doubles per blob component: J v~ and J dv~ of the first two solves (4 + 4 planes), which the
+// forward pass of the third adds up into the blob state, then J dv and J L dv (4 + 6).
+constexpr int kPlaneParts = 10;
 // The value of element i = 3 b + a from `planes` partial sums.
 __device__ __forceinline__ double plane_sum(const double* __restrict__ part, long long n3, long long i, int planes) {
   double x = part[i];
@@ -396,8 +399,9 @@ void plane_inverse(const FftCtx<R>& f, R* dst, R* dst2, int mode, const PlaneBlo
 template <typename R> struct SymParams;
 // z transform, symbol and inverse of a side without two-stage register kernels.
 template <typename R> void fft_z_any(const FftCtx<R>& f, const SymParams<R>& sp, cudaStream_t st);
-// Step 9 and the blob side of step 8 from the gathered J v~, J dv~, J dv, J L dv (partial sums of 4, 4,
-// 4 and 6 planes' room), with the end-of-step bookkeeping.
+// Step 9 and the blob side of step 8 from the gathered J v~ (partial sums of 4 planes' room) or, with excess
+// mass, J v~ and J dv~ in the blob state and the partial sums of J dv and J L dv (4 and 6 planes' room), with the
+// end-of-step bookkeeping.
 void blob_finish_plane(const BlobParams& p, BlobState s, const double* parts, bool inertial, long long* step_dev,
                        int* hist_dev, cudaStream_t st);
 

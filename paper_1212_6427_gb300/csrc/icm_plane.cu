@@ -378,24 +378,37 @@ __device__ __forceinline__ R gather_lap_lanes(const R* __restrict__ rows, const 
   return quad_sum(acc);
 }
 
-// Component i = 3 b + a of what step 5 or 6 spreads: dp = m_e (u - J v~ - du) of step 4, with
-// weight m~_f/(rho (m~_f + m_e)) in step 5, less m_e J dv~ in step 6.
+// Component i = 3 b + a of dp = m_e (u - J v~ - du), the momentum change of step 4.
+__device__ __forceinline__ double plane_dp(const PlaneBlobs& pb, int i, double jvt) {
+  const BlobParams& p = pb.p;
+  double du = p.slip == 1 ? 0.0 : 0.5 * (p.eta / p.rho) * p.dt * pb.s.g[i];
+  if (p.slip == 2) du += pb.s.w1[i] - pb.s.w0[i];
+  return pb.s.me[i / 3] * (pb.s.u[i] - jvt - du);
+}
+
+// Component i of what step 5 or 6 spreads: dp with weight m~_f/(rho (m~_f + m_e)), or less m_e J dv~.
 __device__ __forceinline__ double plane_source(const PlaneBlobs& pb, int i) {
   const BlobParams& p = pb.p;
   const double me = pb.s.me[i / 3];
   const long long n3 = 3 * pb.s.nb;
-  double du = p.slip == 1 ? 0.0 : 0.5 * (p.eta / p.rho) * p.dt * pb.s.g[i];
-  if (p.slip == 2) du += pb.s.w1[i] - pb.s.w0[i];
-  const double dp = me * (pb.s.u[i] - plane_sum(pb.jvt, n3, i, p.kernel) - du);
+  const double dp = plane_dp(pb, i, plane_sum(pb.jvt, n3, i, p.kernel));
   if (pb.source == PLANE_CDP) return p.mtf / (p.rho * (p.mtf + me)) * dp;
   return dp - me * plane_sum(pb.jdvt, n3, i, p.kernel);
 }
 
-// The grid sum of the source of step 6, for the momentum bookkeeping: NT elements per block.
+// The grid sum of the source of step 6, for the momentum bookkeeping, and the values of J v~ and J dv~, whose parts
+// make room for those of J dv in the inverse pass: NT elements per block.
 template <int NT>
 __device__ __forceinline__ void add_source_sum(const PlaneBlobs& pb, int block, int tid, double (*red)[NT]) {
   const int i = block * NT + tid, a = i % 3;
-  const double x = i < 3 * (int)pb.s.nb ? plane_source(pb, i) : 0.0;
+  double x = 0.0;
+  if (i < 3 * (int)pb.s.nb) {
+    const long long n3 = 3 * pb.s.nb;
+    const double jvt = plane_sum(pb.jvt, n3, i, pb.p.kernel), jdvt = plane_sum(pb.jdvt, n3, i, pb.p.kernel);
+    pb.s.jvt[i] = jvt;
+    pb.s.cdp[i] = jdvt;
+    x = plane_dp(pb, i, jvt) - pb.s.me[i / 3] * jdvt;
+  }
   for (int c = 0; c < 3; ++c) red[c][tid] = c == a ? x : 0.0;
   __syncthreads();
   for (int w = NT / 2; w > 0; w >>= 1) {
