@@ -1416,7 +1416,7 @@ icm_status icm_autotune(icm_sim* s, int32_t nsteps, icm_plan* chosen, double* ms
   std::vector<std::pair<int icm_plan::*, std::vector<int>>> knobs;
   if (s->fused || s->plane) knobs.push_back({&icm_plan::fused_blobs, {1, 0}});
   if (s->has_zmap) knobs.push_back({&icm_plan::tma_z, {1, 0}});
-  knobs.push_back({&icm_plan::rhs_kz, {0, 8, 16, 32}});
+  if (rhs_marches(s->prec, s->nx, s->ny, s->nz, s->kT > 0.0)) knobs.push_back({&icm_plan::rhs_kz, {0, 8, 16, 32}});
   knobs.push_back({&icm_plan::fork, {1, 0}});
   if (fft_has_xy_passes(s->prec, s->nx, s->ny)) knobs.push_back({&icm_plan::fused_xy, {0, 1}});
   if (s->has_zalt) knobs.push_back({&icm_plan::z_split, {0, 1}});
@@ -2527,9 +2527,15 @@ icm_status icm_batch_autotune(icm_batch* b, int32_t nsteps) {
   int best_grouped = 0;
   double best_ms = 0.0;
   icm_status st = trial(best, best_grouped, best_ms);
-  const std::vector<std::pair<int icm_plan::*, std::vector<int>>> knobs = {
-      {&icm_plan::fused_blobs, {1, 0}}, {&icm_plan::tma_z, {1, 0}}, {&icm_plan::rhs_kz, {0, 4, 8, 16, 32}},
-      {&icm_plan::fork, {1, 0}}, {&icm_plan::fused_xy, {0, 1}}, {&icm_plan::z_split, {0, 1}}};
+  // rhs_kz where some member's right-hand side marches: elsewhere the trials would only compare noise
+  bool marches = false;
+  for (const icm_sim* m : b->sims) marches = marches || rhs_marches(m->prec, m->nx, m->ny, m->nz, m->kT > 0.0);
+  std::vector<std::pair<int icm_plan::*, std::vector<int>>> knobs = {{&icm_plan::fused_blobs, {1, 0}},
+                                                                     {&icm_plan::tma_z, {1, 0}}};
+  if (marches) knobs.push_back({&icm_plan::rhs_kz, {0, 4, 8, 16, 32}});
+  knobs.push_back({&icm_plan::fork, {1, 0}});
+  knobs.push_back({&icm_plan::fused_xy, {0, 1}});
+  knobs.push_back({&icm_plan::z_split, {0, 1}});
   for (size_t k = 0; st == ICM_OK && k < knobs.size(); ++k)
     for (int val : knobs[k].second) {
       if (best.*(knobs[k].first) == val) continue;
@@ -2557,7 +2563,7 @@ icm_status icm_batch_autotune(icm_batch* b, int32_t nsteps) {
       // the RHS march again: in grouped steps every member's RHS precedes the first
       // group solve, so its latency counts where before it overlapped other members
       for (int kz : {0, 4, 8, 16, 32}) {
-        if (kz == best.rhs_kz || st != ICM_OK) continue;
+        if (!marches || kz == best.rhs_kz || st != ICM_OK) continue;
         icm_plan q = best;
         q.rhs_kz = kz;
         double mq = 0.0;
