@@ -358,6 +358,15 @@ icm_status icm_op_explicit_rhs(icm_sim* sim, const double* fluid_v, const double
  * plane 2m + 1 (words 2-3); unit normals by Box-Muller from u = (word + 1/2) 2^-32. */
 icm_status icm_op_stress_normals(icm_sim* sim, int64_t step, double* out);
 
+/* Pairs of unit normals from given words, by the function that draws the stress normals in the simulation's
+ * precision: out[2i], out[2i + 1] = sqrt(-2 ln u1) cos, sin (2 pi u2), u = (word + 1/2) 2^-32 of words[2i],
+ * words[2i + 1].  Errors: ICM_EINVAL, ICM_ENOMEM. */
+icm_status icm_op_normal_pairs(icm_sim* sim, int64_t n, const uint32_t* words, double* out);
+
+/* Reciprocals as the solves and the coupling sums take them, in FP32 or FP64: out[i] = 1/x[i], x normal
+ * and positive.  No simulation needed.  Errors: ICM_EINVAL, ICM_ENOMEM. */
+icm_status icm_op_reciprocals(int64_t n, int32_t precision, const double* x, double* out);
+
 /* Raw Philox4x32-10 words: for i < n, counter (ctr0 + i, ctr1, ctr2, ctr3) and
  * key (key0, key1); out[4*n].  No simulation needed. */
 icm_status icm_op_philox(int64_t n, uint32_t ctr0, uint32_t ctr1, uint32_t ctr2,

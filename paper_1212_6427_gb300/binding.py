@@ -103,6 +103,8 @@ SIGNATURES = {
     "icm_op_coupling": (_c_i32, [_vp, _c_i64, _dp, _dp, _c_d, _c_d, _dp]),
     "icm_op_explicit_rhs": (_c_i32, [_vp, _dp, _dp, _c_i64, _dp, _dp]),
     "icm_op_stress_normals": (_c_i32, [_vp, _c_i64, _dp]),
+    "icm_op_normal_pairs": (_c_i32, [_vp, _c_i64, ctypes.POINTER(_c_u32), _dp]),
+    "icm_op_reciprocals": (_c_i32, [_c_i64, _c_i32, _dp, _dp]),
     "icm_op_philox": (_c_i32, [_c_i64, _c_u32, _c_u32, _c_u32, _c_u32, _c_u32, _c_u32, ctypes.POINTER(_c_u32)]),
 }
 
@@ -428,6 +430,21 @@ def icm_op_stress_normals(sim, ncell, step):
     out, op = _out(6 * ncell)
     _check(lib().icm_op_stress_normals(sim, int(step), op))
     return out.reshape(6, ncell)
+
+
+def icm_op_normal_pairs(sim, words):
+    """(n, 2) normals from (n, 2) uint32 words."""
+    w = np.ascontiguousarray(words, dtype=np.uint32).reshape(-1, 2)
+    out, op = _out(w.size)
+    _check(lib().icm_op_normal_pairs(sim, len(w), w.ctypes.data_as(ctypes.POINTER(_c_u32)), op))
+    return out.reshape(-1, 2)
+
+
+def icm_op_reciprocals(precision, x):
+    x, xp = _f64(x)
+    out, op = _out(x.size)
+    _check(lib().icm_op_reciprocals(x.size, int(precision), xp, op))
+    return out
 
 
 def icm_op_philox(n, ctr, key):

@@ -1826,6 +1826,46 @@ icm_status icm_op_philox(int64_t n, uint32_t ctr0, uint32_t ctr1, uint32_t ctr2,
 }
 
 }  // extern "C"
+namespace {
+// Host values through a kernel of n threads on the legacy stream: m_in inputs and m_out results per thread.
+template <typename IN, typename RUN>
+icm_status map_on_device(int64_t n, int m_in, int m_out, const IN* in, double* out, RUN run) {
+  IN* x = nullptr;
+  double* y = nullptr;
+  cudaError_t e = cudaMalloc(&x, sizeof(IN) * m_in * n);
+  if (e == cudaSuccess) e = cudaMalloc(&y, sizeof(double) * m_out * n);
+  if (e == cudaSuccess) e = cudaMemcpy(x, in, sizeof(IN) * m_in * n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    run(x, y);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(out, y, sizeof(double) * m_out * n, cudaMemcpyDeviceToHost);
+  cudaFree(x);
+  cudaFree(y);
+  if (e == cudaSuccess) return ICM_OK;
+  cudaGetLastError();
+  return e == cudaErrorMemoryAllocation ? fail(ICM_ENOMEM, "device allocation failed")
+                                        : fail(ICM_ECUDA, "%s", cudaGetErrorString(e));
+}
+}  // namespace
+extern "C" {
+
+icm_status icm_op_normal_pairs(icm_sim* s, int64_t n, const uint32_t* words, double* out) {
+  if (!s || n < 0 || n > 0x7FFFFFFF || (n > 0 && (!words || !out))) return fail(ICM_EINVAL, "bad arguments");
+  if (n == 0) return ICM_OK;
+  return map_on_device(n, 2, 2, words, out,
+                       [&](const uint32_t* x, double* y) { normal_pairs(s->prec, (int)n, x, y, nullptr); });
+}
+
+icm_status icm_op_reciprocals(int64_t n, int32_t precision, const double* x, double* out) {
+  if (n < 0 || n > 0x7FFFFFFF || (precision != 32 && precision != 64) || (n > 0 && (!x || !out)))
+    return fail(ICM_EINVAL, "bad arguments");
+  if (n == 0) return ICM_OK;
+  return map_on_device(n, 1, 1, x, out,
+                       [&](const double* in, double* y) { symbol_reciprocals(precision, (int)n, in, y, nullptr); });
+}
+
+}  // extern "C"
 
 // ---------------------------------------------------------------------------
 // Batched replicas: the steps of every member simulation captured into one graph

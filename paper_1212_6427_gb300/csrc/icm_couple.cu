@@ -231,9 +231,23 @@ __global__ void __launch_bounds__(9 * 32) k_couple_final(const double* __restric
   if (lane == 0) out[9 * pair + e] = x * scale;
 }
 
+template <typename R>
+__global__ void k_reciprocals(int n, const double* __restrict__ x, double* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = (double)recip<R>((R)x[i]);
+}
+
 CoupleDims couple_dims(int nx, int ny, int nz) { return CoupleDims{{nx, ny, nz}, {nx / 2 + 1, ny, nz}}; }
 
 }  // namespace
+
+void symbol_reciprocals(int precision, int n, const double* x, double* out, cudaStream_t st) {
+  const unsigned blocks = (unsigned)((n + 127) / 128);
+  if (precision == 32)
+    k_reciprocals<float><<<blocks, 128, 0, st>>>(n, x, out);
+  else
+    k_reciprocals<double><<<blocks, 128, 0, st>>>(n, x, out);
+}
 
 size_t couple_scratch_doubles(int nx, int ny, int nz, int npair) {
   const CoupleDims d = couple_dims(nx, ny, nz);

@@ -705,6 +705,16 @@ __global__ void k_normals(GridParams g, uint32_t step, R* __restrict__ out) {
   for (int a = 0; a < 6; ++a) out[a * g.ncell + c] = z[a];
 }
 
+template <typename R>
+__global__ void k_normal_pairs(int n, const uint32_t* __restrict__ words, double* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  R p, q;
+  NormalPair<R>::apply(words[2 * i], words[2 * i + 1], p, q);
+  out[2 * i] = (double)p;
+  out[2 * i + 1] = (double)q;
+}
+
 __global__ void k_philox(long long n, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1,
                          uint32_t* __restrict__ out) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -911,6 +921,14 @@ template <typename R>
 void stress_normals(const GridParams& g, long long step, R* out, cudaStream_t st) {
   const int bs = 256;
   k_normals<R><<<(unsigned)((g.ncell + bs - 1) / bs), bs, 0, st>>>(g, (uint32_t)step, out);
+}
+
+void normal_pairs(int precision, int n, const uint32_t* words, double* out, cudaStream_t st) {
+  const unsigned blocks = (unsigned)((n + 127) / 128);
+  if (precision == 32)
+    k_normal_pairs<float><<<blocks, 128, 0, st>>>(n, words, out);
+  else
+    k_normal_pairs<double><<<blocks, 128, 0, st>>>(n, words, out);
 }
 
 void philox_words(long long n, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1,

@@ -405,6 +405,11 @@ template <typename R> void fft_z_any(const FftCtx<R>& f, const SymParams<R>& sp,
 void blob_finish_plane(const BlobParams& p, BlobState s, const double* parts, bool inertial, long long* step_dev,
                        int* hist_dev, cudaStream_t st);
 
+// The functions the noise and the symbol are made of, on given arguments (one thread each): n pairs of normals from
+// 2 n words (icm_grid.cu), n reciprocals (icm_couple.cu).
+void normal_pairs(int precision, int n, const uint32_t* words, double* out, cudaStream_t st);
+void symbol_reciprocals(int precision, int n, const double* x, double* out, cudaStream_t st);
+
 // Coupling matrices J(qi) (a - b L)^-1 P S(qj) (row-major 3 x 3 each) of npair pairs of
 // positions as sums over wave vectors (icm_couple.cu).  qi_dev, qj_dev: npair positions each,
 // wrapped into the box; scratch: couple_scratch_doubles of them, 16-byte aligned.
