@@ -265,7 +265,10 @@ __device__ __forceinline__ void for_each_blob_of_plane(const PlaneBlobs& pb, int
         int at = 0;
         if ((tid & 31) == 0 && m) at = atomicAdd(count, __popc(m));
         at = __shfl_sync(0xffffffffu, at, 0);
-        if (hit) list[at + __popc(m & ((1u << (tid & 31)) - 1u))] = (uint16_t)(base + j * NT + tid - start);
+        const int slot = at + __popc(m & ((1u << (tid & 31)) - 1u)), off = base + j * NT + tid - start;
+        if (hit && index_ok(slot, kPlaneList, pb.p.err) && index_ok(off, 65536, pb.p.err) &&
+            index_ok(first[j], nz, pb.p.err))
+          list[slot] = (uint16_t)off;
       }
       base += SCAN;
       __syncthreads();
@@ -286,7 +289,9 @@ __device__ __forceinline__ void for_each_blob_of_plane(const PlaneBlobs& pb, int
     }
     if (tid < threads)
       for (int t = tid >> 2; t < found; t += threads / 4) {
+        if (!index_ok(t, kPlaneList, pb.p.err)) continue;   // (the same for the four lanes)
         const int b = start + list[t];
+        if (!index_ok(b, nb, pb.p.err)) continue;
         f(b, plane_of(zf[b]) - (EXT ? 1 : 0), tid & 3);
       }
     start = base;
@@ -640,12 +645,13 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (NT == 256 ? 3 : 2) : 1)
       if (c >= 0 && c < pb.p.kernel) {   // the same for the four lanes
         const R j = three ? gather_lanes<R, 3>(rows, A, S.pofx, rec[b], comp, c, r, pb.p.err)
                           : gather_lanes<R, 4>(rows, A, S.pofx, rec[b], comp, c, r, pb.p.err);
-        if (r == 0) pb.part[c * n3 + i] = (double)j;
+        if (r == 0 && index_ok(pb.part + c * n3 + i - pb.jvt, kPlaneParts * n3, pb.p.err)) pb.part[c * n3 + i] = (double)j;
       }
       if (GATHER == 2) {
         const R jl = three ? gather_lap_lanes<R, 3>(rows, A, S.pofx, rec[b], comp, c, r, pb.p.err)
                            : gather_lap_lanes<R, 4>(rows, A, S.pofx, rec[b], comp, c, r, pb.p.err);
-        if (r == 0) pb.part_lap[(c + 1) * n3 + i] = (double)jl;
+        if (r == 0 && index_ok(pb.part_lap + (c + 1) * n3 + i - pb.jvt, kPlaneParts * n3, pb.p.err))
+          pb.part_lap[(c + 1) * n3 + i] = (double)jl;
       }
     });
   }
