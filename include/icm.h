@@ -146,13 +146,13 @@ typedef struct icm_plan {
                           other sides and in between, in separate kernels; 0: separate kernels     */
   int32_t tma_z;       /* 1: persistent z pass fed by TMA (z sides <= 256 with register kernels);
                           0: one block per z tile                                                  */
-  int32_t rhs_kz;      /* right-hand-side kernel of FP32 grids (but up to 2^20 cells at kT = 0, or with Nx
-                          up to 16, or 32): 4..64 z planes marched by each block, or 0 for persistent blocks (as
-                          many as the SMs hold) marching even shares of all tile-planes (default 0
-                          when each of two blocks per SM gets at least 8 tile-planes of 32 x 16
-                          cells, else the fewest planes that give every SM one or two blocks).
-                          Those grids and FP64 draw the stress normals in a pass of their own and
-                          do not march                                                             */
+  int32_t rhs_kz;      /* right-hand-side kernel of FP32 grids, except those of up to 2^20 cells at kT = 0
+                          or with Nx up to 16, or 32: 4..64 z planes marched by each block, or 0 for
+                          persistent blocks (as many as the SMs hold) marching even shares of all
+                          tile-planes (default 0 when each of two blocks per SM gets at least 8
+                          tile-planes of 32 x 16 cells, else the fewest planes that give every SM
+                          one or two blocks).  The excepted grids and FP64 draw the stress normals
+                          in a pass of their own and do not march                                  */
   int32_t fork;        /* 1: the blob-side prologue runs on a second stream beside the RHS          */
   int32_t fused_xy;    /* 1: forward x and y FFT passes fused on thread-block clusters (FP32,
                           Nx = Ny in 32, 64, 128, 256); 0 (default): whole z planes in one launch
